@@ -262,8 +262,8 @@ size_t refine_ws(Carver &c, int64_t N, int32_t D, int64_t S, int32_t k, int32_t 
 size_t cross_ws(Carver &c, int64_t Nq, int64_t Nc, int32_t D, int32_t k, const atsne_knn_opts &o,
                 bool radius, TcPlan *plan, TcWs *tws) {
     if (exact_on_tensor_cores(o, k) && Nq > 0 && !(radius && o.precision == ATSNE_FP8_RERANK)) {
-        TcPlan pl = tc_plan(Nc, D, Nq, k, o.precision, o.rerank_k);
-        if (radius) pl.cap = RADIUS_CAP;  // only the points inside the radius are buffered
+        const TcPlan pl = radius ? tc_plan_radius(Nc, D, Nq, k, o.precision, o.rerank_k)
+                                 : tc_plan(Nc, D, Nq, k, o.precision, o.rerank_k);
         if (plan) *plan = pl;
         tc_workspace(c, Nc, D, Nq, true, pl, tws);
     }
@@ -271,7 +271,7 @@ size_t cross_ws(Carver &c, int64_t Nq, int64_t Nc, int32_t D, int32_t k, const a
 }
 
 // Autotuner: room for the largest candidate's tensor-core workspace.
-constexpr int TUNE_MAX_CAND = 8;
+constexpr int TUNE_MAX_CAND = 9;
 size_t tune_ws(int64_t N, int32_t D, int32_t k, int64_t S, const atsne_knn_opts &o, int *cand, int *n_cand) {
     const int64_t Q = S > 0 ? S : N;
     int c_[TUNE_MAX_CAND];
@@ -510,7 +510,7 @@ atsne_status atsne_tune_knn(const float *X, int64_t N, int32_t D, const int32_t 
         }
         if (st == ATSNE_OK && e == cudaSuccess && ms < best_ms) {
             best_ms = ms;
-            best = pl.splits;
+            best = tc_splits(pl);
         }
     }
     if (e0) cudaEventDestroy(e0);

@@ -27,6 +27,11 @@ struct TcPlan {
     int passes = 1, Dp = 0, row_tiles = 0, splits = 1, cols_per_split = 0, ksel = 0, cap = 0;
     int halves = 1;  // candidate buffers per (row, split): one per column half of a tile
     bool certify = true;  // rows certified exact (else the ksel best keys re-ranked, approximate)
+    // fixed thresholds (knn_filter.cu); the fields above then describe the
+    // adaptive launch over the rows it gives up
+    bool filter = false;
+    int S = 0, blk = 0, rank = 0;                // sampled rows, columns per block, the threshold's rank
+    int fsplits = 1, fcols = 0, fcap = 0;
 };
 // Row and column order of a large self kNN (points grouped by nearest
 // centroid; each row tile streams its own groups' column tiles first).
@@ -45,7 +50,9 @@ struct TcWs {
     float *nrm = nullptr, *stats = nullptr;
     unsigned *gmax = nullptr;
     char *cand = nullptr, *meta = nullptr;
+    size_t metas = 0;
     unsigned *row_hist = nullptr;
+    int64_t hist_rows = 0;
     float *scale = nullptr, *qscale = nullptr;  // FP8 row scales
     float *qnrm = nullptr, *qstats = nullptr;   // queries from another array: norms, error stats
     int32_t *flag_rows = nullptr, *flag_count = nullptr;
@@ -53,13 +60,21 @@ struct TcWs {
     bool ordered = false;                       // rows and columns in the order of OrderWs
     unsigned long long *clock = nullptr;        // one split: tiles issued by all CTAs
     OrderWs ord;
+    // fixed thresholds: the rows' thresholds, the sampled rows' copies and norm
+    // pieces, the block values, and the rows given up with their copies
+    float *tau = nullptr, *minima = nullptr;
+    uint16_t *shi = nullptr, *sext = nullptr, *rhi = nullptr, *rlo = nullptr;
+    int32_t *retry_rows = nullptr;
 };
 // Limit of the tensor kernel's pipeline waits (process-wide; default 1 s).
 uint64_t pipeline_wait_ns();
 void set_pipeline_wait_ns(uint64_t ns);
-// splits > 0 forces the column split count; else the one atsne_tune_knn
-// recorded for this shape, else the rule.
+// splits > 0 forces the column split count; 0: the one atsne_tune_knn recorded
+// for this shape, else the rule; < 0: the rule.
 TcPlan tc_plan(int64_t N, int D, int64_t Q, int k, int precision, int rerank_k, int splits = 0);
+TcPlan tc_plan_radius(int64_t N, int D, int64_t Q, int k, int precision, int rerank_k);
+int tc_splits(const TcPlan &pl);  // the plan's column splits (the tunable)
+int filter_splits(int64_t row_pairs, int64_t col_tiles, int max_splits);
 int tuned_splits(int64_t N, int D, int64_t Q, int k, int precision, int rerank_k);
 void set_tuned_splits(int64_t N, int D, int64_t Q, int k, int precision, int rerank_k, int splits);
 void clear_tuned_splits();
@@ -79,7 +94,8 @@ atsne_status radius_filter_launch(int32_t *idx, float *d2, int64_t rows, int k, 
 atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist, int64_t Q, int k,
                           const TcPlan &pl, const TcWs &w, int32_t *idx_out, float *d2_out,
                           cudaStream_t stream, const float *Xq = nullptr,
-                          const float *radius = nullptr, const float *hint = nullptr);
+                          const float *radius = nullptr, const float *hint = nullptr,
+                          const int64_t *qcount = nullptr);
 
 // ---- calibrate ------------------------------------------------------------
 size_t calibrate_smem_bytes(int k);

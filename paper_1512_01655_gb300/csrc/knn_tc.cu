@@ -9,33 +9,37 @@
 //   knn_prep   x -> hi (+ lo) BF16 copies padded to Dp = 64*ceil(D/64), the
 //              FP32 norm ||x||^2, and the norms of what the BF16 copies miss
 //              (used to bound the key error).
-//   knn_tc     persistent, warp-specialised: warp 0 issues TMA loads of
-//              128-query x 64 and 256-point x 64 BF16 tiles (128-byte swizzle)
-//              into a shared-memory ring; warp 1 issues tcgen05.mma
-//              (M=128, N=256, K=16) into one of two TMEM accumulators; warps
-//              2-5 read the other accumulator back (tcgen05.ld, one query row
-//              per thread), form the keys, and append every key below the
-//              row's running threshold tau to a per-(row, column split)
-//              candidate buffer. Each thread also counts its buffered
-//              distances in 64 buckets (8 per octave below an upper bound of
-//              any distance of the row); tau is lowered to the upper edge of
-//              the bucket in which the count reaches ksel, a valid bound on
-//              the ksel-th distance within 9%. Buffers are sized for about
-//              2.5x the survivors of a streaming top-ksel, so the exact
-//              compaction of a full buffer (warp radix select) is rare.
-//              When few query rows leave the SMs idle, the columns are cut
-//              into splits (units ordered split-major); the splits of a row
-//              then also count into one histogram per row in global memory,
-//              so each split filters with the bound of the whole row.
-//   knn_merge  one warp per query: one pass stages the keys below the
-//              splits' lowest tau (+2E) in shared memory; there the k-th
-//              smallest key is selected, every candidate within 2E of it (E
-//              bounds the key error, see row_error_bound) is re-ranked by
-//              FP32 direct differences, and a certificate is checked: if the
-//              k-th exact distance is below ||x_i||^2 + min(tau) - E, no
-//              point outside the buffers can belong to the k nearest, and
-//              the row is exact. Rows that fail are listed for the
-//              brute-force kernel.
+//   knn_filter (knn_filter.cu) the contraction with a fixed threshold per row,
+//              taken from a sample of the corpus; the keys below it are
+//              buffered. The path of every corpus of at least
+//              FILTER_MIN_ROWS rows in the BF16 and FP32 modes.
+//   knn_merge  one warp per query: the k-th smallest buffered key is selected,
+//              every candidate within 2E of it (E bounds the key error, see
+//              row_error_bound) is re-ranked by FP32 direct differences, and a
+//              certificate is checked: if the k-th exact distance is below
+//              ||x_i||^2 + min(tau) - E, no point outside the buffers can
+//              belong to the k nearest, and the row is exact.
+//   knn_tc     the same contraction with a threshold that adapts as the columns
+//              stream by: for the rows that the fixed threshold (a statistical
+//              guess) left with too few keys, too many, or no certificate, for
+//              the FP8 mode and for small corpora. Persistent,
+//              warp-specialised: warp 0 issues TMA loads of 128-query x 64 and
+//              256-point x 64 BF16 tiles (128-byte swizzle) into a
+//              shared-memory ring; warp 1 issues tcgen05.mma (M=128, N=256,
+//              K=16) into one of two TMEM accumulators; the epilogue warps read
+//              the other accumulator back (tcgen05.ld, one query row per
+//              thread), form the keys, and append every key below the row's
+//              running threshold tau to a per-(row, column split) candidate
+//              buffer. Each thread also counts its buffered distances in 64
+//              buckets; tau is lowered to the upper edge of the bucket in which
+//              the count reaches ksel. Buffers are sized for about 2.5x the
+//              survivors of a streaming top-ksel, so the exact compaction of a
+//              full buffer (warp radix select) is rare. When few query rows
+//              leave the SMs idle, the columns are cut into splits (units
+//              ordered split-major); the splits of a row then also count into
+//              one histogram per row in global memory, so each split filters
+//              with the bound of the whole row.
+//   Rows that still lack a certificate go to the brute-force kernel.
 //
 // Every wait on an mbarrier is bounded (1 s); on expiry the CTA raises the
 // device status word, stops issuing work, drains its own copies and MMAs and
@@ -53,6 +57,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "knn_keys.cuh"
 #include "tc_ptx.cuh"
 #include "warp_sort.cuh"
 
@@ -73,11 +78,8 @@ constexpr int NBUCKET = 64;      // a thread's distance buckets: 2 octaves of d^
 constexpr int HSHIFT = 18;       // float bits >> HSHIFT: exponent and 5 mantissa bits (32 per octave)
 constexpr int GH_BUCKETS = 48;   // a row's global histogram (column splits): 6 octaves, 8 per octave
 constexpr int GH_SHIFT = 20;
-
-struct Cand {
-    float key;
-    int32_t idx;
-};
+constexpr int64_t FILTER_MIN_ROWS = 1024;       // a smaller corpus is not sampled
+constexpr int64_t RETRY_SPLIT_ROWS = 32768;  // rows given up by the fixed threshold that may be split
 
 // PASSES: 1 = one BF16 pass, 3 = BF16 hi/lo in three passes, 8 = one FP8
 // (E4M3, per-row scale) pass. A k-block is one 128-byte swizzle row: 64 BF16
@@ -149,7 +151,6 @@ struct TcParams {
     const float *scale;    // FP8: [N] corpus row scales (x ~ scale * q)
     const float *qscale;   // FP8 with a query list: [Q] query row scales
     const float *qnrm;     // queries from another array: [Q] their ||x||^2 (no self exclusion)
-    const float *radius;   // radius mode: [Q] squared radius per query row (else nullptr)
     const float *hint;     // [Q] upper bounds of each query row's k-th squared distance (or nullptr)
     const float4 *qst;     // queries from another array: their error statistics
     const float4 *st;      // corpus rows' error statistics (for listed queries)
@@ -159,6 +160,10 @@ struct TcParams {
     const unsigned *lo_max;  // max norm of the corpus' BF16 low halves (float bits), or nullptr
                              // when the queries' low halves are not covered by it
     const int32_t *qlist;  // query row -> corpus index (nullptr: identity)
+    // the rows given up by the fixed-threshold kernel: row r of this launch is
+    // query row rlist[r], *rcount rows in all, their splits from retry_plan
+    const int32_t *rlist, *rcount;
+    int64_t bufs;          // room for that many (row, split) buffers
     int64_t Q, N;
     int KB;                // Dp / 64
     int splits, cols_per_split, row_tiles;
@@ -170,6 +175,26 @@ struct TcParams {
     uint64_t wait_ns;      // limit of each pipeline wait (the drains of issued copies and MMAs keep WAIT_NS)
 };
 
+// Rows, row tiles and column splits of a launch whose row count is only known
+// on the device. Few rows are cut into as many splits as give every SM two
+// units; more than RETRY_SPLIT_ROWS have no row histograms and take one.
+struct UnitPlan {
+    int64_t Q;
+    int row_tiles, splits, cols_per_split;
+};
+__device__ __forceinline__ UnitPlan retry_plan(int64_t count, int64_t N, int64_t bufs) {
+    UnitPlan u;
+    u.Q = count;
+    u.row_tiles = (int)((count + TC_BM - 1) / TC_BM);
+    const int64_t tiles = (N + TC_BN - 1) / TC_BN;
+    int64_t s = 1;
+    if (count > 0 && count <= RETRY_SPLIT_ROWS)
+        s = max((int64_t)1, min(min((tiles + 3) / 4, bufs / count), (int64_t)((304 + u.row_tiles - 1) / u.row_tiles)));
+    u.cols_per_split = (int)((tiles + s - 1) / s * TC_BN);
+    u.splits = (int)((N + u.cols_per_split - 1) / u.cols_per_split);
+    return u;
+}
+
 // Absolute bucket of a squared distance on the thread grid (32 per octave),
 // and the upper edge of bucket b.
 __device__ __forceinline__ int dbucket(float d) { return (int)(__float_as_uint(fmaxf(d, 1e-30f)) >> HSHIFT); }
@@ -180,10 +205,6 @@ __device__ __forceinline__ uint32_t sign_into_mask(float v, uint32_t mask) {
     uint32_t r;
     asm("shf.l.wrap.b32 %0, %1, %2, 1;" : "=r"(r) : "r"(__float_as_uint(v)), "r"(mask));
     return r;
-}
-
-__device__ __forceinline__ float key_of_bits(uint32_t u) {
-    return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
 }
 
 __device__ __forceinline__ unsigned lanemask_lt() {
@@ -289,10 +310,10 @@ knn_prep_kernel(const float *__restrict__ X, const int32_t *__restrict__ rows, i
                 __nv_bfloat16 *__restrict__ bext, __nv_bfloat16 *__restrict__ aext, int *status) {
     const int lane = threadIdx.x & 31;
     const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    // the constant query slice of the folded norms: -1/2 in its first three columns
-    if (aext && blockIdx.x == 0)
-        for (int t = threadIdx.x; t < TC_BM * 16; t += blockDim.x)
-            aext[t] = __float2bfloat16_rn((t & 15) < 3 ? -0.5f : 0.f);
+    if (aext && blockIdx.x == 0) fold_query_slice(aext);
+    // the norm slices of the rows that fill the last column tile: +inf, a key no row keeps
+    if (bext && r >= nrows && r < (nrows + TC_BN - 1) / TC_BN * TC_BN && lane < 16)
+        bext[r * 16 + lane] = __float2bfloat16_rn(lane == 0 ? INFINITY : 0.f);
     if (r >= nrows) return;
     int64_t src = rows ? rows[r] : r;
     if (src < 0 || src >= N) src = 0;  // flagged by the caller's index check
@@ -320,15 +341,7 @@ knn_prep_kernel(const float *__restrict__ X, const int32_t *__restrict__ rows, i
     n = warp_sum(n);
     res = warp_sum(res);
     l2 = warp_sum(l2);
-    if (bext && lane < 16) {
-        // the row's FP32 squared norm as three BF16 pieces h1 + h2 + h3 (each
-        // the rounded remainder of the previous: together within 2^-24 of it)
-        const __nv_bfloat16 h1 = __float2bfloat16_rn(n);
-        const float r1 = n - __bfloat162float(h1);
-        const __nv_bfloat16 h2 = __float2bfloat16_rn(r1);
-        const __nv_bfloat16 h3 = __float2bfloat16_rn(r1 - __bfloat162float(h2));
-        bext[r * 16 + lane] = lane == 0 ? h1 : lane == 1 ? h2 : lane == 2 ? h3 : __float2bfloat16_rn(0.f);
-    }
+    if (bext && lane < 16) bext[r * 16 + lane] = norm_piece(n, lane);
     if (!__all_sync(0xffffffffu, finite) && lane == 0) raise_status(status, DEV_NONFINITE);
     if (lane == 0 && nrm) {
         nrm[r] = n;
@@ -383,36 +396,6 @@ knn_prep_fp8_kernel(const float *__restrict__ X, const int32_t *__restrict__ row
 // ---------------------------------------------------------------------------
 // the fused contraction + filter kernel
 // ---------------------------------------------------------------------------
-// Bound on |estimated - true| key (= squared distance - ||x_i||^2) for query
-// row statistics st = (||x||, residual norm of its BF16 copy, norm of its low
-// part) against any corpus point (gmax: the corpus maxima of the same): the
-// terms the BF16 copies drop (Cauchy-Schwarz on the residual norms), the FP32
-// accumulation of the products, and the FP32 norms.
-__device__ __forceinline__ float key_error_bound(float4 st, const unsigned *gmax, float acc_coef,
-                                                 float sq_coef) {
-    const float amax = __uint_as_float(gmax[0]);
-    const float rmax = __uint_as_float(gmax[1]);
-    const float lmax = __uint_as_float(gmax[2]);
-    const float a = st.x, r = st.y, l = st.z;
-    const float drop = l * lmax + r * amax + a * rmax;
-    return 2.f * drop + acc_coef * a * amax + (4e-6f + sq_coef) * amax * amax + 4e-6f * a * a;
-}
-
-// The same bound over the corpus points of norm at most amax_cap only (a
-// point farther in norm than sqrt(d) from the query is farther than sqrt(d)
-// in distance). Their residuals are capped by the BF16 rounding bound:
-// ||x - hi|| <= 2^-9 ||x|| and ||lo|| <= 2^-8 ||x|| (round to nearest, 8
-// significand bits), plus a tiny absolute term for subnormal values.
-__device__ __forceinline__ float key_error_bound_capped(float4 st, const unsigned *gmax, float acc_coef,
-                                                        float sq_coef, float amax_cap) {
-    const float amax = fminf(__uint_as_float(gmax[0]), amax_cap);
-    const float rmax = fminf(__uint_as_float(gmax[1]), 0x1p-9f * amax + 1e-30f);
-    const float lmax = fminf(__uint_as_float(gmax[2]), 0x1p-8f * amax + 1e-30f);
-    const float a = st.x, r = st.y, l = st.z;
-    const float drop = l * lmax + r * amax + a * rmax;
-    return 2.f * drop + acc_coef * a * amax + (4e-6f + sq_coef) * amax * amax + 4e-6f * a * a;
-}
-
 // Fire-and-forget request of the 128-byte line holding p into L2.
 __device__ __forceinline__ void prefetch_l2(const void *p) {
     asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<uint64_t>(p)));
@@ -495,7 +478,9 @@ __global__ void __launch_bounds__(TcCfg<PASSES>::THREADS, 1) knn_tc_kernel(const
     __syncthreads();
     fence_after_sync();
     const uint32_t tbase = s.tmem_base;
-    const int n_units = p.row_tiles * p.splits;
+    UnitPlan up{p.Q, p.row_tiles, p.splits, p.cols_per_split};
+    if (p.rcount) up = retry_plan(*p.rcount, p.N, p.bufs);
+    const int n_units = up.row_tiles * up.splits;
 
     if (warp == 0) {
         if (lane == 0) {
@@ -512,9 +497,9 @@ __global__ void __launch_bounds__(TcCfg<PASSES>::THREADS, 1) knn_tc_kernel(const
             }
             int un = 0;  // units begun by this CTA
             for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x, ++un) {
-                const int rt = u % p.row_tiles, sp = u / p.row_tiles;
-                const int64_t c0 = (int64_t)sp * p.cols_per_split;
-                const int64_t c1 = min(p.N, c0 + p.cols_per_split);
+                const int rt = u % up.row_tiles, sp = u / up.row_tiles;
+                const int64_t c0 = (int64_t)sp * up.cols_per_split;
+                const int64_t c1 = min(p.N, c0 + up.cols_per_split);
                 const int64_t ntl = (c1 - c0 + TC_BN - 1) / TC_BN;
                 int64_t s0 = 0;
                 const int64_t ps = p.pro ? p.pro[2 * rt] : 0, pn = p.pro ? p.pro[2 * rt + 1] : 0;
@@ -571,9 +556,9 @@ __global__ void __launch_bounds__(TcCfg<PASSES>::THREADS, 1) knn_tc_kernel(const
             bool ok = true;
             if (C::FOLD && !mbar_wait(&s.ext_bar, 0, &s.abort_flag, p.wait_ns)) ok = false;
             for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
-                const int sp = u / p.row_tiles;
-                const int64_t c0 = (int64_t)sp * p.cols_per_split;
-                const int64_t c1 = min(p.N, c0 + p.cols_per_split);
+                const int sp = u / up.row_tiles;
+                const int64_t c0 = (int64_t)sp * up.cols_per_split;
+                const int64_t c1 = min(p.N, c0 + up.cols_per_split);
                 const int64_t ntl = (c1 - c0 + TC_BN - 1) / TC_BN;
                 for (int64_t ti = 0; ti < ntl && ok; ++ti) {
                     if (!mbar_wait(&s.acc_empty[acc], acc_phase ^ 1u, &s.abort_flag, p.wait_ns)) {
@@ -648,15 +633,15 @@ __global__ void __launch_bounds__(TcCfg<PASSES>::THREADS, 1) knn_tc_kernel(const
         constexpr int NCH = CW / 32;           // 32-column TMEM loads per tile
         const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
         uint32_t *hist = s.sel_hist[e];
-        const int subs = p.splits * C::HALVES;  // candidate buffers per query row
+        const int subs = up.splits * C::HALVES;  // candidate buffers per query row
         int acc = 0;
         uint32_t acc_phase = 0;
         bool ok = true;
         int un = 0;  // units begun by this CTA
         for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x, ++un) {
-            const int rt = u % p.row_tiles, sp = u / p.row_tiles;
-            const int64_t c0 = (int64_t)sp * p.cols_per_split;
-            const int64_t c1 = min(p.N, c0 + p.cols_per_split);
+            const int rt = u % up.row_tiles, sp = u / up.row_tiles;
+            const int64_t c0 = (int64_t)sp * up.cols_per_split;
+            const int64_t c1 = min(p.N, c0 + up.cols_per_split);
             const int64_t ntl_u = (c1 - c0 + TC_BN - 1) / TC_BN;
             int64_t s0 = 0;  // where the producer started this unit's stream
             const int64_t ps = p.pro ? p.pro[2 * rt] : 0, pn = p.pro ? p.pro[2 * rt + 1] : 0;
@@ -674,21 +659,18 @@ __global__ void __launch_bounds__(TcCfg<PASSES>::THREADS, 1) knn_tc_kernel(const
             }
             const int64_t row = (int64_t)rt * TC_BM + quarter * 32 + lane;
             const bool cross = p.qnrm != nullptr;  // queries from another array than the corpus
-            const int qraw = row < p.Q ? (cross ? (int)row : (p.qlist ? p.qlist[row] : (int)row)) : -1;
+            const int64_t r0 = row < up.Q ? (p.rlist ? p.rlist[row] : row) : 0;  // the query row
+            const int qraw = row < up.Q ? (cross ? (int)r0 : (p.qlist ? p.qlist[r0] : (int)r0)) : -1;
             const bool qv = qraw >= 0 && (cross || qraw < p.N);  // listed rows out of range are flagged by the caller
             const int qid = qv ? qraw : -1;
             Cand *buf = qv ? p.cand + ((size_t)row * subs + (size_t)sp * C::HALVES + half) * p.cap : nullptr;
             float tau = qv ? INFINITY : -INFINITY;
             float th = INFINITY;  // bound of this half's kh-th smallest key
             const int kh = C::HALVES > 1 ? (p.ksel + 1) / 2 : p.ksel;
-            int cnt = 0, since = 0, rovf = 0;
-            // radius mode: a fixed threshold, the row's squared radius as a key
-            // widened by twice the key error bound, so that no point inside the
-            // radius is filtered out; no top-k bookkeeping
-            const bool rmode = p.radius != nullptr;
+            int cnt = 0, since = 0;
             // the thread's distance grid: NBUCKET buckets, 32 per octave of d^2,
             // below an anchor; first anchored at t0 = (||x|| + max||y||)^2 >= d
-            const float nx = qv ? (cross ? p.qnrm[row] : p.nrm[qid]) : 0.f;
+            const float nx = qv ? (cross ? p.qnrm[r0] : p.nrm[qid]) : 0.f;
             const float ai = sqrtf(nx), amax = __uint_as_float(p.gmax[0]);
             const float t0 = (ai + amax) * (ai + amax) * 1.0001f + 1e-30f;
             int top = dbucket(t0);
@@ -697,7 +679,7 @@ __global__ void __launch_bounds__(TcCfg<PASSES>::THREADS, 1) knn_tc_kernel(const
             // grid below t0 (8 buckets per octave): the splits cover disjoint
             // columns and the counts only grow, so the bucket where the summed
             // count reaches ksel bounds the row's ksel-th distance for all of them.
-            unsigned *gh = (p.splits > 1 && qv) ? p.row_hist + (size_t)row * GH_BUCKETS : nullptr;
+            unsigned *gh = (up.splits > 1 && qv) ? p.row_hist + (size_t)row * GH_BUCKETS : nullptr;
             const int gbase = (int)(__float_as_uint(t0) >> GH_SHIFT) - (GH_BUCKETS - 1);
             auto global_tau = [&]() {
                 int cum = 0, b = 0;
@@ -718,15 +700,15 @@ __global__ void __launch_bounds__(TcCfg<PASSES>::THREADS, 1) knn_tc_kernel(const
                     tau = fminf(tau, __uint_as_float((uint32_t)(gbase + b + 1) << GH_SHIFT) - nx);
             };
             if (gh) global_tau();
-            if ((rmode || (p.hint && PASSES != 8)) && qv) {  // FP8 keys carry no error bound
-                // the radius (or the hint, an upper bound of the k-th squared
-                // distance) as a key threshold, widened by twice the key error
-                // bound so that no point inside is filtered out
-                const float rad = rmode ? p.radius[row] : p.hint[row];
+            if (p.hint && PASSES != 8 && qv) {  // FP8 keys carry no error bound
+                // the hint, an upper bound of the k-th squared distance, as a
+                // key threshold, widened by twice the key error bound so that
+                // no point inside is filtered out
+                const float rad = p.hint[r0];
                 if (isfinite(rad)) {
                     // the points that must pass lie within sqrt(rad) of the
                     // query, so their norms are at most ||x|| + sqrt(rad)
-                    const float4 qs = cross ? p.qst[row] : p.st[qid];
+                    const float4 qs = cross ? p.qst[r0] : p.st[qid];
                     const float widen =
                         2.f * key_error_bound_capped(qs, p.gmax, p.acc_coef, p.sq_coef,
                                                      qs.x + sqrtf(fmaxf(rad, 0.f)) * (1.f + 1e-6f) + 1e-30f) +
@@ -737,7 +719,7 @@ __global__ void __launch_bounds__(TcCfg<PASSES>::THREADS, 1) knn_tc_kernel(const
                     if (ht < top) top = ht;
                 }
             }
-            bool rebased = rmode || (p.hint && PASSES != 8);
+            bool rebased = p.hint && PASSES != 8;
             // largest and smallest buffered keys, for the first re-anchoring of the grid
             float kmx = -INFINITY, kmn = INFINITY;
             uint32_t *dh = &s.dhist[e][0][lane];
@@ -764,7 +746,7 @@ __global__ void __launch_bounds__(TcCfg<PASSES>::THREADS, 1) knn_tc_kernel(const
             }
             // FP8: x_i . x_j ~ s_i s_j (q_i . q_j); the row's scale, the
             // columns' -2 s_j beside their norms
-            const float si = PASSES == 8 && qv ? (p.qscale ? p.qscale[row] : p.scale[qid]) : 1.f;
+            const float si = PASSES == 8 && qv ? (p.qscale ? p.qscale[r0] : p.scale[qid]) : 1.f;
             // the partner half may still be on an earlier unit: its bound is
             // taken only when its tag is this unit
             volatile unsigned long long *tau_mine =
@@ -923,15 +905,6 @@ __global__ void __launch_bounds__(TcCfg<PASSES>::THREADS, 1) knn_tc_kernel(const
                             for (int i = 0; i < 2; ++i) t2[i] = (j0 & 8) ? t4[2 * i + 1] : t4[2 * i];
                             const float key = C::FOLD ? -2.f * ((j0 & 16) ? t2[1] : t2[0]) : ((j0 & 16) ? t2[1] : t2[0]);
                             const int col = colb + j0;
-                            if (rmode) {  // no compaction: a full buffer sends the row to the fallback
-                                if (has) {
-                                    if (cnt < p.cap)
-                                        buf[cnt++] = Cand{key, col};
-                                    else
-                                        rovf = 1;
-                                }
-                                continue;
-                            }
                             if (has) buf[cnt] = Cand{key, col};
                             cnt += has;
                             const float dd2 = nx + key;
@@ -956,7 +929,6 @@ __global__ void __launch_bounds__(TcCfg<PASSES>::THREADS, 1) knn_tc_kernel(const
                     acc = 0;
                     acc_phase ^= 1u;
                 }
-                if (rmode) continue;  // the threshold is fixed
                 // Once kh keys are buffered, the largest of them bounds the
                 // kh-th (and, with ksel buffered, the ksel-th) smallest, and
                 // the grid is re-anchored and recounted: the first anchor
@@ -1071,7 +1043,7 @@ __global__ void __launch_bounds__(TcCfg<PASSES>::THREADS, 1) knn_tc_kernel(const
             if (!ok) break;
             if (qv)
                 p.meta[(size_t)row * subs + (size_t)sp * C::HALVES + half] =
-                    make_int4(cnt, __float_as_int(tau), rovf, 0);
+                    make_int4(cnt, __float_as_int(tau), 0, p.rcount ? META_RETRY : META_FIRST);
         }
     }
     fence_before_sync();
@@ -1092,6 +1064,12 @@ struct MergeParams {
     // ordered rows and columns (knn_order.cu): position -> row; the kernel's
     // rows, norms and candidate columns are positions, the outputs rows
     const int32_t *perm;
+    // the rows given up by the fixed-threshold kernel (as in TcParams), or nullptr
+    const int32_t *rlist, *rcount;
+    int64_t bufs;
+    const int64_t *qcount;  // if given, the rows in use (device; at most Q)
+    int tag;                // of the launch that wrote the buffers
+    bool flag_out;          // flag output rows (for the brute-force kernel), else query rows
     const float *X;
     int D, k, ksel;
     int rc, mst;            // re-rank set and staged keys per row (shared memory)
@@ -1123,6 +1101,7 @@ __device__ __forceinline__ float row_error_bound(const MergeParams &p, float4 st
 // certificate the staged keys are read once, by the collection of the re-rank
 // set, so the re-rank set takes their place (p.rc <= p.mst) and five blocks
 // fit on an SM instead of four.
+constexpr int merge_reg_keys(bool cert) { return 32 * (cert ? 24 : 36); }
 size_t merge_smem_bytes(bool cert, int rc, int mst) {
     return (size_t)MERGE_WARPS * (256 * 4 + (size_t)mst * 8 + (cert ? (size_t)rc * 8 : 0) + TIE_MAX * 12);
 }
@@ -1134,20 +1113,30 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
     uint32_t *hist = reinterpret_cast<uint32_t *>(mg_smem) + w * 256;
     const int MST = p.mst, RC = p.rc;
     const int RCS = CERT ? RC : 0;  // the re-rank set's own region (else it is the staging region)
-    float *sk = reinterpret_cast<float *>(mg_smem + MERGE_WARPS * 1024) + w * MST;
-    int *sj = reinterpret_cast<int *>(mg_smem + MERGE_WARPS * (1024 + MST * 4)) + w * MST;
+    // MST keys, then MST indices of this warp
+    float *sk0 = reinterpret_cast<float *>(mg_smem + MERGE_WARPS * 1024) + w * 2 * MST;
+    float *sk = sk0;
+    int *sjg = reinterpret_cast<int *>(sk0) + MST;
     float *rdw = CERT ? reinterpret_cast<float *>(mg_smem + MERGE_WARPS * (1024 + MST * 8)) + w * RC : sk;
-    int *rjw = CERT ? reinterpret_cast<int *>(mg_smem + MERGE_WARPS * (1024 + MST * 8 + RC * 4)) + w * RC : sj;
+    int *rjg = CERT ? reinterpret_cast<int *>(mg_smem + MERGE_WARPS * (1024 + MST * 8 + RC * 4)) + w * RC : sjg;
     double *dmw = reinterpret_cast<double *>(mg_smem + MERGE_WARPS * (1024 + MST * 8 + RCS * 8)) + w * TIE_MAX;
     int *mpw = reinterpret_cast<int *>(mg_smem + MERGE_WARPS * (1024 + MST * 8 + RCS * 8 + TIE_MAX * 8)) +
                w * TIE_MAX;
     const int sel = CERT ? p.k : p.ksel;  // rank of the key that bounds the re-rank set
-    const int64_t row = (int64_t)blockIdx.x * MERGE_WARPS + w;
-    if (row >= p.Q) return;
     const bool cross = p.Xq != nullptr;
-    const int qid = cross ? (int)row : (p.qlist ? p.qlist[row] : (int)row);
-    const int64_t orow = p.perm ? p.perm[row] : row;  // the output row (and the query's row of X)
-    const int S = p.splits;
+    int64_t Q = p.qcount ? min(*p.qcount, p.Q) : p.Q;
+    int S = p.splits;
+    if (p.rcount) {
+        const UnitPlan up = retry_plan(*p.rcount, p.N, p.bufs);
+        Q = up.Q;
+        S = up.splits * p.splits;  // splits of a row by buffers of a split
+    }
+    for (int64_t row = (int64_t)blockIdx.x * MERGE_WARPS + w; row < Q; row += (int64_t)gridDim.x * MERGE_WARPS) {
+    __syncwarp();
+    const int64_t r0 = p.rlist ? p.rlist[row] : row;  // the query row
+    const int qid = cross ? (int)r0 : (p.qlist ? p.qlist[r0] : (int)r0);
+    const int self = cross ? -1 : qid;                // the fixed threshold buffers the query itself too
+    const int64_t orow = p.perm ? p.perm[r0] : r0;    // the output row (and the query's row of X)
     const Cand *cb = p.cand + (size_t)row * S * p.cap;
     const int4 *mt = p.meta + (size_t)row * S;
 
@@ -1156,6 +1145,10 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
     float tau_min = INFINITY;
     for (int u = lane; u < S; u += 32) {
         const int4 m = mt[u];
+        if (m.w != p.tag) {  // a unit that a stopped launch never finished
+            ovf = 1;
+            continue;
+        }
         total += min(max(m.x, 0), p.cap);
         ovf |= m.z;
         tau_min = fminf(tau_min, __int_as_float(m.y));
@@ -1168,6 +1161,11 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
     }
     bool good = !ovf && total >= sel && qid >= 0 && (cross || qid < p.N);
     int nr = 0;
+    const bool regs = total <= merge_reg_keys(CERT) && S <= 256;
+    // the staged indices: beside the staged keys, or, with the keys in
+    // registers, in their place (without a certificate behind the re-rank set)
+    int *sj = regs ? reinterpret_cast<int *>(sk0) + (CERT ? 0 : RC) : sjg;
+    int *rjw = CERT ? rjg : sj;
     if (good) {
         // One pass over the buffers stages every (key, index) at or below
         // tau_min. When at least sel keys lie below tau_min, the sel-th
@@ -1176,63 +1174,142 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
         // are collected from the buffers.
         // the row's buffers requested into L2 at once (the staging pass below
         // walks them one 512-byte step at a time)
-        for (int u = 0; u < S; ++u) {
+        for (int u = S >= 32 ? lane : 0; u < S; u += S >= 32 ? 32 : 1) {
             const int c = min(max(mt[u].x, 0), p.cap);
             const char *bb = reinterpret_cast<const char *>(cb + (size_t)u * p.cap);
-            for (int o = lane * 128; o < c * (int)sizeof(Cand); o += 32 * 128) prefetch_l2(bb + o);
+            for (int o = S >= 32 ? 0 : lane * 128; o < c * (int)sizeof(Cand); o += S >= 32 ? 128 : 32 * 128)
+                prefetch_l2(bb + o);
         }
-        const float E = CERT ? row_error_bound(p, cross ? p.qstats[row] : p.stats[qid]) : 0.f;
+        const float E = CERT ? row_error_bound(p, cross ? p.qstats[r0] : p.stats[qid]) : 0.f;
         const float slim = tau_min;  // the select needs no key above tau_min
-        int ns = 0, nlt = 0;
-        for (int u0 = 0; u0 < S; u0 += 32) {
-          const int cu = u0 + lane < S ? min(max(mt[u0 + lane].x, 0), p.cap) : 0;  // the counts of 32 splits at once
-          for (int j = 0; j < 32 && u0 + j < S; ++j) {
-            const int c = __shfl_sync(0xffffffffu, cu, j);
-            const Cand *b = cb + (size_t)(u0 + j) * p.cap;
-            // two candidates per lane in one 16-byte load; two such loads
-            // in flight per step (positions past c are not staged)
-            auto load2 = [&](int i, Cand &e0, Cand &e1) {
-                e0 = Cand{INFINITY, -1};
-                e1 = Cand{INFINITY, -1};
-                if (i + 1 < c) {
-                    const float4 v = __ldcs(reinterpret_cast<const float4 *>(b + i));
-                    e0 = Cand{v.x, __float_as_int(v.y)};
-                    e1 = Cand{v.z, __float_as_int(v.w)};
-                } else if (i < c) {
-                    e0 = b[i];
+        // A row whose buffered keys fit the registers (the fixed threshold
+        // lets through two or three times ksel) keeps them there, six loads in
+        // flight per lane, with their indices in shared memory: the sel-th
+        // smallest is found by bisection on the keys' bits, counting with the
+        // warp's reduction (it stops at any threshold with exactly sel keys
+        // below it), without the radix select's shared-memory atomics.
+        constexpr int NK = merge_reg_keys(CERT) / 32;
+        uint32_t u[NK];
+        int n_others = 0;
+        float theta = 0.f;
+        if (regs) {
+            // the buffers' entries as one sequence: exclusive starts in `hist`
+            int run = 0;
+            for (int u0 = 0; u0 < S; u0 += 32) {
+                const int c = u0 + lane < S ? min(max(mt[u0 + lane].x, 0), p.cap) : 0;
+                int incl = c;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += t;
                 }
-            };
-            auto stage2 = [&](int i, Cand e0, Cand e1) {
-                nlt += (e0.key < tau_min) + (e1.key < tau_min);
-                const bool t0 = i < c && e0.key <= slim, t1 = i + 1 < c && e1.key <= slim;
-                const unsigned m0 = __ballot_sync(0xffffffffu, t0);
-                const unsigned m1 = __ballot_sync(0xffffffffu, t1);
-                const unsigned lt = lanemask_lt();
-                const int pos = ns + __popc(m0 & lt) + __popc(m1 & lt);
-                if (t0 && pos < MST) {
-                    sk[pos] = e0.key;
-                    sj[pos] = e0.idx;
-                }
-                if (t1 && pos + t0 < MST) {
-                    sk[pos + t0] = e1.key;
-                    sj[pos + t0] = e1.idx;
-                }
-                ns += __popc(m0) + __popc(m1);
-            };
-            for (int base = 0; base < c; base += 128) {
-                const int i = base + 2 * lane;
-                Cand e0, e1, e2, e3;
-                load2(i, e0, e1);
-                load2(i + 64, e2, e3);
-                stage2(i, e0, e1);
-                stage2(i + 64, e2, e3);
+                if (u0 + lane < S) hist[u0 + lane] = (uint32_t)(run + incl - c);
+                run += __shfl_sync(0xffffffffu, incl, 31);
             }
-          }
+            __syncwarp();
+            int top = 1;  // search step: the largest power of two below S
+            while (2 * top < S) top <<= 1;
+            uint32_t lo = 0xffffffffu, hi = 0u;
+            constexpr int B = 6;  // loads in flight per lane
+#pragma unroll
+            for (int i0 = 0; i0 < NK; i0 += B) {
+                Cand e[B];
+#pragma unroll
+                for (int i = 0; i < B; ++i) e[i] = Cand{INFINITY, -1};
+                if (i0 * 32 < total) {
+#pragma unroll
+                    for (int i = 0; i < B; ++i) {
+                        const int t = (i0 + i) * 32 + lane;
+                        int b = 0;
+                        for (int o = top; o > 0; o >>= 1)
+                            if (b + o < S && (int)hist[b + o] <= t) b += o;
+                        if (t < total) e[i] = cb[(size_t)b * p.cap + (t - (int)hist[b])];
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < B; ++i) {
+                    const int t = (i0 + i) * 32 + lane;
+                    const bool on = t < total && e[i].idx != self;
+                    u[i0 + i] = on ? float_key(e[i].key) : 0xffffffffu;
+                    if (t < total) sj[t] = e[i].idx;
+                    if (on) {
+                        ++n_others;
+                        lo = min(lo, u[i0 + i]);
+                        hi = max(hi, u[i0 + i]);
+                    }
+                }
+            }
+            n_others = (int)__reduce_add_sync(0xffffffffu, (unsigned)n_others);
+            lo = __reduce_min_sync(0xffffffffu, lo);
+            hi = __reduce_max_sync(0xffffffffu, hi);
+            if (n_others < sel) good = false;
+            while (good && lo < hi) {
+                const uint32_t mid = lo + ((hi - lo) >> 1);
+                int c = 0;
+#pragma unroll
+                for (int i = 0; i < NK; ++i) c += u[i] <= mid;
+                c = (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
+                if (c >= sel) {
+                    hi = mid;
+                    if (c == sel) break;
+                } else {
+                    lo = mid + 1u;
+                }
+            }
+            theta = key_of_bits(hi);
+            __syncwarp();
+        }
+        bool staged = false;
+        int ns = 0;
+        if (!regs) {
+        int nlt = 0, others = 0;  // others: buffered keys but the query's own
+        // 32 buffers at a time, their entries taken as one sequence: a row's
+        // buffers may be many and short (column splits), and a lane finds its
+        // entry's buffer by a binary search over the lanes' counts; four loads
+        // in flight per lane
+        for (int u0 = 0; u0 < S; u0 += 32) {
+            const int cu = u0 + lane < S ? min(max(mt[u0 + lane].x, 0), p.cap) : 0;
+            int incl = cu;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += t;
+            }
+            const int n_all = __shfl_sync(0xffffffffu, incl, 31);
+            for (int base = 0; base < n_all; base += 128) {
+                Cand e[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int t = base + 32 * q + lane;
+                    int b = 0;  // the first buffer whose inclusive count exceeds t
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1)
+                        if (__shfl_sync(0xffffffffu, incl, b + o - 1) <= t) b += o;
+                    const int first = __shfl_sync(0xffffffffu, incl - cu, b);
+                    e[q] = Cand{INFINITY, -1};
+                    if (t < n_all) e[q] = cb[(size_t)(u0 + b) * p.cap + (t - first)];
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const bool on = base + 32 * q + lane < n_all && e[q].idx != self;
+                    others += on;
+                    nlt += on && e[q].key < tau_min;
+                    const bool take = on && e[q].key <= slim;
+                    const unsigned tm = __ballot_sync(0xffffffffu, take);
+                    const int pos = ns + __popc(tm & lanemask_lt());
+                    if (take && pos < MST) {
+                        sk[pos] = e[q].key;
+                        sj[pos] = e[q].idx;
+                    }
+                    ns += __popc(tm);
+                }
+            }
         }
         nlt = (int)__reduce_add_sync(0xffffffffu, (unsigned)nlt);
         __syncwarp();
         int n_less = 0;
-        const bool staged = nlt >= sel && ns <= MST;
+        if ((int)__reduce_add_sync(0xffffffffu, (unsigned)others) < sel) good = false;
+        staged = nlt >= sel && ns <= MST;
         uint32_t prefix;
         if (staged) {
             prefix = warp_select([&](int i) { return sk[i]; }, ns, sel, hist, lane, n_less);
@@ -1244,13 +1321,15 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
                         const Cand *b = cb + (size_t)u * p.cap;
                         for (int base = 0; base < c; base += 32) {
                             const int i = base + lane;
-                            fn(i < c, i < c ? b[i].key : 0.f);
+                            const bool on = i < c && b[i].idx != self;
+                            fn(on, on ? b[i].key : 0.f);
                         }
                     }
                 },
                 sel, hist, lane, n_less);
         }
-        const float theta = key_of_bits(prefix);
+        theta = key_of_bits(prefix);
+        }
         // the re-rank set, collected in two bands of keys: (-inf, theta] then
         // (theta, lim]
         auto take_batch = [&](bool take, int idx) {
@@ -1260,7 +1339,18 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
             nr += __popc(tm);
         };
         auto collect = [&](float lo, float hi) {  // keys in (lo, hi]
-            if (staged && hi <= slim) {  // all staged: every key up to slim was
+            if (regs) {
+                const uint32_t ul = isinf(lo) ? 0u : float_key(lo), uh = float_key(hi);
+#pragma unroll
+                for (int i = 0; i < NK; ++i) {
+                    if (i * 32 >= total) continue;
+                    const int t = i * 32 + lane;
+                    const bool in = u[i] != 0xffffffffu && u[i] > ul && u[i] <= uh;
+                    const int idx = in ? sj[t] : -1;
+                    if (!CERT) __syncwarp();  // compacted in place, as below
+                    take_batch(in, idx);
+                }
+            } else if (staged && hi <= slim) {  // all staged: every key up to slim was
                 for (int base = 0; base < ns; base += 32) {
                     const int i = base + lane;
                     const bool in = i < ns && sk[i] > lo && sk[i] <= hi;
@@ -1278,7 +1368,7 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
                         const int i = base + lane;
                         Cand e{INFINITY, -1};
                         if (i < c) e = b[i];
-                        take_batch(i < c && e.key > lo && e.key <= hi, e.idx);
+                        take_batch(i < c && e.idx != self && e.key > lo && e.key <= hi, e.idx);
                     }
                 }
             }
@@ -1303,18 +1393,12 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
             }
             __syncwarp();
         };
-        const float *xq = cross ? p.Xq + (int64_t)row * p.D : p.X + (p.perm ? orow : (int64_t)qid) * p.D;
+        const float *xq = cross ? p.Xq + r0 * p.D : p.X + (p.perm ? orow : (int64_t)qid) * p.D;
         const bool vec4 = (p.D & 3) == 0 && (reinterpret_cast<uintptr_t>(p.X) & 15) == 0 &&
                           (reinterpret_cast<uintptr_t>(xq) & 15) == 0;
         // exact FP32 distances of rjw[from, to) in the library's one summation
         // order (group8_d2_pair), eight candidates per warp step
         auto rerank = [&](int from, int to) {
-            // every candidate row requested into L2 first (rows of at most
-            // 1 KB: longer ones gain less than the requests cost)
-            for (int t = from + lane; p.D <= 256 && t < to; t += 32) {
-                const char *xr = reinterpret_cast<const char *>(p.X + (int64_t)rjw[t] * p.D);
-                for (int o = 0; o < p.D * 4; o += 128) prefetch_l2(xr + o);
-            }
             const int g = lane >> 3, gl = lane & 7;
             for (int t0 = from; t0 < to; t0 += 8) {
                 const int ta = t0 + g, tb = t0 + 4 + g;
@@ -1344,7 +1428,7 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
             for (int t = lane; t < nr1; t += 32) dk0 = fmaxf(dk0, rdw[t]);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) dk0 = fmaxf(dk0, __shfl_xor_sync(0xffffffffu, dk0, o));
-            const float4 st = cross ? p.qstats[row] : p.stats[qid];
+            const float4 st = cross ? p.qstats[r0] : p.stats[qid];
             Ec = fminf(E, key_error_bound_capped(st, p.gmax, p.acc_coef, p.sq_coef,
                                                   st.x + sqrtf(dk0) * (1.f + 1e-6f) + 1e-30f));
             collect(theta, theta + 2.f * Ec);
@@ -1382,7 +1466,7 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
             fp64_near_ties(rdw, rjw, nr, p.k, xq, p.X, p.D, dmw, mpw, lane);
             if (CERT) {
                 const float dk = rdw[p.k - 1];
-                const float nx = cross ? p.qnrm[row] : p.nrm[qid];
+                const float nx = cross ? p.qnrm[r0] : p.nrm[qid];
                 const float lb = nx + tau_min - Ec;
                 // certified: no point outside the buffers can be closer than dk
                 good = isinf(tau_min) || dk < lb * (1.f - 1e-6f);
@@ -1397,7 +1481,8 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
             p.d2_out[orow * p.k + t] = rdw[t];
         }
     } else if (lane == 0) {
-        p.flag_rows[atomicAdd(p.flag_count, 1)] = (int)orow;
+        p.flag_rows[atomicAdd(p.flag_count, 1)] = (int)(p.flag_out ? orow : r0);
+    }
     }
 }
 
@@ -1422,7 +1507,7 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32) radius_merge_kernel(MergePar
     for (int u = lane; u < S; u += 32) {
         const int4 m = mt[u];
         total += min(max(m.x, 0), p.cap);
-        ovf |= m.z;
+        ovf |= m.z | (m.w != p.tag);  // a unit that a stopped launch never finished
     }
     total = (int)__reduce_add_sync(0xffffffffu, (unsigned)total);
     ovf = (int)__reduce_or_sync(0xffffffffu, (unsigned)ovf);
@@ -1498,7 +1583,9 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
     return fn;
 }
 
-atsne_status make_bf16_map(CUtensorMap *m, const void *base, int64_t rows, int Dp, int box_rows) {
+}  // namespace
+
+atsne_status tc_map_bf16(CUtensorMap *m, const void *base, int64_t rows, int Dp, int box_rows) {
     auto enc = tensor_map_encoder();
     if (!enc) return set_error(ATSNE_ECUDA, "cuTensorMapEncodeTiled unavailable");
     cuuint64_t dims[2] = {(cuuint64_t)Dp, (cuuint64_t)rows};
@@ -1514,7 +1601,7 @@ atsne_status make_bf16_map(CUtensorMap *m, const void *base, int64_t rows, int D
 
 // Rows of 16 BF16 (32 bytes: the norm slices of the folded one-pass mode),
 // box_rows rows per copy in the 32-byte swizzle layout.
-atsne_status make_ext_map(CUtensorMap *m, const void *base, int64_t rows, int box_rows) {
+atsne_status tc_map_ext(CUtensorMap *m, const void *base, int64_t rows, int box_rows) {
     auto enc = tensor_map_encoder();
     if (!enc) return set_error(ATSNE_ECUDA, "cuTensorMapEncodeTiled unavailable");
     cuuint64_t dims[2] = {16u, (cuuint64_t)rows};
@@ -1527,6 +1614,8 @@ atsne_status make_ext_map(CUtensorMap *m, const void *base, int64_t rows, int bo
     if (r != CUDA_SUCCESS) return set_error(ATSNE_ECUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
     return ATSNE_OK;
 }
+
+namespace {
 
 // The FP32 accumulation term of the key error bound: (K steps of 16 + 8) * 2^-21,
 // the folded norms adding one step in the one-pass BF16 mode.
@@ -1610,15 +1699,65 @@ int tc_split_candidates(int64_t N, int D, int64_t Q, int k, int precision, int r
     const int64_t row_tiles = (Q + TC_BM - 1) / TC_BM;
     const int64_t units[] = {0, 152, 304, 608, 1216, 2048, 4096, 8192};
     int n = 0;
+    out[n++] = tc_splits(tc_plan(N, D, Q, k, precision, rerank_k, -1));  // the rule's
     for (int64_t u : units) {
         if (n == max_out) break;
         const int want = u == 0 ? 1 : (int)((u + row_tiles - 1) / row_tiles);
-        const int s = tc_plan(N, D, Q, k, precision, rerank_k, want).splits;
+        const int s = tc_splits(tc_plan(N, D, Q, k, precision, rerank_k, want));
         bool dup = false;
         for (int i = 0; i < n; ++i) dup |= out[i] == s;
         if (!dup) out[n++] = s;
     }
     return n;
+}
+
+int tc_splits(const TcPlan &pl) { return pl.filter ? pl.fsplits : pl.splits; }
+
+// The fixed-threshold plan (knn_filter.cu): the sample its thresholds come from
+// and the buffers for what lies below them.
+static void plan_filter(TcPlan &pl, int64_t N, int64_t Q, int splits) {
+    const int64_t pairs = (Q + 2 * TC_BM - 1) / (2 * TC_BM);
+    const int64_t col_tiles = (N + TC_BN - 1) / TC_BN;
+    const int cw = TC_BN / F_PARTS;
+    if (N < FILTER_MIN_ROWS) return;
+    // S rows, about 32 sqrt(N): the sample's pass and what the thresholds let
+    // through then cost about the same
+    int S = 512;
+    while (S < 65536 && (double)S * S < 0.5 * 1024.0 * (double)N) S <<= 1;
+    while (S > N / 2) S >>= 1;
+    // of n keys below a threshold about x = n S / N are sampled; taking the
+    // r-th smallest sampled key as the threshold leaves fewer than ksel corpus
+    // keys below it when r or more of x = ksel S / N expected fall there:
+    // r - 3 sqrt(r) = x, about one row in a thousand
+    const double x = (double)pl.ksel * S / (double)N;
+    const double rt = 1.5 + sqrt(2.25 + x);
+    const double r = rt * rt;
+    const double expect = r * (double)N / S;
+    if (expect > 0.4 * (double)N) return;
+    // only the best key of each block of sampled columns is kept: a share q of
+    // the blocks holds one of the r. The largest block that leaves q below 0.6
+    const double f = r / S;
+    int blk = cw;
+    auto share = [&](int b) { return 1.0 - pow(1.0 - f, b); };
+    if (share(cw) > 0.6) blk = 32;
+    if (blk == 32 && share(32) > 0.6) blk = 8;
+    while (S / blk > 1024) blk = blk == 8 ? 32 : cw;
+    if (share(blk) > 0.9) return;
+    pl.filter = true;
+    pl.S = S;
+    pl.blk = blk;
+    pl.rank = (int)fmax(1.0, floor(share(blk) * (S / blk) + 0.5));
+    if (splits <= 0) splits = filter_splits(pairs, col_tiles, 64);
+    if (splits > 64) splits = 64;
+    if (splits > col_tiles) splits = (int)col_tiles;
+    const int64_t per = (col_tiles + splits - 1) / splits;
+    pl.fcols = (int)(per * TC_BN);
+    pl.fsplits = (int)((N + pl.fcols - 1) / pl.fcols);
+    // a row's neighbours may all lie in one split (a corpus sorted by class),
+    // but spread over the parts of its tiles
+    int64_t cap = (int64_t)ceil(2.0 * expect / F_PARTS) + 48;
+    if (cap > per * cw) cap = per * cw;
+    pl.fcap = (int)((cap + 15) / 16 * 16);
 }
 
 TcPlan tc_plan(int64_t N, int D, int64_t Q, int k, int precision, int rerank_k, int splits) {
@@ -1627,13 +1766,19 @@ TcPlan tc_plan(int64_t N, int D, int64_t Q, int k, int precision, int rerank_k, 
     pl.certify = precision != ATSNE_FP8_RERANK && precision != ATSNE_BF16_RERANK_APPROX;
     const int ke = pl.passes == 8 ? 128 : TC_BK;  // elements per 128-byte row
     pl.Dp = ((D + ke - 1) / ke) * ke;
+    int ks = rerank_k > 0 ? rerank_k : (pl.passes == 3 ? k + 38 : !pl.certify ? 4 * k : 2 * k);
+    if (!pl.certify && ks > RCAP_FP8 / 2) ks = RCAP_FP8 / 2;
+    if (ks < k) ks = k;
+    pl.ksel = ks;
+    if (splits == 0) splits = tuned_splits(N, D, Q, k, precision, rerank_k);
+    if (pl.passes != 8) plan_filter(pl, N, Q, splits);
+    if (pl.filter) splits = 0;  // the adaptive kernel then only takes the rows given up
+    // The adaptive kernel: (row tile, column split) units, one split per row
+    // tile when the row tiles alone give every SM at least two units (a split
+    // restarts the streaming top-k, whose k' ln(n / k') survivors dominate the
+    // epilogue), else about 2048 units, each at least 4 column tiles long
     pl.row_tiles = (int)((Q + TC_BM - 1) / TC_BM);
     const int64_t col_tiles = (N + TC_BN - 1) / TC_BN;
-    // (row tile, column split) units: one split per row tile when the row tiles
-    // alone give every SM at least two units (a split restarts the streaming
-    // top-k, whose k' ln(n / k') survivors dominate the epilogue), else about
-    // 2048 units, each at least 4 column tiles long
-    if (splits <= 0) splits = tuned_splits(N, D, Q, k, precision, rerank_k);
     int64_t S = splits > 0 ? splits : pl.row_tiles >= 304 ? 1 : (2048 + pl.row_tiles - 1) / pl.row_tiles;
     const int64_t max_s = (col_tiles + 3) / 4;
     if (S > max_s) S = max_s;
@@ -1641,10 +1786,6 @@ TcPlan tc_plan(int64_t N, int D, int64_t Q, int k, int precision, int rerank_k, 
     const int64_t tiles_per = (col_tiles + S - 1) / S;
     pl.cols_per_split = (int)(tiles_per * TC_BN);
     pl.splits = (int)((N + pl.cols_per_split - 1) / pl.cols_per_split);
-    int ks = rerank_k > 0 ? rerank_k : (pl.passes == 3 ? k + 38 : !pl.certify ? 4 * k : 2 * k);
-    if (!pl.certify && ks > RCAP_FP8 / 2) ks = RCAP_FP8 / 2;
-    if (ks < k) ks = k;
-    pl.ksel = ks;
     // A streaming top-ksel over n columns in random order admits about
     // ksel (1 + ln(n / ksel)) keys; the bucketed threshold somewhat more.
     // The buffer holds 2.5x the model so that the exact compaction of a full
@@ -1663,6 +1804,20 @@ TcPlan tc_plan(int64_t N, int D, int64_t Q, int k, int precision, int rerank_k, 
     return pl;
 }
 
+// Queries from another array with radii: the radii are the thresholds, nothing
+// is sampled, and what does not fit the buffers goes to the brute-force kernel.
+TcPlan tc_plan_radius(int64_t N, int D, int64_t Q, int k, int precision, int rerank_k) {
+    TcPlan pl = tc_plan(N, D, Q, k, precision, rerank_k);
+    const int64_t col_tiles = (N + TC_BN - 1) / TC_BN;
+    const int s = filter_splits((Q + 2 * TC_BM - 1) / (2 * TC_BM), col_tiles, 64);
+    pl.filter = true;
+    pl.S = 0;
+    pl.fcols = (int)((col_tiles + s - 1) / s * TC_BN);
+    pl.fsplits = (int)((N + pl.fcols - 1) / pl.fcols);
+    pl.fcap = RADIUS_CAP;
+    return pl;
+}
+
 size_t tc_workspace(Carver &c, int64_t N, int D, int64_t Q, bool list, const TcPlan &pl, TcWs *ws) {
     TcWs w;
     const size_t per = pl.passes == 8 ? (size_t)pl.Dp / 2 : (size_t)pl.Dp;  // 16-bit words per row
@@ -1677,35 +1832,89 @@ size_t tc_workspace(Carver &c, int64_t N, int D, int64_t Q, bool list, const TcP
     w.nrm = c.take<float>((size_t)N);
     w.stats = c.take<float>((size_t)N * 4);
     w.gmax = c.take<unsigned>(4);
-    w.cand = c.take<char>((size_t)Q * pl.splits * pl.halves * pl.cap * sizeof(Cand));
-    w.meta = c.take<char>((size_t)Q * pl.splits * pl.halves * sizeof(int4));
-    w.row_hist = pl.splits > 1 ? c.take<unsigned>((size_t)Q * GH_BUCKETS) : nullptr;
+    // the adaptive kernel's launch (all rows, or those given up) and the
+    // fixed-threshold one before it use the same buffers in turn
+    const bool adaptive = !pl.filter || pl.S > 0;
+    const size_t abufs = adaptive ? (size_t)Q * pl.splits * pl.halves : 0;
+    const size_t fbufs = pl.filter ? (size_t)Q * pl.fsplits * F_PARTS : 0;
+    const size_t cands = abufs * pl.cap > fbufs * pl.fcap ? abufs * pl.cap : fbufs * pl.fcap;
+    w.cand = c.take<char>(cands * sizeof(Cand));
+    w.metas = abufs > fbufs ? abufs : fbufs;
+    w.meta = c.take<char>(w.metas * sizeof(int4));
+    w.hist_rows = pl.filter ? (pl.S > 0 ? hmin(Q, RETRY_SPLIT_ROWS) : 0) : pl.splits > 1 ? Q : 0;
+    w.row_hist = w.hist_rows > 0 ? c.take<unsigned>((size_t)w.hist_rows * GH_BUCKETS) : nullptr;
     w.flag_rows = c.take<int32_t>((size_t)Q);
-    w.flag_count = c.take<int32_t>(1);
-    w.bext = pl.passes == 1 ? c.take<uint16_t>((size_t)N * 16) : nullptr;
-    w.aext = pl.passes == 1 ? c.take<uint16_t>((size_t)TC_BM * 16) : nullptr;
+    w.flag_count = c.take<int32_t>(2);
+    w.bext = pl.passes == 1 ? c.take<uint16_t>((size_t)((N + TC_BN - 1) / TC_BN * TC_BN) * 16) : nullptr;
+    w.aext = pl.passes == 1 || pl.S > 0 ? c.take<uint16_t>((size_t)TC_BM * 16) : nullptr;
+    if (pl.filter) w.tau = c.take<float>((size_t)Q);
+    if (pl.S > 0) {
+        w.shi = c.take<uint16_t>((size_t)pl.S * per);
+        w.sext = c.take<uint16_t>((size_t)pl.S * 16);
+        w.minima = c.take<float>((size_t)Q * (pl.S / pl.blk));
+        w.retry_rows = c.take<int32_t>((size_t)Q);
+        w.rhi = c.take<uint16_t>((size_t)Q * per);
+        w.rlo = pl.passes == 3 ? c.take<uint16_t>((size_t)Q * per) : nullptr;
+    }
     w.ordered = knn_ordered(N, D, list, pl);
     // the global column clock where many units stream a corpus larger than L2
     // on short rows (longer rows keep the natural start; the contraction, not
     // the copies, sets their pace)
-    w.clock = pl.splits == 1 && N >= ORD_MIN_ROWS && D <= ORD_MAX_DIM ? c.take<unsigned long long>(1) : nullptr;
+    w.clock = !pl.filter && pl.splits == 1 && N >= ORD_MIN_ROWS && D <= ORD_MAX_DIM
+                  ? c.take<unsigned long long>(1) : nullptr;
     if (w.ordered) order_workspace(c, N, D, pl, &w.ord);
     if (ws) *ws = w;
     return c.bytes();
 }
 
+// The BF16 copies of the rows given up by the fixed threshold, one warp per row.
+__global__ void __launch_bounds__(256)
+knn_gather_kernel(const int32_t *__restrict__ rows, const int32_t *__restrict__ count, int Dp,
+                  const uint16_t *__restrict__ hi, const uint16_t *__restrict__ lo, uint16_t *__restrict__ rhi,
+                  uint16_t *__restrict__ rlo) {
+    const int lane = threadIdx.x & 31, n = *count;
+    for (int r = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); r < n; r += (int)(gridDim.x * blockDim.x) >> 5) {
+        const int64_t a = (int64_t)rows[r] * Dp, b = (int64_t)r * Dp;
+        for (int t = lane; t < (Dp >> 3); t += 32) {
+            reinterpret_cast<uint4 *>(rhi + b)[t] = reinterpret_cast<const uint4 *>(hi + a)[t];
+            if (lo) reinterpret_cast<uint4 *>(rlo + b)[t] = reinterpret_cast<const uint4 *>(lo + a)[t];
+        }
+    }
+}
+
+// The merge of a launch's buffers over `grid` blocks.
+static atsne_status merge_launch(const TcPlan &pl, MergeParams m, int grid, cudaStream_t stream) {
+    if (!pl.certify) {
+        // the re-rank set is the ksel best keys (ties included); the staged
+        // keys are those below the lowest tau, about twice as many
+        int rc = 64;
+        while (rc < pl.ksel + pl.ksel / 4) rc <<= 1;
+        m.rc = rc < RCAP_FP8 ? rc : RCAP_FP8;
+        m.mst = (m.rc + merge_reg_keys(false)) / 2;  // the re-rank set and the indices of keys in registers
+    } else {
+        m.rc = RCAP;
+        m.mst = MSTAGE;
+    }
+    static_assert(2 * MSTAGE >= merge_reg_keys(true), "indices of keys in registers");
+    const size_t ms = merge_smem_bytes(pl.certify, m.rc, m.mst);
+    void (*kern)(MergeParams) = pl.certify ? knn_merge_kernel<true> : knn_merge_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ms);
+    if (e != cudaSuccess) return cuda_error(e, "knn_tc_merge attribute");
+    return launch_kernel("knn_tc_merge", kern, grid, MERGE_WARPS * 32, ms, stream, m);
+}
+
 atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist, int64_t Q, int k,
                           const TcPlan &pl, const TcWs &w, int32_t *idx_out, float *d2_out,
-                          cudaStream_t stream, const float *Xq, const float *radius, const float *hint) {
+                          cudaStream_t stream, const float *Xq, const float *radius, const float *hint,
+                          const int64_t *qcount) {
     int *status = device_status_word();
     cudaError_t e = cudaMemsetAsync(w.gmax, 0, 4 * sizeof(unsigned), stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(w.flag_count, 0, sizeof(int32_t), stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w.flag_count, 0, 2 * sizeof(int32_t), stream);
     if (e == cudaSuccess && w.clock) e = cudaMemsetAsync(w.clock, 0, sizeof(unsigned long long), stream);
     if (e == cudaSuccess && w.row_hist)
-        e = cudaMemsetAsync(w.row_hist, 0, (size_t)Q * GH_BUCKETS * sizeof(unsigned), stream);
+        e = cudaMemsetAsync(w.row_hist, 0, (size_t)w.hist_rows * GH_BUCKETS * sizeof(unsigned), stream);
     // a unit that a timed-out kernel never finished reads as an empty buffer
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(w.meta, 0, (size_t)Q * pl.splits * pl.halves * sizeof(int4), stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w.meta, 0, w.metas * sizeof(int4), stream);
     if (e != cudaSuccess) return cuda_error(e, "knn_tc memset");
     const bool fp8 = pl.passes == 8;
     const void *a_hi = w.hi, *a_lo = w.lo;
@@ -1731,12 +1940,13 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
         auto *lo = reinterpret_cast<__nv_bfloat16 *>(w.lo);
         // ordered rows and columns: the copies, norms and statistics in the order
         if (ordered) ATSNE_TRY(knn_order_launch(X, N, D, pl, TC_BM, TC_BN, w.ord, stream));
-        ATSNE_TRY(launch_kernel("knn_prep", knn_prep_kernel, ceil_div(N * 32, 256), 256, 0, stream, X,
+        const int64_t prows = w.bext ? (N + TC_BN - 1) / TC_BN * TC_BN : N;  // the norm slices fill whole tiles
+        ATSNE_TRY(launch_kernel("knn_prep", knn_prep_kernel, ceil_div(prows * 32, 256), 256, 0, stream, X,
                                 ordered ? (const int32_t *)w.ord.perm : (const int32_t *)nullptr, N, N, D,
                                 pl.Dp, pl.passes, hi, lo, w.nrm,
                                 reinterpret_cast<float4 *>(w.stats), w.gmax,
                                 reinterpret_cast<__nv_bfloat16 *>(w.bext),
-                                reinterpret_cast<__nv_bfloat16 *>(w.aext), status));
+                                reinterpret_cast<__nv_bfloat16 *>(pl.passes == 1 ? w.aext : nullptr), status));
         if (Xq) {
             ATSNE_TRY(launch_kernel("knn_prep", knn_prep_kernel, ceil_div(Q * 32, 256), 256, 0, stream, Xq,
                                     (const int32_t *)nullptr, Q, Q, D, pl.Dp, pl.passes,
@@ -1757,25 +1967,94 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
             a_lo = w.qlo;
         }
     }
+    // queries that are corpus rows have the corpus' low halves
+    const unsigned *lo_max = pl.passes == 3 && !Xq ? w.gmax + 2 : nullptr;
+    const float acc_coef = acc_coef_of(pl), sq_coef = pl.passes == 1 ? 0.5f * acc_coef : 0.f;
+    MergeParams m;
+    memset(&m, 0, sizeof(m));
+    m.Q = Q;
+    m.N = N;
+    m.qlist = qlist;
+    m.perm = ordered ? w.ord.perm : nullptr;
+    m.X = X;
+    m.D = D;
+    m.k = k;
+    m.nrm = w.nrm;
+    m.stats = reinterpret_cast<const float4 *>(w.stats);
+    m.Xq = Xq;
+    m.qnrm = w.qnrm;
+    m.qstats = reinterpret_cast<const float4 *>(w.qstats);
+    m.gmax = w.gmax;
+    m.acc_coef = acc_coef;
+    m.sq_coef = sq_coef;
+    m.idx_out = idx_out;
+    m.d2_out = d2_out;
+    m.ksel = pl.ksel;
+    m.cand = reinterpret_cast<const Cand *>(w.cand);
+    m.meta = reinterpret_cast<const int4 *>(w.meta);
+    m.qcount = qcount;
+    m.bufs = Q * (int64_t)pl.splits;
+    // the fixed-threshold launch; the rows it gives up follow in the adaptive one
+    const bool retry = pl.filter && !radius;
+    if (pl.filter) {
+        FilterArgs f;
+        f.a_hi = a_hi;
+        f.a_lo = a_lo;
+        f.a_rows = (qlist || Xq) ? Q : N;
+        f.Q = Q;
+        f.N = N;
+        f.D = D;
+        f.qlist = qlist;
+        f.cross = Xq != nullptr;
+        f.radius = radius;
+        f.hint = hint;
+        f.lo_max = lo_max;
+        f.acc_coef = acc_coef;
+        f.sq_coef = sq_coef;
+        f.qcount = qcount;
+        ATSNE_TRY(knn_filter_launch(pl, w, f, stream));
+        m.splits = pl.fsplits * F_PARTS;
+        m.cap = pl.fcap;
+        m.tag = META_FIRST;
+        m.flag_out = !retry;
+        m.flag_rows = retry ? w.retry_rows : w.flag_rows;
+        m.flag_count = retry ? w.flag_count + 1 : w.flag_count;
+        if (radius) {
+            ATSNE_TRY(launch_kernel("knn_tc_merge", radius_merge_kernel, ceil_div(Q, MERGE_WARPS),
+                                    MERGE_WARPS * 32, 0, stream, m, radius));
+            ATSNE_TRY(knn_bruteforce_rows(X, N, D, qlist, w.flag_rows, w.flag_count, Q, k, idx_out, d2_out,
+                                          stream, Xq));
+            return launch_kernel("radius_filter", radius_filter_kernel, ceil_div(Q * k, 256), 256, 0, stream,
+                                 idx_out, d2_out, Q, k, radius);
+        }
+        ATSNE_TRY(merge_launch(pl, m, ceil_div(Q, MERGE_WARPS), stream));
+        ATSNE_TRY(launch_kernel("knn_gather", knn_gather_kernel, (int)hmin(4 * num_sms(), ceil_div(Q * 32, 256)), 256,
+                                0, stream, (const int32_t *)w.retry_rows, (const int32_t *)(w.flag_count + 1), pl.Dp,
+                                reinterpret_cast<const uint16_t *>(a_hi), reinterpret_cast<const uint16_t *>(a_lo),
+                                w.rhi, w.rlo));
+        a_hi = w.rhi;
+        a_lo = w.rlo;
+    }
+    const int64_t a_rows = (qlist || Xq || retry) ? Q : N;
     TcParams p;
     memset(&p, 0, sizeof(p));
     if (fp8) {
-        ATSNE_TRY(make_u8_map(&p.tm_a_hi, a_hi, (qlist || Xq) ? Q : N, pl.Dp, TC_BM));
+        ATSNE_TRY(make_u8_map(&p.tm_a_hi, a_hi, a_rows, pl.Dp, TC_BM));
         ATSNE_TRY(make_u8_map(&p.tm_b_hi, w.hi, N, pl.Dp, TC_BN));
     } else {
-        ATSNE_TRY(make_bf16_map(&p.tm_a_hi, a_hi, (qlist || Xq) ? Q : N, pl.Dp, TC_BM));
-        ATSNE_TRY(make_bf16_map(&p.tm_b_hi, w.hi, N, pl.Dp, TC_BN));
+        ATSNE_TRY(tc_map_bf16(&p.tm_a_hi, a_hi, a_rows, pl.Dp, TC_BM));
+        ATSNE_TRY(tc_map_bf16(&p.tm_b_hi, w.hi, N, pl.Dp, TC_BN));
     }
     if (pl.passes == 1) {
-        ATSNE_TRY(make_ext_map(&p.tm_a_ext, w.aext, TC_BM, TC_BM));
-        ATSNE_TRY(make_ext_map(&p.tm_b_ext, w.bext, N, TC_BN));
+        ATSNE_TRY(tc_map_ext(&p.tm_a_ext, w.aext, TC_BM, TC_BM));
+        ATSNE_TRY(tc_map_ext(&p.tm_b_ext, w.bext, N, TC_BN));
     } else {
         p.tm_a_ext = p.tm_a_hi;
         p.tm_b_ext = p.tm_b_hi;
     }
     if (pl.passes == 3) {
-        ATSNE_TRY(make_bf16_map(&p.tm_a_lo, a_lo, (qlist || Xq) ? Q : N, pl.Dp, TC_BM));
-        ATSNE_TRY(make_bf16_map(&p.tm_b_lo, w.lo, N, pl.Dp, TC_BN));
+        ATSNE_TRY(tc_map_bf16(&p.tm_a_lo, a_lo, a_rows, pl.Dp, TC_BM));
+        ATSNE_TRY(tc_map_bf16(&p.tm_b_lo, w.lo, N, pl.Dp, TC_BN));
     } else {
         p.tm_a_lo = p.tm_a_hi;
         p.tm_b_lo = p.tm_b_hi;
@@ -1783,18 +2062,19 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
     p.scale = w.scale;
     p.qscale = (qlist || Xq) ? w.qscale : nullptr;
     p.qnrm = Xq ? w.qnrm : nullptr;
-    p.radius = radius;
     p.hint = hint;
-    p.pro = ordered ? w.ord.pro : nullptr;
+    p.pro = ordered && !retry ? w.ord.pro : nullptr;
+    p.rlist = retry ? w.retry_rows : nullptr;
+    p.rcount = retry ? w.flag_count + 1 : nullptr;
+    p.bufs = m.bufs;
     p.clock = w.clock;
     p.qst = reinterpret_cast<const float4 *>(w.qstats);
     p.st = reinterpret_cast<const float4 *>(w.stats);
-    p.acc_coef = acc_coef_of(pl);
-    p.sq_coef = pl.passes == 1 ? 0.5f * p.acc_coef : 0.f;
+    p.acc_coef = acc_coef;
+    p.sq_coef = sq_coef;
     p.nrm = w.nrm;
     p.gmax = w.gmax;
-    // queries that are corpus rows have the corpus' low halves
-    p.lo_max = pl.passes == 3 && !Xq ? w.gmax + 2 : nullptr;
+    p.lo_max = lo_max;
     p.qlist = qlist;
     p.Q = Q;
     p.N = N;
@@ -1810,7 +2090,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
     p.status = status;
     p.wait_ns = pipeline_wait_ns();
     const int units = pl.row_tiles * pl.splits;
-    const int grid = (int)hmin(units, num_sms());
+    const int grid = retry ? num_sms() : (int)hmin(units, num_sms());
     if (pl.passes == 3) {
         const size_t smem = tc_smem_bytes<3>();
         e = cudaFuncSetAttribute(knn_tc_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1827,60 +2107,18 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
         if (e != cudaSuccess) return cuda_error(e, "knn_tc attribute");
         ATSNE_TRY(launch_kernel("knn_tc", knn_tc_kernel<1>, grid, TcCfg<1>::THREADS, smem, stream, p));
     }
-    MergeParams m;
-    m.cand = p.cand;
-    m.meta = p.meta;
-    m.splits = pl.splits * pl.halves;  // candidate buffers per row
+    // buffers per row: of a split where the splits are known on the device only
+    m.splits = retry ? pl.halves : pl.splits * pl.halves;
     m.cap = pl.cap;
-    m.Q = Q;
-    m.N = N;
-    m.qlist = qlist;
-    m.perm = ordered ? w.ord.perm : nullptr;
-    m.X = X;
-    m.D = D;
-    m.k = k;
-    m.nrm = w.nrm;
-    m.stats = reinterpret_cast<const float4 *>(w.stats);
-    m.Xq = Xq;
-    m.qnrm = w.qnrm;
-    m.qstats = reinterpret_cast<const float4 *>(w.qstats);
-    m.gmax = w.gmax;
-    m.acc_coef = acc_coef_of(pl);
-    m.sq_coef = pl.passes == 1 ? 0.5f * m.acc_coef : 0.f;
-    m.idx_out = idx_out;
-    m.d2_out = d2_out;
+    m.rlist = p.rlist;
+    m.rcount = p.rcount;
+    m.tag = retry ? META_RETRY : META_FIRST;
+    m.flag_out = true;
     m.flag_rows = w.flag_rows;
     m.flag_count = w.flag_count;
-    m.ksel = pl.ksel;
-    if (radius) {
-        ATSNE_TRY(launch_kernel("knn_tc_merge", radius_merge_kernel, ceil_div(Q, MERGE_WARPS),
-                                MERGE_WARPS * 32, 0, stream, m, radius));
-        ATSNE_TRY(knn_bruteforce_rows(X, N, D, qlist, w.flag_rows, w.flag_count, Q, k, idx_out, d2_out,
-                                      stream, Xq));
-        return launch_kernel("radius_filter", radius_filter_kernel, ceil_div(Q * k, 256), 256, 0, stream,
-                             idx_out, d2_out, Q, k, radius);
-    }
-    if (!pl.certify) {
-        // the re-rank set is the ksel best keys (ties included); the staged
-        // keys are those below the lowest tau, about twice as many
-        int rc = 64;
-        while (rc < pl.ksel + pl.ksel / 4) rc <<= 1;
-        m.rc = rc < RCAP_FP8 ? rc : RCAP_FP8;
-        m.mst = 2 * m.rc;
-        const size_t ms = merge_smem_bytes(false, m.rc, m.mst);
-        e = cudaFuncSetAttribute(knn_merge_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ms);
-        if (e != cudaSuccess) return cuda_error(e, "knn_tc_merge attribute");
-        ATSNE_TRY(launch_kernel("knn_tc_merge", knn_merge_kernel<false>, ceil_div(Q, MERGE_WARPS),
-                                MERGE_WARPS * 32, ms, stream, m));
-    } else {
-        m.rc = RCAP;
-        m.mst = MSTAGE;
-        const size_t ms = merge_smem_bytes(true, m.rc, m.mst);
-        e = cudaFuncSetAttribute(knn_merge_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ms);
-        if (e != cudaSuccess) return cuda_error(e, "knn_tc_merge attribute");
-        ATSNE_TRY(launch_kernel("knn_tc_merge", knn_merge_kernel<true>, ceil_div(Q, MERGE_WARPS),
-                                MERGE_WARPS * 32, ms, stream, m));
-    }
+    ATSNE_TRY(merge_launch(pl, m,
+                           retry ? (int)hmin(4 * num_sms(), ceil_div(Q, MERGE_WARPS)) : ceil_div(Q, MERGE_WARPS),
+                           stream));
     return knn_bruteforce_rows(X, N, D, qlist, w.flag_rows, w.flag_count, Q, k, idx_out, d2_out, stream,
                                Xq);
 }
