@@ -37,22 +37,23 @@ __device__ __forceinline__ float key_error_bound(float4 st, const unsigned *gmax
     const float rmax = __uint_as_float(gmax[1]);
     const float lmax = __uint_as_float(gmax[2]);
     const float a = st.x, r = st.y, l = st.z;
-    const float drop = l * lmax + r * amax + a * rmax;
+    const float drop = l * lmax + r * amax + (a + r) * rmax;
     return 2.f * drop + acc_coef * a * amax + (4e-6f + sq_coef) * amax * amax + 4e-6f * a * a;
 }
 
 // The same bound over the corpus points of norm at most amax_cap only (a
 // point farther in norm than sqrt(d) from the query is farther than sqrt(d)
-// in distance). Their residuals are capped by the BF16 rounding bound:
-// ||x - hi|| <= 2^-9 ||x|| and ||lo|| <= 2^-8 ||x|| (round to nearest, 8
-// significand bits), plus a tiny absolute term for subnormal values.
+// in distance). Their residuals are capped by the BF16 rounding bound, the unit
+// roundoff 2^-8 of 8 significand bits rounded to nearest (257 becomes 256):
+// ||x - hi|| and ||lo|| are at most 2^-8 ||x||, plus a tiny absolute term for
+// subnormal values.
 __device__ __forceinline__ float key_error_bound_capped(float4 st, const unsigned *gmax, float acc_coef,
                                                         float sq_coef, float amax_cap) {
     const float amax = fminf(__uint_as_float(gmax[0]), amax_cap);
-    const float rmax = fminf(__uint_as_float(gmax[1]), 0x1p-9f * amax + 1e-30f);
+    const float rmax = fminf(__uint_as_float(gmax[1]), 0x1p-8f * amax + 1e-30f);
     const float lmax = fminf(__uint_as_float(gmax[2]), 0x1p-8f * amax + 1e-30f);
     const float a = st.x, r = st.y, l = st.z;
-    const float drop = l * lmax + r * amax + a * rmax;
+    const float drop = l * lmax + r * amax + (a + r) * rmax;
     return 2.f * drop + acc_coef * a * amax + (4e-6f + sq_coef) * amax * amax + 4e-6f * a * a;
 }
 
