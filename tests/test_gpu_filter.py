@@ -1,0 +1,86 @@
+"""The tensor-core kNN with sampled thresholds at the sizes where its tiles,
+k-steps, samples and splits have their edges, and on layouts that mislead the
+sample (their rows then take the adaptive kernel): the certified lists equal
+those of the CUDA-core kernel, index for index and bit for bit (both return
+distances in one summation order and settle near ties in FP64, the CUDA-core
+kernel those with the (k + 1)-th neighbour where its list holds it: it is asked
+for one more)."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def at():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_1512_01655_gb300 as pkg
+    return pkg
+
+
+def rows(N, D, seed, scale=1.0):
+    g = np.random.default_rng(seed)
+    return torch.from_numpy((scale * g.normal(size=(N, D))).astype(np.float32)).cuda()
+
+
+def same(at, X, k, precision="fp32", **kw):
+    i, d = at.atsne_knn(X, k, precision=precision, **kw)
+    ri, rd = at.atsne_knn(X, k + 1, precision="fp32_cuda", **kw)
+    at.atsne_check()
+    assert torch.equal(i, ri[:, :k]) and torch.equal(d, rd[:, :k])
+
+
+@pytest.mark.parametrize("N,D,k", [(1023, 16, 30), (1024, 1, 30), (1025, 17, 90), (1279, 63, 10), (1281, 65, 60),
+                                   (2049, 128, 200), (4097, 129, 5), (5000, 48, 128), (3000, 15, 1)])
+def test_tile_and_k_step_edges(at, N, D, k):
+    same(at, rows(N, D, N + D), k)
+
+
+@pytest.mark.parametrize("S", [1, 127, 129, 257, 700])
+def test_few_queries_cut_into_column_splits(at, S):
+    X = rows(9001, 40, S)
+    q = torch.from_numpy(np.random.default_rng(S).integers(0, 9001, S).astype(np.int32)).cuda()
+    same(at, X, 50, queries=q)
+
+
+def test_layouts_that_mislead_the_sample(at):
+    base = rows(40, 24, 1)
+    for X in (base.repeat(60, 1), base.repeat_interleave(60, 0),                       # exact duplicates
+              (8 * rows(256, 24, 2)).repeat_interleave(18, 0) + 0.1 * rows(4608, 24, 3),  # groups smaller than k
+              (5 * rows(32, 24, 4)).repeat(150, 1) + rows(4800, 24, 5),                 # period of 32 rows
+              rows(4000, 24, 6) * torch.exp(3 * rows(4000, 1, 7))):                     # norms over decades
+        same(at, X.contiguous(), 30)
+    i, d = at.atsne_knn(torch.ones((2000, 8), device="cuda"), 20)
+    at.atsne_check()
+    assert (d == 0).all() and (i[25] == torch.tensor([j for j in range(21) if j != 25][:20], device="cuda")).all()
+
+
+@pytest.mark.parametrize("f", [0.5, 1.0, 4.0])
+def test_hints_right_loose_and_wrong(at, f):
+    X = rows(6000, 32, 11)
+    q = torch.arange(0, 6000, 9, dtype=torch.int32, device="cuda")
+    i, d = at.atsne_knn(X, 40, queries=q, precision="fp32_cuda")
+    ti, td = at.atsne_knn_rows(X, q, 40, hint_d2=(f * d[:, -1]).contiguous())
+    at.atsne_check()
+    assert torch.equal(ti, i) and torch.equal(td, d)
+
+
+@pytest.mark.parametrize("Nq,Nc", [(1, 1024), (300, 2000), (2500, 1500), (129, 7013)])
+def test_queries_from_another_array(at, Nq, Nc):
+    Xq, Xc = rows(Nq, 50, Nq), rows(Nc, 50, Nc + 1)
+    i, d = at.atsne_knn_cross(Xq, Xc, 20)
+    ri, rd = at.atsne_knn_cross(Xq, Xc, 20, precision="fp32_cuda")
+    at.atsne_check()
+    assert torch.equal(i, ri) and torch.equal(d, rd)
+    r = (rd[:, 9] * 1.0001).contiguous()
+    r[::3], r[1::7] = 0.0, float("inf")
+    i, d = at.atsne_knn_cross(Xq, Xc, 20, radius_d2=r)
+    ri, rd = at.atsne_knn_cross(Xq, Xc, 20, radius_d2=r, precision="fp32_cuda")
+    at.atsne_check()
+    # with radii only the CUDA-core kernel replaces near ties' distances by
+    # their FP64 values: within (4 ceil(D / 32) + 8) 2^-24 of the FP32 sums
+    assert torch.equal(i, ri) and torch.equal(d.isinf(), rd.isinf())
+    fin = ~d.isinf()
+    assert ((d[fin] - rd[fin]).abs() <= 16 * 2.0 ** -24 * rd[fin]).all()
