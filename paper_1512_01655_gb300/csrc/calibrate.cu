@@ -58,11 +58,14 @@ __device__ __forceinline__ void bisect(const float *row, int k, float target, fl
 }
 
 __global__ void __launch_bounds__(CAL_THREADS)
-calibrate_kernel(const float *__restrict__ d2, int64_t rows, int k, float perplexity, float target,
-                 float tol, int max_iter, float *__restrict__ P, float *__restrict__ beta_out, int *status) {
+calibrate_kernel(const float *__restrict__ d2, int64_t rows_max, int k, float perplexity, float target,
+                 float tol, int max_iter, float *__restrict__ P, float *__restrict__ beta_out, int *status,
+                 const int64_t *__restrict__ count) {
     extern __shared__ float sm[];
     const int stride = k | 1;
+    const int64_t rows = count ? min(*count, rows_max) : rows_max;
     const int64_t r0 = (int64_t)blockIdx.x * CAL_THREADS;
+    if (r0 >= rows) return;
     const int nr = (int)(rows - r0 < CAL_THREADS ? rows - r0 : CAL_THREADS);
     const float *src = d2 + r0 * k;
     for (int t = threadIdx.x; t < nr * k; t += CAL_THREADS) {
@@ -117,7 +120,7 @@ calibrate_kernel(const float *__restrict__ d2, int64_t rows, int k, float perple
 size_t calibrate_smem_bytes(int k) { return sizeof(float) * CAL_THREADS * (size_t)(k | 1); }
 
 atsne_status calibrate_launch(const float *d2, int64_t rows, int k, float perplexity, float tol,
-                              int max_iter, float *P, float *beta, cudaStream_t stream) {
+                              int max_iter, float *P, float *beta, cudaStream_t stream, const int64_t *count) {
     if (rows <= 0) return ATSNE_OK;
     const size_t smem = calibrate_smem_bytes(k);
     static size_t attr = 0;
@@ -129,7 +132,7 @@ atsne_status calibrate_launch(const float *d2, int64_t rows, int k, float perple
     }
     return launch_kernel("calibrate_beta", calibrate_kernel, ceil_div(rows, CAL_THREADS),
                          CAL_THREADS, smem, stream, d2, rows, k, perplexity, logf(perplexity), tol, max_iter, P,
-                         beta, device_status_word());
+                         beta, device_status_word(), count);
 }
 
 }  // namespace atsne

@@ -100,7 +100,8 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
 // ---- calibrate ------------------------------------------------------------
 size_t calibrate_smem_bytes(int k);
 atsne_status calibrate_launch(const float *d2, int64_t rows, int k, float perplexity, float tol,
-                              int max_iter, float *P, float *beta, cudaStream_t stream);
+                              int max_iter, float *P, float *beta, cudaStream_t stream,
+                              const int64_t *count = nullptr);  // the rows in use (device; at most `rows`)
 
 // ---- symmetrize -------------------------------------------------------------
 struct SymWs {
@@ -155,7 +156,7 @@ atsne_status u8_copy_launch(const char *name, const float *X, int64_t N, int D, 
 atsne_status refine_scatter_launch(const int32_t *subset, int64_t S, int64_t N, int k, const int32_t *ti,
                                    const float *td, const float *tp, const float *tb, int32_t *idx,
                                    float *d2, float *P, float *beta, float *rho,
-                                   cudaStream_t stream);
+                                   cudaStream_t stream, const int64_t *count = nullptr);
 
 // ---- forest -------------------------------------------------------------------
 struct ForestView {

@@ -307,9 +307,11 @@ __global__ void __launch_bounds__(256)
 knn_prep_kernel(const float *__restrict__ X, const int32_t *__restrict__ rows, int64_t nrows, int64_t N,
                 int D, int Dp, int passes, __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo,
                 float *__restrict__ nrm, float4 *__restrict__ stats, unsigned *__restrict__ gmax,
-                __nv_bfloat16 *__restrict__ bext, __nv_bfloat16 *__restrict__ aext, int *status) {
+                __nv_bfloat16 *__restrict__ bext, __nv_bfloat16 *__restrict__ aext, int *status,
+                const int64_t *__restrict__ count) {
     const int lane = threadIdx.x & 31;
     const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (count) nrows = min(*count, nrows);
     if (aext && blockIdx.x == 0) fold_query_slice(aext);
     // the norm slices of the rows that fill the last column tile: +inf, a key no row keeps
     if (bext && r >= nrows && r < (nrows + TC_BN - 1) / TC_BN * TC_BN && lane < 16)
@@ -1946,14 +1948,16 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
                                 pl.Dp, pl.passes, hi, lo, w.nrm,
                                 reinterpret_cast<float4 *>(w.stats), w.gmax,
                                 reinterpret_cast<__nv_bfloat16 *>(w.bext),
-                                reinterpret_cast<__nv_bfloat16 *>(pl.passes == 1 ? w.aext : nullptr), status));
+                                reinterpret_cast<__nv_bfloat16 *>(pl.passes == 1 ? w.aext : nullptr), status,
+                                (const int64_t *)nullptr));
         if (Xq) {
             ATSNE_TRY(launch_kernel("knn_prep", knn_prep_kernel, ceil_div(Q * 32, 256), 256, 0, stream, Xq,
                                     (const int32_t *)nullptr, Q, Q, D, pl.Dp, pl.passes,
                                     reinterpret_cast<__nv_bfloat16 *>(w.qhi),
                                     reinterpret_cast<__nv_bfloat16 *>(w.qlo), w.qnrm,
                                     reinterpret_cast<float4 *>(w.qstats), (unsigned *)nullptr,
-                                    (__nv_bfloat16 *)nullptr, (__nv_bfloat16 *)nullptr, status));
+                                    (__nv_bfloat16 *)nullptr, (__nv_bfloat16 *)nullptr, status,
+                                    (const int64_t *)nullptr));
             a_hi = w.qhi;
             a_lo = w.qlo;
         } else if (qlist) {
@@ -1962,7 +1966,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
                                     reinterpret_cast<__nv_bfloat16 *>(w.qhi),
                                     reinterpret_cast<__nv_bfloat16 *>(w.qlo), (float *)nullptr,
                                     (float4 *)nullptr, (unsigned *)nullptr, (__nv_bfloat16 *)nullptr,
-                                    (__nv_bfloat16 *)nullptr, status));
+                                    (__nv_bfloat16 *)nullptr, status, qcount));
             a_hi = w.qhi;
             a_lo = w.qlo;
         }

@@ -49,9 +49,9 @@ __global__ void refine_scatter_kernel(const int32_t *__restrict__ subset, int64_
                                       const float *__restrict__ tp, const float *__restrict__ tb,
                                       int32_t *__restrict__ idx, float *__restrict__ d2,
                                       float *__restrict__ P, float *__restrict__ beta,
-                                      float *__restrict__ rho) {
+                                      float *__restrict__ rho, const int64_t *__restrict__ count) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= S * k) return;
+    if (e >= (count ? min(*count, S) : S) * k) return;
     const int64_t s = e / k;
     const int t = (int)(e - s * k);
     const int64_t i = subset[s];
@@ -348,10 +348,10 @@ atsne_status precision_launch(const int32_t *a, const int32_t *e, int64_t rows, 
 atsne_status refine_scatter_launch(const int32_t *subset, int64_t S, int64_t N, int k, const int32_t *ti,
                                    const float *td, const float *tp, const float *tb, int32_t *idx,
                                    float *d2, float *P, float *beta, float *rho,
-                                   cudaStream_t stream) {
+                                   cudaStream_t stream, const int64_t *count) {
     if (S <= 0) return ATSNE_OK;
     return launch_kernel("refine_scatter", refine_scatter_kernel, ceil_div(S * k, 256), 256, 0,
-                         stream, subset, S, N, k, ti, td, tp, tb, idx, d2, P, beta, rho);
+                         stream, subset, S, N, k, ti, td, tp, tb, idx, d2, P, beta, rho, count);
 }
 
 size_t delete_workspace(Carver &c, int64_t N, int D, int k, DeleteWs *ws) {
