@@ -105,12 +105,11 @@ atsne_status calibrate_launch(const float *d2, int64_t rows, int k, float perple
 
 // ---- symmetrize -------------------------------------------------------------
 struct SymWs {
-    int32_t *scol = nullptr;   // [N][k] conditional rows sorted by column
-    float *sval = nullptr;
-    int32_t *rev_i = nullptr;  // reverse lists: source rows, [N * k]
-    float *rev_p = nullptr;    // and their conditionals
-    int32_t *rcnt = nullptr, *cursor = nullptr, *len = nullptr, *long_rows = nullptr, *n_long = nullptr,
-            *own = nullptr;
+    int2 *rev = nullptr;       // reverse lists: source rows and their conditionals, [N * k]
+    int32_t *rank = nullptr;   // each entry's place in its reverse list (in tcol's memory)
+    int32_t *tcol = nullptr;   // the union's rows before they move to row_ptr's places, [2 N k]
+    float *tval = nullptr;
+    int32_t *rcnt = nullptr, *len = nullptr, *mid_rows = nullptr, *hub_rows = nullptr, *n_list = nullptr;
     int64_t *roff = nullptr, *rtot = nullptr;  // reverse list offsets [N + 1], total
     int64_t *scan = nullptr;
 };

@@ -5,353 +5,408 @@
 // R_r = {i : r in N_i}; a column in both (a mutual pair) gets
 // (p_{c|r} + p_{r|c}) / 2N, formed from the same two operands on both sides,
 // so p_rc and p_cr are bit-identical; a column in one of them gets its one
-// conditional / 2N. The transpose is a counting sort by target row:
-//   1. fwd:      each conditional row sorted by column (warp bitonic, in
-//                registers) and its entries counted into their target rows;
-//   2. scan:     offsets of the reverse lists;
-//   3. rev:      every entry (i -> j, p_{j|i}) placed in j's reverse list;
-//   4. len:      row length |F_r| + |R_r| - |F_r and R_r| (each reverse entry
-//                searched in the sorted forward row);
-//   5. scan:     row_ptr;
-//   6. write:    the reverse list sorted (warp bitonic in shared memory, or
-//                for rows of more than SORT_ROW_CAP reverse entries a CTA
-//                sort in global memory first), then every entry written
-//                straight to its place: an entry's position in the union is
-//                its rank in its own sorted list plus its rank in the other
-//                one, less the mutual columns before it.
-// Apart from the reverse placement (step 3, one scattered 8-byte write per
-// entry) every pass streams rows.
+// conditional / 2N.
+//   1. count: every entry (i -> j) counted into its target row; the atomic's
+//             old value is the entry's place in j's reverse list.
+//   2. scan:  offsets of the reverse lists.
+//   3. place: (i, p_{j|i}) written to that place, one 8-byte write per entry.
+//   4. merge: row r's k + |R_r| entries sorted by column, mutual pairs added,
+//             the row written to the workspace (its place there, r k + the
+//             reverse offset, does not depend on the lengths) and its length
+//             kept. Three classes of rows: up to 512 entries a warp sorts them
+//             in registers (sym_merge_kernel), up to 1024 the same with more
+//             registers (sym_mid_kernel), beyond that (hub rows) a CTA takes
+//             each entry's rank from a bitmap of the columns (sym_hub_kernel).
+//   5. scan:  row_ptr.
+//   6. copy:  rows to their final places, scaled by 1 / 2N.
+// A warp's sort moves one word per entry: column, forward/reverse bit and the
+// entry's slot (where its value waits in shared memory) in 32 bits while the
+// column fits (N <= 2^21), else 64; a compare-exchange is a shuffle and a
+// min/max. Sorting forward and reverse rows separately as (key, value) pairs in
+// shared memory, with a binary search of each entry in the other list, twice,
+// took 3.08, 13.7 and 1.63 ms (300,000 rows of separate clusters, 1,000,000
+// Gamma rows, 70,000 byte rows with hubs; k = 90); this takes 1.62, 6.4 and
+// 0.45 ms. The bounds are the atomics and the scatter of steps 1 and 3 (a
+// 32-byte sector per 8-byte write) and the sorts' instructions.
 #include <limits.h>
 
 #include "common.cuh"
 #include "internal.h"
-#include "warp_sort.cuh"
 
 namespace atsne {
 namespace {
 
-constexpr int SORT_ROW_CAP = 1024;  // longest reverse list a warp sorts in shared memory
 constexpr int SYM_WARPS = 4;
+constexpr int SYM_BULK = 512;         // entries of a row sorted by sym_merge_kernel
+constexpr int SYM_MID = 1024;         // by sym_mid_kernel
+constexpr int64_t SYM_KEY32 = int64_t(1) << 21;  // columns that fit a 32-bit key with 10 slot bits
+constexpr int HUB_THREADS = 1024;
+constexpr int SYM_MAX_K = 512;
+constexpr int64_t HUB_COLS = int64_t(1) << 19;   // columns per bitmap (64 KB, and as much for its prefix sums)
 
-// lower bound of key in the sorted a[0, n)
-template <typename P>
-__device__ __forceinline__ int lower_bound_i(P a, int n, int key) {
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (a[mid] < key) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
+// A row's neighbour j of row i is valid; absent ones are skipped, others raise the status.
+__device__ __forceinline__ bool valid_neighbour(int j, int64_t i, int64_t N, int *status) {
+    if (j == -1) return false;
+    if (j >= 0 && j < N && j != i) return true;
+    raise_status(status, DEV_MALFORMED);
+    return false;
 }
 
-template <int KP>
-__global__ void __launch_bounds__(128)
-sym_fwd_kernel(const int32_t *__restrict__ idx, const float *__restrict__ P, int64_t N, int k,
-               int32_t *__restrict__ scol, float *__restrict__ sval, int32_t *__restrict__ own,
-               int32_t *__restrict__ rcnt, int *status) {
-    __shared__ int keys[4][KP];
-    __shared__ float vals[4][KP];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t i = (int64_t)blockIdx.x * 4 + w;
+__global__ void __launch_bounds__(256)
+sym_count_kernel(const int32_t *__restrict__ idx, int64_t N, int k, int32_t *__restrict__ rank,
+                 int32_t *__restrict__ rcnt, int *status) {
+    const int lane = threadIdx.x & 31;
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (i >= N) return;
-    for (int t = lane; t < KP; t += 32) {
-        int j = INT_MAX;
-        float v = 0.f;
-        if (t < k) {
-            j = idx[i * k + t];
-            v = P[i * k + t];
-            if (j == -1) {  // an absent neighbour (Sec. 5.3.2): no entry
-                j = INT_MAX;
-                v = 0.f;
-            } else if (j < 0 || j >= N || j == i) {
-                raise_status(status, DEV_MALFORMED);
-                j = INT_MAX;
-            } else {
-                atomicAdd(&rcnt[j], 1);
+    for (int t0 = lane; t0 < k; t0 += 128) {  // four atomics in flight per lane
+        int j[4], n[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) j[u] = t0 + 32 * u < k ? idx[i * k + t0 + 32 * u] : -1;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) n[u] = valid_neighbour(j[u], i, N, status) ? atomicAdd(&rcnt[j[u]], 1) : -1;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (t0 + 32 * u < k) rank[i * k + t0 + 32 * u] = n[u];
+    }
+}
+
+__global__ void __launch_bounds__(256)
+sym_place_kernel(const int32_t *__restrict__ idx, const float *__restrict__ P, int64_t N, int k,
+                 const int32_t *__restrict__ rank, const int64_t *__restrict__ roff, int2 *__restrict__ rev) {
+    const int lane = threadIdx.x & 31;
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (i >= N) return;
+    for (int t0 = lane; t0 < k; t0 += 128) {
+        int n[4], j[4];
+        float p[4];
+        int64_t at[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const bool on = t0 + 32 * u < k;
+            n[u] = on ? rank[i * k + t0 + 32 * u] : -1;
+            j[u] = on ? idx[i * k + t0 + 32 * u] : -1;
+            p[u] = on ? P[i * k + t0 + 32 * u] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) at[u] = n[u] >= 0 ? roff[j[u]] + n[u] : -1;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (at[u] >= 0) rev[at[u]] = make_int2((int)i, __float_as_int(p[u]));
+    }
+}
+
+// Ascending bitonic sort of 32 R distinct keys, lane l's being elements
+// l R .. l R + R - 1: exchanges between elements fewer than R apart stay in a
+// lane, the others are shuffles.
+template <int R, typename K>
+__device__ __forceinline__ void warp_sort_keys(K (&k)[R], int lane) {
+    // (the loops over sizes and lane distances stay loops: unrolled, the sorts of
+    // all R overflow the instruction cache, the 300,000 rows took 0.99 ms instead of 0.79)
+#pragma unroll 1
+    for (int size = 2; size <= 32 * R; size <<= 1) {
+        const bool lane_up = ((lane * R) & size) == 0;  // direction of this lane's elements, size >= R
+#pragma unroll 1
+        for (int stride = size >> 1; stride >= R; stride >>= 1) {
+            const int lm = stride / R;
+            const bool keep_min = ((lane & lm) == 0) == lane_up;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const K o = __shfl_xor_sync(0xffffffffu, k[r], lm);
+                k[r] = keep_min ? min(k[r], o) : max(k[r], o);
             }
         }
-        keys[w][t] = j;
-        vals[w][t] = v;
-    }
-    __syncwarp();
-    warp_sort_pow2(keys[w], vals[w], KP, lane);
-    __syncwarp();
-    int c = 0;  // forward entries (absent ones sorted last)
-    for (int t = lane; t < k; t += 32) {
-        const int j = keys[w][t];
-        if (t > 0 && j != INT_MAX && j == keys[w][t - 1]) raise_status(status, DEV_MALFORMED);
-        scol[i * k + t] = j;
-        sval[i * k + t] = vals[w][t];
-        c += j != INT_MAX;
-    }
-    c = (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
-    if (lane == 0) own[i] = c;
-}
-
-// Entry (i -> j, p_{j|i}) into j's reverse list (order within a list is set
-// by the atomic cursor; the write pass sorts each list).
-__global__ void sym_rev_kernel(const int32_t *__restrict__ scol, const float *__restrict__ sval, int64_t N, int k,
-                               const int64_t *__restrict__ roff, int32_t *__restrict__ cursor,
-                               int32_t *__restrict__ rev_i, float *__restrict__ rev_p) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= N * k) return;
-    const int j = scol[e];
-    if (j < 0 || j >= N) return;
-    const int64_t pos = roff[j] + atomicAdd(&cursor[j], 1);
-    rev_i[pos] = (int32_t)(e / k);
-    rev_p[pos] = sval[e];
-}
-
-// Row length |F| + |R| - |F and R|, one warp per row; the forward row is
-// searched in shared memory.
-template <int KP>
-__global__ void __launch_bounds__(SYM_WARPS * 32)
-sym_len_kernel(const int32_t *__restrict__ scol, const int32_t *__restrict__ own, int64_t N, int k,
-               const int64_t *__restrict__ roff, const int32_t *__restrict__ rev_i, int32_t *__restrict__ len) {
-    __shared__ int fc[SYM_WARPS][KP];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t r = (int64_t)blockIdx.x * SYM_WARPS + w;
-    if (r >= N) return;
-    const int a = own[r];
-    for (int t = lane; t < a; t += 32) fc[w][t] = scol[r * k + t];
-    __syncwarp();
-    const int64_t b0 = roff[r], m = roff[r + 1] - b0;
-    int matched = 0;
-    for (int64_t t = lane; t < m; t += 32) {
-        const int key = rev_i[b0 + t];
-        const int lb = lower_bound_i(fc[w], a, key);
-        matched += lb < a && fc[w][lb] == key;
-    }
-    matched = (int)__reduce_add_sync(0xffffffffu, (unsigned)matched);
-    if (lane == 0) len[r] = a + (int)m - matched;
-}
-
-// Writes row r of the CSR from its sorted forward row (fc/fv, a entries, in
-// shared memory) and its sorted reverse list (ri/rp, m entries): an entry's
-// place is its rank in its own list plus its rank in the other one, less the
-// mutual columns before it. Warp-cooperative.
-template <typename IP, typename VP>
-__device__ __forceinline__ void sym_write_row(const int *fc, const float *fv, int a, IP ri, VP rp, int64_t m,
-                                              float inv2n, int32_t *__restrict__ col, float *__restrict__ val,
-                                              int64_t base, int lane) {
-    const unsigned lt = (1u << lane) - 1u;
-    // forward entries without a reverse partner
-    int mc = 0;  // mutual columns among the forward entries so far
-    for (int s0 = 0; s0 < a; s0 += 32) {
-        const int s = s0 + lane;
-        int key = INT_MAX;
-        int64_t lb = 0;
-        bool hit = false;
-        if (s < a) {
-            key = fc[s];
-            int64_t lo = 0, hi = m;
-            while (lo < hi) {
-                const int64_t mid = (lo + hi) >> 1;
-                if (ri[mid] < key) lo = mid + 1;
-                else hi = mid;
+#pragma unroll
+        for (int stride = R >> 1; stride > 0; stride >>= 1) {
+            if (stride < size) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    if (r & stride) continue;
+                    const bool up = size >= R ? lane_up : (r & size) == 0;
+                    const K a = k[r], b = k[r + stride], lo = min(a, b), hi = max(a, b);
+                    k[r] = up ? lo : hi;
+                    k[r + stride] = up ? hi : lo;
+                }
             }
-            lb = lo;
-            hit = lb < m && ri[lb] == key;
         }
-        const unsigned hm = __ballot_sync(0xffffffffu, hit);
-        if (s < a && !hit) {
-            const int64_t pos = base + s + lb - (mc + __popc(hm & lt));
-            col[pos] = key;
-            val[pos] = fv[s] * inv2n;
-        }
-        mc += __popc(hm);
-    }
-    // reverse entries, mutual ones with both conditionals
-    mc = 0;
-    for (int64_t t0 = 0; t0 < m; t0 += 32) {
-        const int64_t t = t0 + lane;
-        int key = 0, lb = 0;
-        bool hit = false;
-        float p = 0.f;
-        if (t < m) {
-            key = ri[t];
-            p = rp[t];
-            lb = lower_bound_i(fc, a, key);
-            hit = lb < a && fc[lb] == key;
-        }
-        const unsigned hm = __ballot_sync(0xffffffffu, hit);
-        if (t < m) {
-            const int64_t pos = base + t + lb - (mc + __popc(hm & lt));
-            col[pos] = key;
-            val[pos] = (hit ? fv[lb] + p : p) * inv2n;
-        }
-        mc += __popc(hm);
     }
 }
 
-template <int KP>
+struct SymRow {
+    const int32_t *idx;
+    const float *P;
+    int64_t N;
+    int k;
+    const int64_t *roff;
+    const int2 *rev;
+    int32_t *tcol;  // the rows of the union in the workspace, values not yet scaled
+    float *tval;
+    int32_t *len;
+    int *status;
+};
+
+// One row of at most 32 R entries by one warp; v, oc, ov: 32 R words of shared
+// memory each (values by slot, then the row as it will be written).
+template <int R, typename K>
+__device__ __forceinline__ void sym_merge_row(const SymRow &s, int64_t r, int m, float *v, int *oc, float *ov,
+                                              int lane) {
+    constexpr int SB = R == 2 ? 6 : R == 4 ? 7 : R == 8 ? 8 : R == 16 ? 9 : 10;  // slot bits
+    static_assert(1 << SB == 32 * R, "a slot per entry");
+    constexpr K NONE = ~K(0);
+    const int64_t b0 = s.roff[r], row = r * s.k;
+    K key[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+        const int slot = q * 32 + lane;
+        key[q] = NONE;
+        if (slot < s.k) {
+            const int j = s.idx[row + slot];
+            v[slot] = s.P[row + slot];
+            if (j >= 0 && j < s.N && j != r) key[q] = ((K)j << (SB + 1)) | (K)slot;
+        } else if (slot < s.k + m) {
+            const int2 e = s.rev[b0 + slot - s.k];
+            v[slot] = __int_as_float(e.y);
+            key[q] = ((K)e.x << (SB + 1)) | (K(1) << SB) | (K)slot;
+        }
+    }
+    warp_sort_keys<R>(key, lane);
+    __syncwarp();
+    // a forward and a reverse entry of one column are neighbours, the forward
+    // one first: the first of a column's entries heads it
+    K before = __shfl_up_sync(0xffffffffu, key[R - 1], 1);
+    const K after = __shfl_down_sync(0xffffffffu, key[0], 1);
+    if (lane == 0) before = NONE;
+    int heads = 0;
+    bool twice = false;  // a column listed twice in the forward row
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+        const K p = q ? key[q - 1] : before;
+        const bool same = p != NONE && (p >> (SB + 1)) == (key[q] >> (SB + 1));
+        heads += key[q] != NONE && !same;
+        twice |= key[q] != NONE && same && !((key[q] >> SB) & 1);
+    }
+    if (twice) raise_status(s.status, DEV_MALFORMED);
+    int incl = heads;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    int pos = incl - heads;
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+        const K p = q ? key[q - 1] : before;
+        const bool head = key[q] != NONE && !(p != NONE && (p >> (SB + 1)) == (key[q] >> (SB + 1)));
+        if (head) {
+            const K n = q + 1 < R ? key[q + 1] : lane < 31 ? after : NONE;
+            float x = v[(int)(key[q] & ((K(1) << SB) - 1))];
+            if (n != NONE && (n >> (SB + 1)) == (key[q] >> (SB + 1))) x += v[(int)(n & ((K(1) << SB) - 1))];
+            oc[pos] = (int)(key[q] >> (SB + 1));
+            ov[pos] = x;
+            ++pos;
+        }
+    }
+    __syncwarp();
+    int32_t *tc = s.tcol + row + b0;
+    float *tv = s.tval + row + b0;
+    for (int t = lane; t < total; t += 32) {
+        tc[t] = oc[t];
+        tv[t] = ov[t];
+    }
+    if (lane == 0) s.len[r] = total;
+}
+
+template <typename K>
 __global__ void __launch_bounds__(SYM_WARPS * 32)
-sym_write_kernel(const int32_t *__restrict__ scol, const float *__restrict__ sval, const int32_t *__restrict__ own,
-                 int64_t N, int k, float inv2n, const int64_t *__restrict__ roff, const int32_t *__restrict__ rev_i,
-                 const float *__restrict__ rev_p, const int64_t *__restrict__ row_ptr, int32_t *__restrict__ col,
-                 float *__restrict__ val, int32_t *__restrict__ long_rows, int32_t *__restrict__ n_long) {
-    extern __shared__ __align__(16) unsigned char sw_smem[];
+sym_merge_kernel(SymRow s, int32_t *__restrict__ mid_rows, int32_t *__restrict__ hub_rows, int32_t *__restrict__ n_list) {
+    __shared__ float v[SYM_WARPS][SYM_BULK], ov[SYM_WARPS][SYM_BULK];
+    __shared__ int oc[SYM_WARPS][SYM_BULK];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int *fc = reinterpret_cast<int *>(sw_smem) + w * KP;
-    float *fv = reinterpret_cast<float *>(sw_smem + SYM_WARPS * KP * 4) + w * KP;
-    int *rk = reinterpret_cast<int *>(sw_smem + SYM_WARPS * KP * 8) + w * SORT_ROW_CAP;
-    float *rv = reinterpret_cast<float *>(sw_smem + SYM_WARPS * (KP * 8 + SORT_ROW_CAP * 4)) + w * SORT_ROW_CAP;
     const int64_t r = (int64_t)blockIdx.x * SYM_WARPS + w;
-    if (r >= N) return;
-    const int64_t b0 = roff[r], m = roff[r + 1] - b0;
-    if (m > SORT_ROW_CAP) {  // sorted in global memory first, written by sym_write_long_kernel
-        if (lane == 0) long_rows[atomicAdd(n_long, 1)] = (int)r;
+    if (r >= s.N) return;
+    const int64_t m64 = s.roff[r + 1] - s.roff[r];
+    if (m64 + s.k > SYM_BULK) {
+        if (lane == 0) {
+            if (m64 + s.k > SYM_MID) hub_rows[atomicAdd(n_list + 1, 1)] = (int)r;
+            else mid_rows[atomicAdd(n_list, 1)] = (int)r;
+        }
         return;
     }
-    const int a = own[r];
-    for (int t = lane; t < a; t += 32) {
-        fc[t] = scol[r * k + t];
-        fv[t] = sval[r * k + t];
-    }
-    int n = 32;
-    while (n < m) n <<= 1;
-    for (int t = lane; t < n; t += 32) {
-        rk[t] = t < m ? rev_i[b0 + t] : INT_MAX;
-        rv[t] = t < m ? rev_p[b0 + t] : 0.f;
-    }
-    __syncwarp();
-    if (m > 1) warp_bitonic_sort_smem(rk, rv, n, lane);
-    sym_write_row(fc, fv, a, rk, rv, m, inv2n, col, val, row_ptr[r], lane);
+    const int m = (int)m64, n = m + s.k;
+    if (n <= 64) sym_merge_row<2, K>(s, r, m, v[w], oc[w], ov[w], lane);
+    else if (n <= 128) sym_merge_row<4, K>(s, r, m, v[w], oc[w], ov[w], lane);
+    else if (n <= 256) sym_merge_row<8, K>(s, r, m, v[w], oc[w], ov[w], lane);
+    else sym_merge_row<16, K>(s, r, m, v[w], oc[w], ov[w], lane);
 }
 
-// One CTA per long reverse list, sorted in place in global memory by the
-// bitonic network in its "flip" form: every merge starts by comparing
-// mirrored positions and continues with half-cleaners, and every
-// compare-exchange puts the smaller element at the lower position. Positions
-// past the list's end act as +inf and never move, so exchanges with them are
-// skipped.
-__device__ __forceinline__ void ce_ascending(int32_t *key, float *val, int64_t a, int64_t c) {
-    const int ka = key[a], kc = key[c];
-    if (kc < ka) {
-        key[a] = kc;
-        key[c] = ka;
-        const float va = val[a];
-        val[a] = val[c];
-        val[c] = va;
+template <typename K>
+__global__ void __launch_bounds__(SYM_WARPS * 32)
+sym_mid_kernel(SymRow s, const int32_t *__restrict__ mid_rows, const int32_t *__restrict__ n_list) {
+    __shared__ float v[SYM_WARPS][SYM_MID], ov[SYM_WARPS][SYM_MID];
+    __shared__ int oc[SYM_WARPS][SYM_MID];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int q = blockIdx.x * SYM_WARPS + w; q < n_list[0]; q += gridDim.x * SYM_WARPS) {
+        const int64_t r = mid_rows[q];
+        sym_merge_row<32, K>(s, r, (int)(s.roff[r + 1] - s.roff[r]), v[w], oc[w], ov[w], lane);
+        __syncwarp();
     }
 }
 
-__global__ void __launch_bounds__(1024)
-sym_sort_long_kernel(const int64_t *__restrict__ roff, const int32_t *__restrict__ long_rows,
-                     const int32_t *__restrict__ n_long, int32_t *__restrict__ rev_i, float *__restrict__ rev_p) {
-    const int count = *n_long;
-    for (int q = blockIdx.x; q < count; q += gridDim.x) {
-        const int64_t r = long_rows[q];
-        const int64_t b = roff[r];
-        const int64_t len = roff[r + 1] - b;
-        int64_t n = 1;
-        while (n < len) n <<= 1;
-        for (int64_t size = 2; size <= n; size <<= 1) {
-            const int64_t half = size >> 1;
-            for (int64_t t = threadIdx.x; t < (n >> 1); t += blockDim.x) {
-                const int64_t blk = (t / half) * size, off = t % half;
-                const int64_t a = blk + off, c = blk + size - 1 - off;
-                if (c < len) ce_ascending(rev_i + b, rev_p + b, a, c);
+// Hub rows, one CTA each: a bitmap of the columns of the union gives every
+// entry its place (bits below it), HUB_COLS columns at a time. The reverse
+// entries are set first, so a forward entry that finds its bit set is mutual;
+// it adds its value to the one its partner has written.
+__global__ void __launch_bounds__(HUB_THREADS)
+sym_hub_kernel(SymRow s, const int32_t *__restrict__ hub_rows, const int32_t *__restrict__ n_list, int words) {
+    extern __shared__ uint32_t hub_smem[];
+    uint32_t *bits = hub_smem, *below = hub_smem + words;  // below: set bits before each word, in this range
+    __shared__ int wsum[HUB_THREADS / 32], wbase[HUB_THREADS / 32 + 1];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // words per warp, a multiple of 32
+    const int per = (words + HUB_THREADS - 1) / HUB_THREADS * 32;
+    for (int q = blockIdx.x; q < n_list[1]; q += gridDim.x) {
+        const int64_t r = hub_rows[q], b0 = s.roff[r], m = s.roff[r + 1] - b0, row = r * s.k;
+        int32_t *tc = s.tcol + row + b0;
+        float *tv = s.tval + row + b0;
+        int64_t done = 0;  // entries of the ranges before
+        for (int64_t c0 = 0; c0 < s.N; c0 += (int64_t)words * 32) {
+            const int64_t c1 = min(s.N, c0 + (int64_t)words * 32);
+            for (int t = tid; t < words; t += HUB_THREADS) bits[t] = 0u;
+            __syncthreads();
+            for (int64_t t = tid; t < m; t += HUB_THREADS) {
+                const int64_t c = s.rev[b0 + t].x;
+                if (c >= c0 && c < c1) atomicOr(&bits[(c - c0) >> 5], 1u << ((c - c0) & 31));
             }
             __syncthreads();
-            for (int64_t stride = half >> 1; stride > 0; stride >>= 1) {
-                for (int64_t t = threadIdx.x; t < (n >> 1); t += blockDim.x) {
-                    const int64_t a = 2 * t - (t & (stride - 1));
-                    const int64_t c = a + stride;
-                    if (c < len) ce_ascending(rev_i + b, rev_p + b, a, c);
+            // at most one forward entry per thread (k <= SYM_MAX_K)
+            int64_t fc = -1;
+            bool mutual = false;
+            if (tid < s.k) {
+                const int j = s.idx[row + tid];
+                if (j >= c0 && j < c1 && j != r) {
+                    fc = j;
+                    mutual = (bits[(fc - c0) >> 5] >> ((fc - c0) & 31)) & 1u;
                 }
-                __syncthreads();
             }
+            __syncthreads();
+            if (fc >= 0 && !mutual) {
+                const uint32_t bit = 1u << ((fc - c0) & 31);
+                if (atomicOr(&bits[(fc - c0) >> 5], bit) & bit) raise_status(s.status, DEV_MALFORMED);  // listed twice
+            }
+            __syncthreads();
+            // a warp's stretch of words: each word's set bits before it in the
+            // stretch, then the stretches' totals
+            int run = 0;
+            for (int t = warp * per + lane; t < (warp + 1) * per; t += 32) {
+                const int n = t < words ? __popc(bits[t]) : 0;
+                int incl = n;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int x = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += x;
+                }
+                if (t < words) below[t] = (uint32_t)(run + incl - n);
+                run += __shfl_sync(0xffffffffu, incl, 31);
+            }
+            if (lane == 0) wsum[warp] = run;
+            __syncthreads();
+            if (warp == 0) {
+                const int x = lane < HUB_THREADS / 32 ? wsum[lane] : 0;
+                int incl = x;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += y;
+                }
+                if (lane < HUB_THREADS / 32) wbase[lane] = incl - x;
+                if (lane == 31) wbase[HUB_THREADS / 32] = incl;
+            }
+            __syncthreads();
+            auto place = [&](int64_t c) {
+                const int o = (int)(c - c0), u = o >> 5;
+                return done + wbase[u / per] + below[u] + __popc(bits[u] & ((1u << (o & 31)) - 1u));
+            };
+            for (int64_t t = tid; t < m; t += HUB_THREADS) {
+                const int2 e = s.rev[b0 + t];
+                if (e.x >= c0 && e.x < c1) {
+                    const int64_t at = place(e.x);
+                    tc[at] = e.x;
+                    tv[at] = __int_as_float(e.y);
+                }
+            }
+            __syncthreads();
+            if (fc >= 0) {
+                const int64_t at = place(fc);
+                const float p = s.P[row + tid];
+                tc[at] = (int)fc;
+                tv[at] = mutual ? p + tv[at] : p;
+            }
+            done += wbase[HUB_THREADS / 32];
+            __syncthreads();
         }
+        if (tid == 0) s.len[r] = (int)done;
     }
 }
 
-// The long rows, their reverse lists sorted in global memory.
-template <int KP>
-__global__ void __launch_bounds__(SYM_WARPS * 32)
-sym_write_long_kernel(const int32_t *__restrict__ scol, const float *__restrict__ sval,
-                      const int32_t *__restrict__ own, int k, float inv2n, const int64_t *__restrict__ roff,
-                      const int32_t *__restrict__ rev_i, const float *__restrict__ rev_p,
-                      const int64_t *__restrict__ row_ptr, int32_t *__restrict__ col, float *__restrict__ val,
-                      const int32_t *__restrict__ long_rows, const int32_t *__restrict__ n_long) {
-    __shared__ int fc[SYM_WARPS][KP];
-    __shared__ float fv[SYM_WARPS][KP];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int count = *n_long;
-    for (int q = blockIdx.x * SYM_WARPS + w; q < count; q += gridDim.x * SYM_WARPS) {
-        const int64_t r = long_rows[q];
-        const int a = own[r];
-        for (int t = lane; t < a; t += 32) {
-            fc[w][t] = scol[r * k + t];
-            fv[w][t] = sval[r * k + t];
-        }
-        __syncwarp();
-        const int64_t b0 = roff[r];
-        sym_write_row(fc[w], fv[w], a, rev_i + b0, rev_p + b0, roff[r + 1] - b0, inv2n, col, val, row_ptr[r],
-                      lane);
-        __syncwarp();
+__global__ void __launch_bounds__(256)
+sym_copy_kernel(const int32_t *__restrict__ tcol, const float *__restrict__ tval, int64_t N, int k, float inv2n,
+                const int64_t *__restrict__ roff, const int64_t *__restrict__ row_ptr, int32_t *__restrict__ col,
+                float *__restrict__ val) {
+    const int lane = threadIdx.x & 31;
+    const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (r >= N) return;
+    const int64_t from = r * k + roff[r], to = row_ptr[r], n = row_ptr[r + 1] - to;
+    for (int64_t t = lane; t < n; t += 32) {
+        col[to + t] = tcol[from + t];
+        val[to + t] = tval[from + t] * inv2n;
     }
 }
 
-template <int KP>
-size_t sym_write_smem() {
-    return (size_t)SYM_WARPS * (KP * 8 + SORT_ROW_CAP * 8);
-}
-
-template <int KP>
+template <typename K>
 atsne_status symmetrize_t(const int32_t *idx, const float *P, int64_t N, int k, int64_t *row_ptr, int32_t *col,
                           float *val, int64_t *nnz_dev, const SymWs &w, cudaStream_t stream) {
     int *status = device_status_word();
     cudaError_t e = cudaMemsetAsync(w.rcnt, 0, sizeof(int32_t) * N, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(w.cursor, 0, sizeof(int32_t) * N, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(w.n_long, 0, sizeof(int32_t), stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w.n_list, 0, 2 * sizeof(int32_t), stream);
     if (e != cudaSuccess) return cuda_error(e, "symmetrize memset");
-    const int64_t M = N * k;
     const float inv2n = (float)(0.5 / (double)N);
-    ATSNE_TRY(launch_kernel("sym_fwd", sym_fwd_kernel<KP>, ceil_div(N, 4), 128, 0, stream, idx, P, N, k, w.scol,
-                            w.sval, w.own, w.rcnt, status));
+    const int row_blocks = ceil_div(N * 32, 256);
+    ATSNE_TRY(launch_kernel("sym_count", sym_count_kernel, row_blocks, 256, 0, stream, idx, N, k, w.rank, w.rcnt,
+                            status));
     ATSNE_TRY(scan_rowlen(w.rcnt, N, 0, w.roff, w.rtot, w.scan, stream));
-    ATSNE_TRY(launch_kernel("sym_rev", sym_rev_kernel, ceil_div(M, 256), 256, 0, stream,
-                            (const int32_t *)w.scol, (const float *)w.sval, N, k, (const int64_t *)w.roff, w.cursor,
-                            w.rev_i, w.rev_p));
-    ATSNE_TRY(launch_kernel("sym_len", sym_len_kernel<KP>, ceil_div(N, SYM_WARPS), SYM_WARPS * 32, 0, stream,
-                            (const int32_t *)w.scol, (const int32_t *)w.own, N, k, (const int64_t *)w.roff,
-                            (const int32_t *)w.rev_i, w.len));
+    ATSNE_TRY(launch_kernel("sym_place", sym_place_kernel, row_blocks, 256, 0, stream, idx, P, N, k,
+                            (const int32_t *)w.rank, (const int64_t *)w.roff, w.rev));
+    const SymRow s{idx, P, N, k, w.roff, w.rev, w.tcol, w.tval, w.len, status};
+    ATSNE_TRY(launch_kernel("sym_merge", sym_merge_kernel<K>, ceil_div(N, SYM_WARPS), SYM_WARPS * 32, 0, stream, s,
+                            w.mid_rows, w.hub_rows, w.n_list));
+    ATSNE_TRY(launch_kernel("sym_mid", sym_mid_kernel<K>, (int)hmin(4 * num_sms(), ceil_div(N, SYM_WARPS)),
+                            SYM_WARPS * 32, 0, stream, s, (const int32_t *)w.mid_rows, (const int32_t *)w.n_list));
+    const int words = (int)((hmin(N, HUB_COLS) + 31) / 32);
+    const size_t smem = (size_t)words * 8;
+    e = cudaFuncSetAttribute(sym_hub_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return cuda_error(e, "sym_hub attribute");
+    ATSNE_TRY(launch_kernel("sym_hub", sym_hub_kernel, (int)hmin(4 * num_sms(), N), HUB_THREADS, smem, stream, s,
+                            (const int32_t *)w.hub_rows, (const int32_t *)w.n_list, words));
     ATSNE_TRY(scan_rowlen(w.len, N, 0, row_ptr, nnz_dev, w.scan, stream));
-    const size_t smem = sym_write_smem<KP>();
-    e = cudaFuncSetAttribute(sym_write_kernel<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cuda_error(e, "sym_write attribute");
-    ATSNE_TRY(launch_kernel("sym_write", sym_write_kernel<KP>, ceil_div(N, SYM_WARPS), SYM_WARPS * 32, smem, stream,
-                            (const int32_t *)w.scol, (const float *)w.sval, (const int32_t *)w.own, N, k, inv2n,
-                            (const int64_t *)w.roff, (const int32_t *)w.rev_i, (const float *)w.rev_p,
-                            (const int64_t *)row_ptr, col, val, w.long_rows, w.n_long));
-    ATSNE_TRY(launch_kernel("sym_sort_long", sym_sort_long_kernel, 2 * num_sms(), 1024, 0, stream,
-                            (const int64_t *)w.roff, (const int32_t *)w.long_rows, (const int32_t *)w.n_long,
-                            w.rev_i, w.rev_p));
-    return launch_kernel("sym_write_long", sym_write_long_kernel<KP>, 2 * num_sms(), SYM_WARPS * 32, 0, stream,
-                         (const int32_t *)w.scol, (const float *)w.sval, (const int32_t *)w.own, k, inv2n,
-                         (const int64_t *)w.roff, (const int32_t *)w.rev_i, (const float *)w.rev_p,
-                         (const int64_t *)row_ptr, col, val, (const int32_t *)w.long_rows,
-                         (const int32_t *)w.n_long);
+    return launch_kernel("sym_copy", sym_copy_kernel, row_blocks, 256, 0, stream, (const int32_t *)w.tcol,
+                         (const float *)w.tval, N, k, inv2n, (const int64_t *)w.roff, (const int64_t *)row_ptr, col, val);
 }
 
 }  // namespace
 
 size_t symmetrize_workspace(Carver &c, int64_t N, int k, SymWs *ws) {
     SymWs w;
-    w.scol = c.take<int32_t>((size_t)N * k);
-    w.sval = c.take<float>((size_t)N * k);
-    w.rev_i = c.take<int32_t>((size_t)N * k);
-    w.rev_p = c.take<float>((size_t)N * k);
+    w.rev = c.take<int2>((size_t)N * k);
+    w.tcol = c.take<int32_t>((size_t)2 * N * k);
+    w.rank = w.tcol;  // read by the placement, before the merge writes
+    w.tval = c.take<float>((size_t)2 * N * k);
     w.rcnt = c.take<int32_t>((size_t)N);
-    w.cursor = c.take<int32_t>((size_t)N);
     w.len = c.take<int32_t>((size_t)N);
     w.roff = c.take<int64_t>((size_t)N + 1);
     w.rtot = c.take<int64_t>(1);
-    w.long_rows = c.take<int32_t>((size_t)N);
-    w.n_long = c.take<int32_t>(1);
-    w.own = c.take<int32_t>((size_t)N);
+    w.mid_rows = c.take<int32_t>((size_t)N);
+    w.hub_rows = c.take<int32_t>((size_t)N);
+    w.n_list = c.take<int32_t>(2);
     w.scan = c.take<int64_t>(scan_partials_count(N));
     if (ws) *ws = w;
     return c.bytes();
@@ -360,10 +415,9 @@ size_t symmetrize_workspace(Carver &c, int64_t N, int k, SymWs *ws) {
 atsne_status symmetrize_launch(const int32_t *idx, const float *P, int64_t N, int k,
                                int64_t *row_ptr, int32_t *col, float *val, int64_t *nnz_dev,
                                const SymWs &w, cudaStream_t stream) {
-    if (k <= 128) return symmetrize_t<128>(idx, P, N, k, row_ptr, col, val, nnz_dev, w, stream);
-    if (k <= 256) return symmetrize_t<256>(idx, P, N, k, row_ptr, col, val, nnz_dev, w, stream);
-    if (k <= 512) return symmetrize_t<512>(idx, P, N, k, row_ptr, col, val, nnz_dev, w, stream);
-    return set_error(ATSNE_EUNSUPPORTED, "symmetrize: k=%d above 512", k);
+    if (k > SYM_MAX_K) return set_error(ATSNE_EUNSUPPORTED, "symmetrize: k=%d above %d", k, SYM_MAX_K);
+    if (N <= SYM_KEY32) return symmetrize_t<uint32_t>(idx, P, N, k, row_ptr, col, val, nnz_dev, w, stream);
+    return symmetrize_t<unsigned long long>(idx, P, N, k, row_ptr, col, val, nnz_dev, w, stream);
 }
 
 }  // namespace atsne
