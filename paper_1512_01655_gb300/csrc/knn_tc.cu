@@ -303,13 +303,12 @@ __device__ uint32_t warp_select(Get get, int count, int kth, uint32_t *hist, int
 // ---------------------------------------------------------------------------
 // prep: BF16 hi/lo copies, norms, error norms
 // ---------------------------------------------------------------------------
-// One warp per row and step, four consecutive values per lane (16-byte loads
-// where every row starts on 16 bytes, 8-byte stores); the corpus maxima leave a
-// warp once, at its end. Bound by the rows read and the copies written: with
-// scalar loads and three atomics per row 70,000 x 784 took 183 us for the
-// three-pass copies, 113 us now (453 MB), 1,000,000 x 128 one pass 2,270 and
-// 282 us (800 MB), 200,000 x 128 three passes 401 and 69 us.
-template <bool VEC>
+// One warp per row and step, four loads in flight per lane; the corpus maxima
+// leave a warp once, at its end (three atomics per row to one address were the
+// bound: 1,000,000 x 128 one pass 2,270 us, 292 now (800 MB);
+// 200,000 x 128 three passes 401 and 71 us; 70,000 x 784 183 and
+// 120 us (453 MB)). A lane sums the values lane, lane + 32, ... in that
+// order: the norms are part of the keys.
 __global__ void __launch_bounds__(256)
 knn_prep_kernel(const float *__restrict__ X, const int32_t *__restrict__ rows, int64_t nrows, int64_t N,
                 int D, int Dp, int passes, __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo,
@@ -333,38 +332,30 @@ knn_prep_kernel(const float *__restrict__ X, const int32_t *__restrict__ rows, i
         if (src < 0 || src >= N) src = 0;  // flagged by the caller's index check
         const float *x = X + src * D;
         float n = 0.f, res = 0.f, l2 = 0.f;
-#pragma unroll 2
-        for (int d = 4 * lane; d < Dp; d += 128) {
+        for (int d0 = lane; d0 < Dp; d0 += 128) {
             float v[4];
-            if (VEC) {
-                const float4 f = d < D ? __ldg(reinterpret_cast<const float4 *>(x + d)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                v[0] = f.x;
-                v[1] = f.y;
-                v[2] = f.z;
-                v[3] = f.w;
-            } else {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) v[i] = d + i < D ? x[d + i] : 0.f;
-            }
-            __nv_bfloat16 h[4], l[4];
+            for (int i = 0; i < 4; ++i) v[i] = d0 + 32 * i < D ? __ldg(x + d0 + 32 * i) : 0.f;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
+                const int d = d0 + 32 * i;
+                if (d >= Dp) continue;
                 finite &= isfinite(v[i]);
-                h[i] = __float2bfloat16_rn(v[i]);
-                const float r1 = v[i] - __bfloat162float(h[i]);
+                const __nv_bfloat16 h = __float2bfloat16_rn(v[i]);
+                const float r1 = v[i] - __bfloat162float(h);
+                hi[r * Dp + d] = h;
                 n = fmaf(v[i], v[i], n);
                 if (passes == 3) {
-                    l[i] = __float2bfloat16_rn(r1);
-                    const float lf = __bfloat162float(l[i]);
+                    const __nv_bfloat16 l = __float2bfloat16_rn(r1);
+                    const float lf = __bfloat162float(l);
                     const float r2 = r1 - lf;
+                    lo[r * Dp + d] = l;
                     res = fmaf(r2, r2, res);
                     l2 = fmaf(lf, lf, l2);
                 } else {
                     res = fmaf(r1, r1, res);
                 }
             }
-            *reinterpret_cast<uint2 *>(hi + r * Dp + d) = *reinterpret_cast<uint2 *>(h);
-            if (passes == 3) *reinterpret_cast<uint2 *>(lo + r * Dp + d) = *reinterpret_cast<uint2 *>(l);
         }
         n = warp_sum(n);
         res = warp_sum(res);
@@ -1973,10 +1964,8 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
         // ordered rows and columns: the copies, norms and statistics in the order
         if (ordered) ATSNE_TRY(knn_order_launch(X, N, D, pl, TC_BM, TC_BN, w.ord, stream));
         const int64_t prows = w.bext ? (N + TC_BN - 1) / TC_BN * TC_BN : N;  // the norm slices fill whole tiles
-        const auto prep = (D & 3) == 0 && ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Xq)) & 15) == 0
-                              ? knn_prep_kernel<true> : knn_prep_kernel<false>;
         const int64_t most = 8 * num_sms();
-        ATSNE_TRY(launch_kernel("knn_prep", prep, (int)hmin(most, ceil_div(prows * 32, 256)), 256, 0, stream, X,
+        ATSNE_TRY(launch_kernel("knn_prep", knn_prep_kernel, (int)hmin(most, ceil_div(prows * 32, 256)), 256, 0, stream, X,
                                 ordered ? (const int32_t *)w.ord.perm : (const int32_t *)nullptr, N, N, D,
                                 pl.Dp, pl.passes, hi, lo, w.nrm,
                                 reinterpret_cast<float4 *>(w.stats), w.gmax,
@@ -1984,7 +1973,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
                                 reinterpret_cast<__nv_bfloat16 *>(pl.passes == 1 ? w.aext : nullptr), status,
                                 (const int64_t *)nullptr));
         if (Xq) {
-            ATSNE_TRY(launch_kernel("knn_prep", prep, (int)hmin(most, ceil_div(Q * 32, 256)), 256, 0, stream, Xq,
+            ATSNE_TRY(launch_kernel("knn_prep", knn_prep_kernel, (int)hmin(most, ceil_div(Q * 32, 256)), 256, 0, stream, Xq,
                                     (const int32_t *)nullptr, Q, Q, D, pl.Dp, pl.passes,
                                     reinterpret_cast<__nv_bfloat16 *>(w.qhi),
                                     reinterpret_cast<__nv_bfloat16 *>(w.qlo), w.qnrm,
@@ -1994,7 +1983,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
             a_hi = w.qhi;
             a_lo = w.qlo;
         } else if (qlist) {
-            ATSNE_TRY(launch_kernel("knn_prep", prep, (int)hmin(most, ceil_div(Q * 32, 256)), 256, 0, stream, X,
+            ATSNE_TRY(launch_kernel("knn_prep", knn_prep_kernel, (int)hmin(most, ceil_div(Q * 32, 256)), 256, 0, stream, X,
                                     qlist, Q, N, D, pl.Dp, pl.passes,
                                     reinterpret_cast<__nv_bfloat16 *>(w.qhi),
                                     reinterpret_cast<__nv_bfloat16 *>(w.qlo), (float *)nullptr,
