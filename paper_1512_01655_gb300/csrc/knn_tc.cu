@@ -71,6 +71,7 @@ constexpr int TC_BN = 256;       // corpus points per tile (TMEM columns per acc
 constexpr int TC_BK = 64;        // BF16 per k-block (one 128-byte swizzle row)
 constexpr uint64_t WAIT_NS = 1000000000ull;
 constexpr int MERGE_WARPS = 4;
+constexpr int MERGE_ONE_ROWS = 4;   // rows per SM up to which a block merges one row
 constexpr int RCAP = 256;        // candidates re-ranked per row at most (certified modes)
 constexpr int MSTAGE = 1024;     // keys below tau staged per row for the merge's select
 constexpr int RCAP_FP8 = 1024;   // modes without a certificate: the largest re-rank set (ksel <= 512)
@@ -1125,25 +1126,32 @@ __device__ __forceinline__ float row_error_bound(const MergeParams &p, float4 st
 // set, so the re-rank set takes their place (p.rc <= p.mst) and five blocks
 // fit on an SM instead of four.
 constexpr int merge_reg_keys(bool cert) { return 32 * (cert ? 24 : 36); }
-size_t merge_smem_bytes(bool cert, int rc, int mst) {
-    return (size_t)MERGE_WARPS * (256 * 4 + (size_t)mst * 8 + (cert ? (size_t)rc * 8 : 0) + TIE_MAX * 12);
+size_t merge_smem_bytes(bool cert, int rc, int mst, int rows) {
+    return (size_t)rows * (256 * 4 + (size_t)mst * 8 + (cert ? (size_t)rc * 8 : 0) + TIE_MAX * 12);
 }
 
-template <bool CERT>
+// ROWS rows per block: one warp each (MERGE_WARPS), or one row (1), whose
+// re-rank the block's other warps share. With few rows a row's own latency is
+// what counts, most of it the re-rank's gathers, a few in flight at a time (500
+// rows of 784 dimensions: 152 us with a warp per row, 102 us; of 50: 45 and 41
+// us; 2,000 rows of 784 191 and 221 us: their warps fill the SMs by themselves).
+template <bool CERT, int ROWS>
 __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kernel(MergeParams p) {
     extern __shared__ __align__(16) unsigned char mg_smem[];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, w = ROWS == 1 ? 0 : warp;
+    __shared__ const int *job_rj;
+    __shared__ int job[4];  // ROWS = 1: the re-rank the warps share: from, to, the query's row (low, high)
     uint32_t *hist = reinterpret_cast<uint32_t *>(mg_smem) + w * 256;
     const int MST = p.mst, RC = p.rc;
     const int RCS = CERT ? RC : 0;  // the re-rank set's own region (else it is the staging region)
     // MST keys, then MST indices of this warp
-    float *sk0 = reinterpret_cast<float *>(mg_smem + MERGE_WARPS * 1024) + w * 2 * MST;
+    float *sk0 = reinterpret_cast<float *>(mg_smem + ROWS * 1024) + w * 2 * MST;
     float *sk = sk0;
     int *sjg = reinterpret_cast<int *>(sk0) + MST;
-    float *rdw = CERT ? reinterpret_cast<float *>(mg_smem + MERGE_WARPS * (1024 + MST * 8)) + w * RC : sk;
-    int *rjg = CERT ? reinterpret_cast<int *>(mg_smem + MERGE_WARPS * (1024 + MST * 8 + RC * 4)) + w * RC : sjg;
-    double *dmw = reinterpret_cast<double *>(mg_smem + MERGE_WARPS * (1024 + MST * 8 + RCS * 8)) + w * TIE_MAX;
-    int *mpw = reinterpret_cast<int *>(mg_smem + MERGE_WARPS * (1024 + MST * 8 + RCS * 8 + TIE_MAX * 8)) +
+    float *rdw = CERT ? reinterpret_cast<float *>(mg_smem + ROWS * (1024 + MST * 8)) + w * RC : sk;
+    int *rjg = CERT ? reinterpret_cast<int *>(mg_smem + ROWS * (1024 + MST * 8 + RC * 4)) + w * RC : sjg;
+    double *dmw = reinterpret_cast<double *>(mg_smem + ROWS * (1024 + MST * 8 + RCS * 8)) + w * TIE_MAX;
+    int *mpw = reinterpret_cast<int *>(mg_smem + ROWS * (1024 + MST * 8 + RCS * 8 + TIE_MAX * 8)) +
                w * TIE_MAX;
     const int sel = CERT ? p.k : p.ksel;  // rank of the key that bounds the re-rank set
     const bool cross = p.Xq != nullptr;
@@ -1154,7 +1162,34 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
         Q = up.Q;
         S = up.splits * p.splits;  // splits of a row by buffers of a split
     }
-    for (int64_t row = (int64_t)blockIdx.x * MERGE_WARPS + w; row < Q; row += (int64_t)gridDim.x * MERGE_WARPS) {
+    // exact FP32 distances of rjw[from, to) in the library's one summation
+    // order (group8_d2_pair), eight candidates per warp step; part of parts
+    auto rerank_part = [&](const float *xq, const int *rjw, int from, int to, int part, int parts) {
+        const bool vec4 = (p.D & 3) == 0 && (reinterpret_cast<uintptr_t>(p.X) & 15) == 0 &&
+                          (reinterpret_cast<uintptr_t>(xq) & 15) == 0;
+        const int g = lane >> 3, gl = lane & 7;
+        for (int t0 = from + 8 * part; t0 < to; t0 += 8 * parts) {
+            const int ta = t0 + g, tb = t0 + 4 + g;
+            const float *xa = ta < to ? p.X + (int64_t)rjw[ta] * p.D : xq;
+            const float *xb = tb < to ? p.X + (int64_t)rjw[tb] * p.D : xq;
+            const float2 s2 = group8_d2_pair(xq, xa, xb, p.D, vec4, gl);
+            if (gl == 0) {
+                if (ta < to) rdw[ta] = s2.x;
+                if (tb < to) rdw[tb] = s2.y;
+            }
+        }
+    };
+    if (ROWS == 1 && warp > 0) {
+        for (;;) {
+            __syncthreads();
+            const int from = job[0], to = job[1];
+            if (to < 0) return;
+            rerank_part(reinterpret_cast<const float *>((uint64_t)(uint32_t)job[2] | (uint64_t)(uint32_t)job[3] << 32),
+                        job_rj, from, to, warp, MERGE_WARPS);
+            __syncthreads();
+        }
+    }
+    for (int64_t row = (int64_t)blockIdx.x * ROWS + w; row < Q; row += (int64_t)gridDim.x * ROWS) {
     __syncwarp();
     const int64_t r0 = p.rlist ? p.rlist[row] : row;  // the query row
     const int qid = cross ? (int)r0 : (p.qlist ? p.qlist[r0] : (int)r0);
@@ -1417,21 +1452,20 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
             __syncwarp();
         };
         const float *xq = cross ? p.Xq + r0 * p.D : p.X + (p.perm ? orow : (int64_t)qid) * p.D;
-        const bool vec4 = (p.D & 3) == 0 && (reinterpret_cast<uintptr_t>(p.X) & 15) == 0 &&
-                          (reinterpret_cast<uintptr_t>(xq) & 15) == 0;
-        // exact FP32 distances of rjw[from, to) in the library's one summation
-        // order (group8_d2_pair), eight candidates per warp step
         auto rerank = [&](int from, int to) {
-            const int g = lane >> 3, gl = lane & 7;
-            for (int t0 = from; t0 < to; t0 += 8) {
-                const int ta = t0 + g, tb = t0 + 4 + g;
-                const float *xa = ta < to ? p.X + (int64_t)rjw[ta] * p.D : xq;
-                const float *xb = tb < to ? p.X + (int64_t)rjw[tb] * p.D : xq;
-                const float2 s2 = group8_d2_pair(xq, xa, xb, p.D, vec4, gl);
-                if (gl == 0) {
-                    if (ta < to) rdw[ta] = s2.x;
-                    if (tb < to) rdw[tb] = s2.y;
+            if (ROWS == 1) {
+                if (lane == 0) {
+                    job[0] = from;
+                    job[1] = to;
+                    job[2] = (int)(uint32_t)reinterpret_cast<uint64_t>(xq);
+                    job[3] = (int)(uint32_t)(reinterpret_cast<uint64_t>(xq) >> 32);
                 }
+                if (lane == 0) job_rj = rjw;
+                __syncthreads();
+                rerank_part(xq, rjw, from, to, 0, MERGE_WARPS);
+                __syncthreads();
+            } else {
+                rerank_part(xq, rjw, from, to, 0, 1);
             }
         };
         collect(-INFINITY, theta);
@@ -1506,6 +1540,10 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
     } else if (lane == 0) {
         p.flag_rows[atomicAdd(p.flag_count, 1)] = (int)(p.flag_out ? orow : r0);
     }
+    }
+    if (ROWS == 1) {
+        if (lane == 0) job[1] = -1;
+        __syncthreads();
     }
 }
 
@@ -1905,8 +1943,8 @@ knn_gather_kernel(const int32_t *__restrict__ rows, const int32_t *__restrict__ 
     }
 }
 
-// The merge of a launch's buffers over `grid` blocks.
-static atsne_status merge_launch(const TcPlan &pl, MergeParams m, int grid, cudaStream_t stream) {
+// The merge of a launch's buffers.
+static atsne_status merge_launch(const TcPlan &pl, MergeParams m, cudaStream_t stream) {
     if (!pl.certify) {
         // the re-rank set is the ksel best keys (ties included); the staged
         // keys are those below the lowest tau, about twice as many
@@ -1919,8 +1957,13 @@ static atsne_status merge_launch(const TcPlan &pl, MergeParams m, int grid, cuda
         m.mst = MSTAGE;
     }
     static_assert(2 * MSTAGE >= merge_reg_keys(true), "indices of keys in registers");
-    const size_t ms = merge_smem_bytes(pl.certify, m.rc, m.mst);
-    void (*kern)(MergeParams) = pl.certify ? knn_merge_kernel<true> : knn_merge_kernel<false>;
+    // one row per block while the rows leave most of the SMs' warps idle, and for
+    // those given up by the fixed threshold, which are few
+    const bool one = m.rcount || m.Q <= MERGE_ONE_ROWS * num_sms();
+    const size_t ms = merge_smem_bytes(pl.certify, m.rc, m.mst, one ? 1 : MERGE_WARPS);
+    void (*kern)(MergeParams) = pl.certify ? (one ? knn_merge_kernel<true, 1> : knn_merge_kernel<true, MERGE_WARPS>)
+                                           : (one ? knn_merge_kernel<false, 1> : knn_merge_kernel<false, MERGE_WARPS>);
+    const int grid = m.rcount ? (int)hmin(4 * num_sms(), m.Q) : ceil_div(m.Q, one ? 1 : MERGE_WARPS);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ms);
     if (e != cudaSuccess) return cuda_error(e, "knn_tc_merge attribute");
     return launch_kernel("knn_tc_merge", kern, grid, MERGE_WARPS * 32, ms, stream, m);
@@ -2053,7 +2096,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
             return launch_kernel("radius_filter", radius_filter_kernel, ceil_div(Q * k, 256), 256, 0, stream,
                                  idx_out, d2_out, Q, k, radius);
         }
-        ATSNE_TRY(merge_launch(pl, m, ceil_div(Q, MERGE_WARPS), stream));
+        ATSNE_TRY(merge_launch(pl, m, stream));
         ATSNE_TRY(launch_kernel("knn_gather", knn_gather_kernel, (int)hmin(4 * num_sms(), ceil_div(Q * 32, 256)), 256,
                                 0, stream, (const int32_t *)w.retry_rows, (const int32_t *)(w.flag_count + 1), pl.Dp,
                                 reinterpret_cast<const uint16_t *>(a_hi), reinterpret_cast<const uint16_t *>(a_lo),
@@ -2142,9 +2185,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
     m.flag_out = true;
     m.flag_rows = w.flag_rows;
     m.flag_count = w.flag_count;
-    ATSNE_TRY(merge_launch(pl, m,
-                           retry ? (int)hmin(4 * num_sms(), ceil_div(Q, MERGE_WARPS)) : ceil_div(Q, MERGE_WARPS),
-                           stream));
+    ATSNE_TRY(merge_launch(pl, m, stream));
     return knn_bruteforce_rows(X, N, D, qlist, w.flag_rows, w.flag_count, Q, k, idx_out, d2_out, stream,
                                Xq);
 }
