@@ -30,7 +30,7 @@ struct TcPlan {
     // fixed thresholds (knn_filter.cu); the fields above then describe the
     // adaptive launch over the rows it gives up
     bool filter = false;
-    int S = 0, blk = 0, rank = 0;                // sampled rows, columns per block, the threshold's rank
+    int S = 0, blk = 0, rank = 0, rank2 = 0;     // sampled rows, columns per block, the thresholds' ranks
     int fsplits = 1, fcols = 0, fcap = 0;
 };
 // Row and column order of a large self kNN (points grouped by nearest

@@ -492,6 +492,45 @@ knn_sample_kernel(const uint16_t *__restrict__ hi, const float *__restrict__ nrm
     if (lane < 16) sext[(int64_t)i * 16 + lane] = norm_piece(nrm[src], lane);
 }
 
+// The rank-th largest of a row's m block values (m <= 1024), by bisection on
+// the values' order-preserving bits, counting the values held in registers.
+// Whole warp.
+__device__ __forceinline__ float rank_largest(const float *mr, int m, int rank, int lane) {
+    const int per = (m + 31) / 32;
+    uint32_t u[32];
+#pragma unroll
+    for (int t = 0; t < 32; ++t) {
+        u[t] = 0u;
+        if (t < per && t * 32 + lane < m) u[t] = float_key(mr[t * 32 + lane]);
+    }
+    // the largest threshold with at least `rank` values at or above it, or
+    // any that has exactly `rank` (a dozen counts instead of 32)
+    uint32_t lo = 0xffffffffu, hi = 0u;
+#pragma unroll
+    for (int t = 0; t < 32; ++t)
+        if (t < per) {
+            if (t * 32 + lane < m) lo = min(lo, u[t]);
+            hi = max(hi, u[t]);
+        }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    while (lo < hi) {
+        const uint32_t mid = hi - ((hi - lo) >> 1);
+        int c = 0;
+#pragma unroll
+        for (int t = 0; t < 32; ++t)
+            if (t < per) c += u[t] >= mid;
+        c = (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
+        if (c >= rank) {
+            lo = mid;
+            if (c == rank) break;
+        } else {
+            hi = mid - 1u;
+        }
+    }
+    return key_of_bits(lo);
+}
+
 struct TauParams {
     const float *minima;  // [Q][m], or nullptr (no sample)
     int m, rank;
@@ -516,40 +555,7 @@ __global__ void __launch_bounds__(128) knn_tau_kernel(TauParams p) {
     if (row >= Q) return;
     float tau = INFINITY;
     if (p.minima) {
-        const float *mr = p.minima + row * p.m;
-        const int per = (p.m + 31) / 32;
-        uint32_t u[32];
-#pragma unroll
-        for (int t = 0; t < 32; ++t) {
-            u[t] = 0u;
-            if (t < per && t * 32 + lane < p.m) u[t] = float_key(mr[t * 32 + lane]);
-        }
-        // the largest threshold with at least `rank` values at or above it, or
-        // any that has exactly `rank` (a dozen counts instead of 32)
-        uint32_t lo = 0xffffffffu, hi = 0u;
-#pragma unroll
-        for (int t = 0; t < 32; ++t)
-            if (t < per) {
-                if (t * 32 + lane < p.m) lo = min(lo, u[t]);
-                hi = max(hi, u[t]);
-            }
-        lo = __reduce_min_sync(0xffffffffu, lo);
-        hi = __reduce_max_sync(0xffffffffu, hi);
-        while (lo < hi) {
-            const uint32_t mid = hi - ((hi - lo) >> 1);
-            int c = 0;
-#pragma unroll
-            for (int t = 0; t < 32; ++t)
-                if (t < per) c += u[t] >= mid;
-            c = (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
-            if (c >= p.rank) {
-                lo = mid;
-                if (c == p.rank) break;
-            } else {
-                hi = mid - 1u;
-            }
-        }
-        const float v = key_of_bits(lo);
+        const float v = rank_largest(p.minima + row * p.m, p.m, p.rank, lane);
         if (isfinite(v)) tau = -2.f * v;
     }
     if (p.bound) {
@@ -570,6 +576,28 @@ __global__ void __launch_bounds__(128) knn_tau_kernel(TauParams p) {
         }
     }
     if (lane == 0) p.tau[row] = tau;
+}
+
+// Starting thresholds of the rows given up for too few keys (marked +inf), one
+// warp per row, in the modes without a certificate: the adaptive kernel tightens
+// a threshold only as it meets nearer keys, and from +inf its first tiles
+// overflow the buffers of a row whose columns are split over many units. Merge
+// and adaptive launch of a list of rows, started from +inf and from here: 7,000
+// rows of 100,000 x 50 (lognormal) 4.87 and 0.28 ms, 500 rows of 70,000 x 784
+// (bytes) 1.47 and 0.38 ms, 20,000 rows of 200,000 x 128 865 and 663 us. A row
+// that failed the certificate stays at +inf: it needs keys past the k-th by
+// twice their error bound, and starting there cost more where nearly all keys
+// lie that close (3,000 equal rows, FP32: 0.12 and 1.2 ms).
+__global__ void __launch_bounds__(128)
+knn_retry_tau_kernel(const float *__restrict__ minima, int m, int rank, const int32_t *__restrict__ rows,
+                     const int32_t *__restrict__ count, float *__restrict__ tau) {
+    const int lane = threadIdx.x & 31, n = *count;
+    for (int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); i < n; i += (int)(gridDim.x * blockDim.x) >> 5) {
+        const int64_t r = rows[i];
+        if (!isinf(tau[r])) continue;
+        const float v = rank_largest(minima + r * m, m, rank, lane);
+        if (lane == 0 && isfinite(v)) tau[r] = -2.f * v;
+    }
 }
 
 template <int PASSES>
@@ -680,6 +708,12 @@ atsne_status knn_filter_launch(const TcPlan &pl, const TcWs &w, const FilterArgs
     ATSNE_TRY(tc_map_ext(&p.tm_a_ext, w.aext, F_BM, F_BM));
     ATSNE_TRY(tc_map_ext(&p.tm_b_ext, w.bext, (a.N + F_BN - 1) / F_BN * F_BN, F_BH));
     return f_launch<1, false>(p, pairs * p.splits, stream);
+}
+
+atsne_status knn_retry_tau_launch(const TcPlan &pl, const TcWs &w, cudaStream_t stream) {
+    return launch_kernel("knn_retry_tau", knn_retry_tau_kernel, 2 * num_sms(), 128, 0, stream, (const float *)w.minima,
+                         pl.S / pl.blk, pl.rank2, (const int32_t *)w.retry_rows, (const int32_t *)(w.flag_count + 1),
+                         w.tau);
 }
 
 }  // namespace atsne

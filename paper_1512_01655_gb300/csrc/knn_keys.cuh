@@ -88,6 +88,9 @@ struct FilterArgs {
     const int64_t *qcount;
 };
 atsne_status knn_filter_launch(const TcPlan &pl, const TcWs &w, const FilterArgs &a, cudaStream_t stream);
+// Starting thresholds of the rows it gave up (TcWs::retry_rows, flag_count[1]):
+// those marked +inf in TcWs::tau get the plan's second rank, the others keep theirs.
+atsne_status knn_retry_tau_launch(const TcPlan &pl, const TcWs &w, cudaStream_t stream);
 // Tensor maps of BF16 rows: 64-column boxes of rows of Dp (128-byte swizzle),
 // and boxes of whole norm slices (rows of 16, 32-byte swizzle).
 atsne_status tc_map_bf16(CUtensorMap *m, const void *base, int64_t rows, int Dp, int box_rows);

@@ -80,6 +80,7 @@ constexpr int HSHIFT = 18;       // float bits >> HSHIFT: exponent and 5 mantiss
 constexpr int GH_BUCKETS = 48;   // a row's global histogram (column splits): 6 octaves, 8 per octave
 constexpr int GH_SHIFT = 20;
 constexpr int64_t FILTER_MIN_ROWS = 1024;       // a smaller corpus is not sampled
+constexpr int64_t RETRY_MAX_SPLITS = 128;       // a row's buffers then fit the merge's register path
 constexpr int64_t RETRY_SPLIT_ROWS = 32768;  // rows given up by the fixed threshold that may be split
 
 // PASSES: 1 = one BF16 pass, 3 = BF16 hi/lo in three passes, 8 = one FP8
@@ -164,6 +165,7 @@ struct TcParams {
     // the rows given up by the fixed-threshold kernel: row r of this launch is
     // query row rlist[r], *rcount rows in all, their splits from retry_plan
     const int32_t *rlist, *rcount;
+    const float *tau0;     // [Q] key thresholds those rows start from
     int64_t bufs;          // room for that many (row, split) buffers
     int64_t Q, N;
     int KB;                // Dp / 64
@@ -190,7 +192,8 @@ __device__ __forceinline__ UnitPlan retry_plan(int64_t count, int64_t N, int64_t
     const int64_t tiles = (N + TC_BN - 1) / TC_BN;
     int64_t s = 1;
     if (count > 0 && count <= RETRY_SPLIT_ROWS)
-        s = max((int64_t)1, min(min((tiles + 3) / 4, bufs / count), (int64_t)((304 + u.row_tiles - 1) / u.row_tiles)));
+        s = max((int64_t)1, min(min((tiles + 3) / 4, bufs / count),
+                                min((int64_t)((304 + u.row_tiles - 1) / u.row_tiles), RETRY_MAX_SPLITS)));
     u.cols_per_split = (int)((tiles + s - 1) / s * TC_BN);
     u.splits = (int)((N + u.cols_per_split - 1) / u.cols_per_split);
     return u;
@@ -744,6 +747,15 @@ __global__ void __launch_bounds__(TcCfg<PASSES>::THREADS, 1) knn_tc_kernel(const
                 }
             }
             bool rebased = p.hint && PASSES != 8;
+            if (p.tau0 && qv) {
+                const float t = p.tau0[r0];
+                if (isfinite(t)) {
+                    tau = fminf(tau, t);
+                    const int ht = dbucket((nx + t) * 1.0001f) + 1;
+                    if (ht < top) top = ht;
+                    rebased = true;
+                }
+            }
             // largest and smallest buffered keys, for the first re-anchoring of the grid
             float kmx = -INFINITY, kmn = INFINITY;
             uint32_t *dh = &s.dhist[e][0][lane];
@@ -1094,6 +1106,7 @@ struct MergeParams {
     const int64_t *qcount;  // if given, the rows in use (device; at most Q)
     int tag;                // of the launch that wrote the buffers
     bool flag_out;          // flag output rows (for the brute-force kernel), else query rows
+    float *tau_mark;        // set to +inf for a flagged row whose buffers did not overflow
     const float *X;
     int D, k, ksel;
     int rc, mst;            // re-rank set and staged keys per row (shared memory)
@@ -1539,6 +1552,7 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
         }
     } else if (lane == 0) {
         p.flag_rows[atomicAdd(p.flag_count, 1)] = (int)(p.flag_out ? orow : r0);
+        if (p.tau_mark && !ovf) p.tau_mark[r0] = INFINITY;
     }
     }
     if (ROWS == 1) {
@@ -1808,6 +1822,10 @@ static void plan_filter(TcPlan &pl, int64_t N, int64_t Q, int splits) {
     pl.S = S;
     pl.blk = blk;
     pl.rank = (int)fmax(1.0, floor(share(blk) * (S / blk) + 0.5));
+    // a row given up for too few keys starts again from a rank that leaves it
+    // short with a probability below 10^-9: r - 7 sqrt(r) = x
+    const double rt2 = 3.5 + sqrt(12.25 + x), f2 = fmin(0.9, rt2 * rt2 / S);
+    pl.rank2 = (int)fmin((double)(S / blk), floor((1.0 - pow(1.0 - f2, blk)) * (S / blk) + 1.0));
     if (splits <= 0) splits = filter_splits(pairs, col_tiles, 64);
     if (splits > 64) splits = 64;
     if (splits > col_tiles) splits = (int)col_tiles;
@@ -2088,6 +2106,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
         m.flag_out = !retry;
         m.flag_rows = retry ? w.retry_rows : w.flag_rows;
         m.flag_count = retry ? w.flag_count + 1 : w.flag_count;
+        m.tau_mark = retry ? w.tau : nullptr;
         if (radius) {
             ATSNE_TRY(launch_kernel("knn_tc_merge", radius_merge_kernel, ceil_div(Q, MERGE_WARPS),
                                     MERGE_WARPS * 32, 0, stream, m, radius));
@@ -2101,6 +2120,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
                                 0, stream, (const int32_t *)w.retry_rows, (const int32_t *)(w.flag_count + 1), pl.Dp,
                                 reinterpret_cast<const uint16_t *>(a_hi), reinterpret_cast<const uint16_t *>(a_lo),
                                 w.rhi, w.rlo));
+        if (!pl.certify) ATSNE_TRY(knn_retry_tau_launch(pl, w, stream));
         a_hi = w.rhi;
         a_lo = w.rlo;
     }
@@ -2135,6 +2155,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
     p.pro = ordered && !retry ? w.ord.pro : nullptr;
     p.rlist = retry ? w.retry_rows : nullptr;
     p.rcount = retry ? w.flag_count + 1 : nullptr;
+    p.tau0 = retry ? w.tau : nullptr;
     p.bufs = m.bufs;
     p.clock = w.clock;
     p.qst = reinterpret_cast<const float4 *>(w.qstats);
@@ -2183,6 +2204,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
     m.rcount = p.rcount;
     m.tag = retry ? META_RETRY : META_FIRST;
     m.flag_out = true;
+    m.tau_mark = nullptr;
     m.flag_rows = w.flag_rows;
     m.flag_count = w.flag_count;
     ATSNE_TRY(merge_launch(pl, m, stream));
