@@ -156,19 +156,88 @@ __device__ __forceinline__ float2 group8_d2_pair(const float *__restrict__ q, co
             df = qv.w - bv.w;
             sb = fmaf(df, df, sb);
         }
+    } else if ((D & 1) == 0 && ((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(xa) |
+                                 reinterpret_cast<uintptr_t>(xb)) & 7) == 0) {
+        // rows of an even number of values (50 dimensions are common): 8-byte
+        // loads, a chunk past D read as zeros, which leave the sums as they are
+        const float2 *q2 = reinterpret_cast<const float2 *>(q);
+        const float2 *a2 = reinterpret_cast<const float2 *>(xa);
+        const float2 *b2 = reinterpret_cast<const float2 *>(xb);
+        const float2 z = make_float2(0.f, 0.f);
+#pragma unroll 2
+        for (int j = gl; 4 * j < D; j += 8) {
+            const bool two = 4 * j + 2 < D;
+            const float2 qv = q2[2 * j], av = a2[2 * j], bv = b2[2 * j];
+            const float2 qw = two ? q2[2 * j + 1] : z, aw = two ? a2[2 * j + 1] : z, bw = two ? b2[2 * j + 1] : z;
+            float df = qv.x - av.x;
+            sa = fmaf(df, df, sa);
+            df = qv.y - av.y;
+            sa = fmaf(df, df, sa);
+            df = qw.x - aw.x;
+            sa = fmaf(df, df, sa);
+            df = qw.y - aw.y;
+            sa = fmaf(df, df, sa);
+            df = qv.x - bv.x;
+            sb = fmaf(df, df, sb);
+            df = qv.y - bv.y;
+            sb = fmaf(df, df, sb);
+            df = qw.x - bw.x;
+            sb = fmaf(df, df, sb);
+            df = qw.y - bw.y;
+            sb = fmaf(df, df, sb);
+        }
     } else {
         for (int j = gl; 4 * j < D; j += 8) {
+            float qv[4], av[4], bv[4];
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 const int e = 4 * j + c;
-                if (e < D) {
-                    float df = q[e] - xa[e];
-                    sa = fmaf(df, df, sa);
-                    df = q[e] - xb[e];
-                    sb = fmaf(df, df, sb);
-                }
+                qv[c] = e < D ? q[e] : 0.f;
+                av[c] = e < D ? xa[e] : 0.f;
+                bv[c] = e < D ? xb[e] : 0.f;
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                float df = qv[c] - av[c];
+                sa = fmaf(df, df, sa);
+                df = qv[c] - bv[c];
+                sb = fmaf(df, df, sb);
             }
         }
+    }
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        sa += __shfl_xor_sync(0xffffffffu, sa, o);
+        sb += __shfl_xor_sync(0xffffffffu, sb, o);
+    }
+    return make_float2(sa, sb);
+}
+
+// The same distances, bit for bit, to rows xa and xb given in BF16 (exact
+// copies, zeros past D, 8-byte aligned); D % 4 == 0 and q 16-byte aligned.
+__device__ __forceinline__ float2 group8_d2_pair_bf16(const float *__restrict__ q, const uint16_t *__restrict__ xa,
+                                                      const uint16_t *__restrict__ xb, int D, int gl) {
+    float sa = 0.f, sb = 0.f;
+    const int n4 = D >> 2;
+    const float4 *q4 = reinterpret_cast<const float4 *>(q);
+    const uint2 *a4 = reinterpret_cast<const uint2 *>(xa);
+    const uint2 *b4 = reinterpret_cast<const uint2 *>(xb);
+    auto add = [](float4 qv, uint2 h, float &s) {
+        float df = qv.x - __uint_as_float(h.x << 16);
+        s = fmaf(df, df, s);
+        df = qv.y - __uint_as_float(h.x & 0xffff0000u);
+        s = fmaf(df, df, s);
+        df = qv.z - __uint_as_float(h.y << 16);
+        s = fmaf(df, df, s);
+        df = qv.w - __uint_as_float(h.y & 0xffff0000u);
+        s = fmaf(df, df, s);
+    };
+#pragma unroll 4
+    for (int j = gl; j < n4; j += 8) {
+        const float4 qv = q4[j];
+        const uint2 av = a4[j], bv = b4[j];
+        add(qv, av, sa);
+        add(qv, bv, sb);
     }
 #pragma unroll
     for (int o = 1; o < 8; o <<= 1) {

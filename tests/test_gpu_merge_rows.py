@@ -54,3 +54,20 @@ def test_rows_given_up_start_from_the_wider_rank(at):
     at.atsne_check()
     ri, rd = oracle(X, q, 12)
     assert torch.equal(i, ri) and torch.equal(d, rd)
+
+
+@pytest.mark.parametrize("D", [2, 6, 48, 50, 51, 98, 785])
+@pytest.mark.parametrize("offset", [0, 1, 2])
+def test_row_widths_and_alignments(at, D, offset):
+    """Rows whose widths and first addresses admit 16-byte, 8-byte or 4-byte
+    loads, of values that the BF16 copies hold exactly or not."""
+    N, k = 1800, 12
+    g = torch.Generator(device="cuda").manual_seed(D)
+    for top in (256, 1024):
+        flat = torch.randint(0, top, (N * D + offset,), generator=g, device="cuda").float()
+        X = flat[offset:].view(N, D)
+        i, d = at.atsne_knn(X, k, precision="fp32")
+        at.atsne_check()
+        ri, rd = oracle(X, torch.arange(N, device="cuda"), k)
+        assert torch.equal(i, ri)
+        assert torch.equal(d, rd) if D * top * top < 2 ** 24 else torch.allclose(d, rd, rtol=(D / 8 + 12) * 2.0 ** -24)
