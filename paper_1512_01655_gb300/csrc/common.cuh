@@ -331,6 +331,9 @@ __device__ __forceinline__ uint32_t float_key(float f) {
     uint32_t u = __float_as_uint(f);
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
+__device__ __forceinline__ float key_of_bits(uint32_t u) {
+    return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
+}
 
 // In-warp bitonic sort of n (key, value) pairs held in shared memory,
 // ascending by (key, value). n is a power of two; the caller pads the unused

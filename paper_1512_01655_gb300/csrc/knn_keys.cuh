@@ -22,10 +22,6 @@ enum : int { META_FIRST = 1, META_RETRY = 2 };
 
 constexpr int F_PARTS = 4;  // candidate buffers per (row, split) of the fixed-threshold kernel
 
-__device__ __forceinline__ float key_of_bits(uint32_t u) {
-    return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
-}
-
 // Bound on |estimated - true| key (= squared distance - ||x_i||^2) for query
 // row statistics st = (||x||, residual norm of its BF16 copy, norm of its low
 // part) against any corpus point (gmax: the corpus maxima of the same): the

@@ -1094,8 +1094,8 @@ __global__ void __launch_bounds__(TcCfg<PASSES>::THREADS, 1) knn_tc_kernel(const
 // merge, FP32 rerank and certificate
 // ---------------------------------------------------------------------------
 struct MergeParams {
-    const Cand *cand;
-    const int4 *meta;
+    Cand *cand;
+    int4 *meta;
     int splits, cap;
     int64_t Q, N;
     const int32_t *qlist;
@@ -1114,6 +1114,7 @@ struct MergeParams {
     int Dp;
     int D, k, ksel;
     int rc, mst;            // re-rank set and staged keys per row (shared memory)
+    bool bounded;           // the keys' error is bounded (key_error_bound)
     const float *nrm;
     const float4 *stats;
     const float *Xq;        // queries from another array (row r = Xq[r]), else nullptr
@@ -1127,6 +1128,97 @@ struct MergeParams {
     int32_t *flag_rows;
     int32_t *flag_count;
 };
+
+// exact FP32 distances of rjw[from, to) in the library's one summation
+// order (group8_d2_pair), eight candidates per warp step; part of parts
+__device__ __forceinline__ void rerank_rows(const MergeParams &p, const float *xq, const int *rjw, float *rdw, int from,
+                                            int to, int part, int parts, bool exact_hi, int lane) {
+    const bool vec4 = (p.D & 3) == 0 && (reinterpret_cast<uintptr_t>(p.X) & 15) == 0 &&
+                      (reinterpret_cast<uintptr_t>(xq) & 15) == 0;
+    const int g = lane >> 3, gl = lane & 7;
+    const bool half = exact_hi && vec4;
+#pragma unroll 1
+    for (int t0 = from + 8 * part; half && t0 < to; t0 += 8 * parts) {
+        const int ta = t0 + g, tb = t0 + 4 + g;
+        const float2 s2 = group8_d2_pair_bf16(xq, p.hi + (int64_t)rjw[min(ta, to - 1)] * p.Dp,
+                                              p.hi + (int64_t)rjw[min(tb, to - 1)] * p.Dp, p.D, gl);
+        if (gl == 0) {
+            if (ta < to) rdw[ta] = s2.x;
+            if (tb < to) rdw[tb] = s2.y;
+        }
+    }
+    for (int t0 = from + 8 * part; !half && t0 < to; t0 += 8 * parts) {
+        const int ta = t0 + g, tb = t0 + 4 + g;
+        const float *xa = ta < to ? p.X + (int64_t)rjw[ta] * p.D : xq;
+        const float *xb = tb < to ? p.X + (int64_t)rjw[tb] * p.D : xq;
+        const float2 s2 = group8_d2_pair(xq, xa, xb, p.D, vec4, gl);
+        if (gl == 0) {
+            if (ta < to) rdw[ta] = s2.x;
+            if (tb < to) rdw[tb] = s2.y;
+        }
+    }
+}
+
+// The k nearest of a re-ranked row, sorted: only the first k + 1 in (distance,
+// index) order are needed: a set of 129 to 512 is cut to the entries at or below
+// its (k + 1)-th distance first when at most 128 remain.
+__device__ __forceinline__ void order_row(const MergeParams &p, const float *xq, float *rdw, int *rjw, int nr, double *dmw,
+                                          int *mpw, int lane) {
+    const int m1 = nr < p.k + 1 ? nr : p.k + 1;
+    int nsrt = nr;
+    if (nr > 128 && nr <= 512) {
+        const int c = warp_smallest_to_front(rdw, rjw, nr, m1, 128, lane);
+        if (c >= 0) nsrt = c;
+    }
+    int ns2 = 32;
+    while (ns2 < nsrt) ns2 <<= 1;
+    for (int t = nsrt + lane; t < ns2; t += 32) {
+        rdw[t] = INFINITY;
+        rjw[t] = INT_MAX;
+    }
+    __syncwarp();
+    warp_sort_pow2(rdw, rjw, ns2, lane);
+    __syncwarp();
+    // near ties among the first k + 1 ordered as the exact distances are
+    fp64_near_ties(rdw, rjw, nr, p.k, xq, p.X, p.D, dmw, mpw, lane);
+}
+
+// The largest key that a point among the k nearest, or tied with the k-th, can
+// have, given the distances rdw[0, n) of n >= k points (FP32 distances lie
+// within (m + 8) 2^-24 of their values, m = 4 ceil(D / 32): twice that for a
+// tie, and both ends). Ec: the key error bound, over the points of norm at most
+// ||x|| + sqrt(the largest of them).
+__device__ __forceinline__ float key_limit(const MergeParams &p, const float *rdw, int n, float4 st, float nx, int lane,
+                                           float &Ec) {
+    float dk0 = 0.f;
+    for (int t = lane; t < n; t += 32) dk0 = fmaxf(dk0, rdw[t]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) dk0 = fmaxf(dk0, __shfl_xor_sync(0xffffffffu, dk0, o));
+    Ec = fminf(key_error_bound(st, p.gmax, p.acc_coef, p.sq_coef),
+               key_error_bound_capped(st, p.gmax, p.acc_coef, p.sq_coef, st.x + sqrtf(dk0) * (1.f + 1e-6f) + 1e-30f));
+    const float e = (float)(4 * ((p.D + 31) / 32) + 8) * 0x1p-24f;
+    return dk0 * (1.f + 4.f * e) - nx + Ec + 1e-6f * (dk0 + nx);
+}
+
+// ordered columns: the collected positions mapped to rows of X, four loads in
+// flight per lane (one at a time per batch of the collection would wait on each)
+__device__ __forceinline__ void map_positions(const MergeParams &p, int *rjw, int from, int to, int lane) {
+    if (!p.perm) return;
+    for (int t0 = from; t0 < to; t0 += 128) {
+        int v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int t = t0 + 32 * q + lane;
+            v[q] = t < to ? p.perm[rjw[t]] : 0;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int t = t0 + 32 * q + lane;
+            if (t < to) rjw[t] = v[q];
+        }
+    }
+    __syncwarp();
+}
 
 // CERT (FP32 and BF16 modes): the k nearest, certified exact or sent to the
 // brute-force kernel. Otherwise (approximate modes): the SEL = ksel best keys
@@ -1145,8 +1237,9 @@ size_t merge_smem_bytes(bool cert, int rc, int mst, int rows) {
 // what counts, most of it the re-rank's gathers, a few in flight at a time (500
 // rows of 784 dimensions: 152 us with a warp per row, 102 us; of 50: 45 and 41
 // us; 2,000 rows of 784 191 and 221 us: their warps fill the SMs by themselves).
-template <bool CERT, int ROWS>
-__global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kernel(MergeParams p) {
+// SELECT: the set is left in the row's buffers for knn_rerank_kernel.
+template <bool CERT, int ROWS, bool SELECT = false>
+__global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : SELECT ? 6 : 5) knn_merge_kernel(MergeParams p) {
     extern __shared__ __align__(16) unsigned char mg_smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, w = ROWS == 1 ? 0 : warp;
     __shared__ const int *job_rj;
@@ -1177,33 +1270,8 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
     // their BF16 copy: half the bytes, the same values (70,000 x 784 bytes, k = 90: merge
     // 2,900 us from the FP32 rows, 2,510 now).
     const bool exact_hi = CERT && p.hi && !p.perm && p.gmax[3] == 0u;
-    // exact FP32 distances of rjw[from, to) in the library's one summation
-    // order (group8_d2_pair), eight candidates per warp step; part of parts
     auto rerank_part = [&](const float *xq, const int *rjw, int from, int to, int part, int parts) {
-        const bool vec4 = (p.D & 3) == 0 && (reinterpret_cast<uintptr_t>(p.X) & 15) == 0 &&
-                          (reinterpret_cast<uintptr_t>(xq) & 15) == 0;
-        const int g = lane >> 3, gl = lane & 7;
-        const bool half = exact_hi && vec4;
-#pragma unroll 1
-        for (int t0 = from + 8 * part; half && t0 < to; t0 += 8 * parts) {
-            const int ta = t0 + g, tb = t0 + 4 + g;
-            const float2 s2 = group8_d2_pair_bf16(xq, p.hi + (int64_t)rjw[min(ta, to - 1)] * p.Dp,
-                                                  p.hi + (int64_t)rjw[min(tb, to - 1)] * p.Dp, p.D, gl);
-            if (gl == 0) {
-                if (ta < to) rdw[ta] = s2.x;
-                if (tb < to) rdw[tb] = s2.y;
-            }
-        }
-        for (int t0 = from + 8 * part; !half && t0 < to; t0 += 8 * parts) {
-            const int ta = t0 + g, tb = t0 + 4 + g;
-            const float *xa = ta < to ? p.X + (int64_t)rjw[ta] * p.D : xq;
-            const float *xb = tb < to ? p.X + (int64_t)rjw[tb] * p.D : xq;
-            const float2 s2 = group8_d2_pair(xq, xa, xb, p.D, vec4, gl);
-            if (gl == 0) {
-                if (ta < to) rdw[ta] = s2.x;
-                if (tb < to) rdw[tb] = s2.y;
-            }
-        }
+        rerank_rows(p, xq, rjw, rdw, from, to, part, parts, exact_hi, lane);
     };
     if (ROWS == 1 && warp > 0) {
         for (;;) {
@@ -1415,10 +1483,11 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
         }
         // the re-rank set, collected in two bands of keys: (-inf, theta] then
         // (theta, lim]
-        auto take_batch = [&](bool take, int idx) {
+        auto take_batch = [&](bool take, int idx, float key) {
             const unsigned tm = __ballot_sync(0xffffffffu, take);
             const int pos = nr + __popc(tm & lanemask_lt());
             if (take && pos < RC) rjw[pos] = idx;
+            if (SELECT && take && pos < RC) rdw[pos] = key;
             nr += __popc(tm);
         };
         auto collect = [&](float lo, float hi) {  // keys in (lo, hi]
@@ -1431,17 +1500,18 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
                     const bool in = u[i] != 0xffffffffu && u[i] > ul && u[i] <= uh;
                     const int idx = in ? sj[t] : -1;
                     if (!CERT) __syncwarp();  // compacted in place, as below
-                    take_batch(in, idx);
+                    take_batch(in, idx, key_of_bits(u[i]));
                 }
             } else if (staged && hi <= slim) {  // all staged: every key up to slim was
                 for (int base = 0; base < ns; base += 32) {
                     const int i = base + lane;
-                    const bool in = i < ns && sk[i] > lo && sk[i] <= hi;
+                    const float key = i < ns ? sk[i] : 0.f;
+                    const bool in = i < ns && key > lo && key <= hi;
                     const int idx = i < ns ? sj[i] : -1;
                     // without a certificate the set is compacted in place
                     // (position <= i): the batch is read before it is written
                     if (!CERT) __syncwarp();
-                    take_batch(in, idx);
+                    take_batch(in, idx, key);
                 }
             } else {
                 for (int u = 0; u < S; ++u) {
@@ -1451,30 +1521,10 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
                         const int i = base + lane;
                         Cand e{INFINITY, -1};
                         if (i < c) e = b[i];
-                        take_batch(i < c && e.idx != self && e.key > lo && e.key <= hi, e.idx);
+                        take_batch(i < c && e.idx != self && e.key > lo && e.key <= hi, e.idx, e.key);
                     }
                 }
             }
-        };
-        // ordered columns: the collected positions mapped to rows of X, four
-        // loads in flight per lane (one at a time per batch of the collection
-        // would wait on each)
-        auto map_rows = [&](int from, int to) {
-            if (!p.perm) return;
-            for (int t0 = from; t0 < to; t0 += 128) {
-                int v[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int t = t0 + 32 * q + lane;
-                    v[q] = t < to ? p.perm[rjw[t]] : 0;
-                }
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int t = t0 + 32 * q + lane;
-                    if (t < to) rjw[t] = v[q];
-                }
-            }
-            __syncwarp();
         };
         const float *xq = cross ? p.Xq + r0 * p.D : p.X + (p.perm ? orow : (int64_t)qid) * p.D;
         auto rerank = [&](int from, int to) {
@@ -1509,51 +1559,27 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
             if (nr > RC) good = false;
             __syncwarp();
             if (!good) break;
-            map_rows(from, nr);
+            if (SELECT) {
+                // the row's own buffers are read and take the set
+                Cand *out = p.cand + (size_t)row * S * p.cap;
+                for (int t = lane; t < nr; t += 32) out[t] = Cand{rdw[t], rjw[t]};
+                break;
+            }
+            map_positions(p, rjw, from, nr, lane);
             rerank(from, nr);
             if (!CERT || round == 1) break;
             __syncwarp();
-            float dk0 = 0.f;
-            for (int t = lane; t < nr; t += 32) dk0 = fmaxf(dk0, rdw[t]);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) dk0 = fmaxf(dk0, __shfl_xor_sync(0xffffffffu, dk0, o));
-            const float4 st = cross ? p.qstats[r0] : p.stats[qid];
-            // the key error bound, over the points of norm at most ||x|| + sqrt(dk0)
-            Ec = fminf(key_error_bound(st, p.gmax, p.acc_coef, p.sq_coef),
-                       key_error_bound_capped(st, p.gmax, p.acc_coef, p.sq_coef,
-                                              st.x + sqrtf(dk0) * (1.f + 1e-6f) + 1e-30f));
-            // No point whose key exceeds this is among the k nearest or ties
-            // with the k-th (FP32 distances lie within (m + 8) 2^-24 of their
-            // values, m = 4 ceil(D / 32): twice that for a tie, and both ends)
-            const float nx = cross ? p.qnrm[r0] : p.nrm[qid];
-            const float e = (float)(4 * ((p.D + 31) / 32) + 8) * 0x1p-24f;
-            const float lim = dk0 * (1.f + 4.f * e) - nx + Ec + 1e-6f * (dk0 + nx);
+            const float lim = key_limit(p, rdw, nr, cross ? p.qstats[r0] : p.stats[qid], cross ? p.qnrm[r0] : p.nrm[qid],
+                                        lane, Ec);
             lo = theta;
             hi = fminf(lim, theta + 2.f * Ec);
             from = nr;
         }
         __syncwarp();
-        if (good && nr >= p.k) {
-            // only the first k + 1 in (distance, index) order are needed: a
-            // set of 129 to 512 is cut to the entries at or below its
-            // (k + 1)-th distance first when at most 128 remain
-            const int m1 = nr < p.k + 1 ? nr : p.k + 1;
-            int nsrt = nr;
-            if (nr > 128 && nr <= 512) {
-                const int c = warp_smallest_to_front(rdw, rjw, nr, m1, 128, lane);
-                if (c >= 0) nsrt = c;
-            }
-            int ns2 = 32;
-            while (ns2 < nsrt) ns2 <<= 1;
-            for (int t = nsrt + lane; t < ns2; t += 32) {
-                rdw[t] = INFINITY;
-                rjw[t] = INT_MAX;
-            }
-            __syncwarp();
-            warp_sort_pow2(rdw, rjw, ns2, lane);
-            __syncwarp();
-            // near ties among the first k + 1 ordered as the exact distances are
-            fp64_near_ties(rdw, rjw, nr, p.k, xq, p.X, p.D, dmw, mpw, lane);
+        if (SELECT) {
+            good = good && nr >= p.k;
+        } else if (good && nr >= p.k) {
+            order_row(p, xq, rdw, rjw, nr, dmw, mpw, lane);
             if (CERT) {
                 const float dk = rdw[p.k - 1];
                 const float nx = cross ? p.qnrm[r0] : p.nrm[qid];
@@ -1565,8 +1591,9 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
             good = false;
         }
     }
+    if (SELECT && lane == 0) p.meta[(size_t)row * S].x = good ? nr : -1;
     if (good) {
-        for (int t = lane; t < p.k; t += 32) {
+        for (int t = lane; !SELECT && t < p.k; t += 32) {
             p.idx_out[orow * p.k + t] = rjw[t];
             p.d2_out[orow * p.k + t] = rdw[t];
         }
@@ -1578,6 +1605,76 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : 5) knn_merge_kern
     if (ROWS == 1) {
         if (lane == 0) job[1] = -1;
         __syncthreads();
+    }
+}
+
+// The re-rank of the sets that knn_merge_kernel<false, ., true> left in the rows'
+// buffers (count in the row's first metadata word), one warp per row. In one kernel
+// the keys that the select holds in registers left 20 warps per SM to wait for
+// the gathers; by itself the re-rank runs 32. Where the keys' error is bounded the
+// k and some best keys are re-ranked first, and of the others only those that can
+// still be among the k nearest: the same lists with about half the gathers.
+// k = 90 of 360 keys: 1,000,000 x 128 41.0 ms in one kernel, 13.1 + 15.4 now;
+// 300,000 x 128 9.2 and 2.1 + 3.5 ms. What is left is bound by the L2's gather rate.
+__global__ void __launch_bounds__(MERGE_WARPS * 32, 8) knn_rerank_kernel(MergeParams p) {
+    extern __shared__ __align__(16) unsigned char mg_smem[];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    float *rdw = reinterpret_cast<float *>(mg_smem) + w * p.rc;
+    int *rjw = reinterpret_cast<int *>(mg_smem + (size_t)MERGE_WARPS * p.rc * 4) + w * p.rc;
+    double *dmw = reinterpret_cast<double *>(mg_smem + (size_t)MERGE_WARPS * p.rc * 8) + w * TIE_MAX;
+    int *mpw = reinterpret_cast<int *>(mg_smem + MERGE_WARPS * ((size_t)p.rc * 8 + TIE_MAX * 8)) + w * TIE_MAX;
+    const bool cross = p.Xq != nullptr;
+    const int64_t Q = p.qcount ? min(*p.qcount, p.Q) : p.Q;
+    const int64_t row = (int64_t)blockIdx.x * MERGE_WARPS + w;
+    if (row >= Q) return;
+    const int n = p.meta[(size_t)row * p.splits].x;
+    if (n < 0) return;  // flagged
+    const int qid = cross ? (int)row : (p.qlist ? p.qlist[row] : (int)row);
+    const int64_t orow = p.perm ? p.perm[row] : row;
+    const float *xq = cross ? p.Xq + row * p.D : p.X + (p.perm ? orow : (int64_t)qid) * p.D;
+    const Cand *cb = p.cand + (size_t)row * p.splits * p.cap;
+#pragma unroll 4
+    for (int t = lane; t < n; t += 32) {
+        const Cand e = cb[t];
+        rdw[t] = e.key;
+        rjw[t] = e.idx;
+    }
+    __syncwarp();
+    // the k and some best keys first: of the others only those that can still be
+    // among the k nearest need their distances
+    int from = 0, to = n, nr = n;
+    if (p.bounded && n > p.k + p.k / 4 + 8 && n <= 512)
+        to = warp_partition_keys(rdw, rjw, n, p.k, p.k + p.k / 8, lane);
+#pragma unroll 1
+    for (;;) {
+        map_positions(p, rjw, from, to, lane);
+        rerank_rows(p, xq, rjw, rdw, from, to, 0, 1, false, lane);
+        __syncwarp();
+        if (from > 0 || to == n) break;
+        float Ec;
+        const float lim = key_limit(p, rdw, to, cross ? p.qstats[row] : p.stats[qid], cross ? p.qnrm[row] : p.nrm[qid],
+                                    lane, Ec);
+        nr = to;
+        for (int base = to; base < n; base += 32) {
+            const int i = base + lane;
+            const float key = i < n ? rdw[i] : 0.f;
+            const int idx = i < n ? rjw[i] : -1;
+            const bool take = i < n && !(key > lim);
+            __syncwarp();  // compacted in place
+            const unsigned tm = __ballot_sync(0xffffffffu, take);
+            const int pos = nr + __popc(tm & lanemask_lt());
+            if (take) rjw[pos] = idx;
+            nr += __popc(tm);
+        }
+        __syncwarp();
+        from = to;
+        to = nr;
+        if (from == to) break;
+    }
+    order_row(p, xq, rdw, rjw, nr, dmw, mpw, lane);
+    for (int t = lane; t < p.k; t += 32) {
+        p.idx_out[orow * p.k + t] = rjw[t];
+        p.d2_out[orow * p.k + t] = rdw[t];
     }
 }
 
@@ -1998,13 +2095,19 @@ static atsne_status merge_launch(const TcPlan &pl, MergeParams m, cudaStream_t s
     // one row per block while the rows leave most of the SMs' warps idle, and for
     // those given up by the fixed threshold, which are few
     const bool one = m.rcount || m.Q <= MERGE_ONE_ROWS * num_sms();
+    const bool split = !pl.certify && !one;
     const size_t ms = merge_smem_bytes(pl.certify, m.rc, m.mst, one ? 1 : MERGE_WARPS);
     void (*kern)(MergeParams) = pl.certify ? (one ? knn_merge_kernel<true, 1> : knn_merge_kernel<true, MERGE_WARPS>)
-                                           : (one ? knn_merge_kernel<false, 1> : knn_merge_kernel<false, MERGE_WARPS>);
+                                           : (one ? knn_merge_kernel<false, 1> : knn_merge_kernel<false, MERGE_WARPS, true>);
     const int grid = m.rcount ? (int)hmin(4 * num_sms(), m.Q) : ceil_div(m.Q, one ? 1 : MERGE_WARPS);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ms);
     if (e != cudaSuccess) return cuda_error(e, "knn_tc_merge attribute");
-    return launch_kernel("knn_tc_merge", kern, grid, MERGE_WARPS * 32, ms, stream, m);
+    ATSNE_TRY(launch_kernel(split ? "knn_select" : "knn_tc_merge", kern, grid, MERGE_WARPS * 32, ms, stream, m));
+    if (!split) return ATSNE_OK;
+    const size_t rs = (size_t)MERGE_WARPS * ((size_t)m.rc * 8 + TIE_MAX * 12);
+    e = cudaFuncSetAttribute(knn_rerank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs);
+    if (e != cudaSuccess) return cuda_error(e, "knn_tc_merge attribute");
+    return launch_kernel("knn_tc_merge", knn_rerank_kernel, grid, MERGE_WARPS * 32, rs, stream, m);
 }
 
 atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist, int64_t Q, int k,
@@ -2088,6 +2191,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
     m.Dp = pl.Dp;
     m.D = D;
     m.k = k;
+    m.bounded = !fp8;
     m.nrm = w.nrm;
     m.stats = reinterpret_cast<const float4 *>(w.stats);
     m.Xq = Xq;
@@ -2099,8 +2203,8 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
     m.idx_out = idx_out;
     m.d2_out = d2_out;
     m.ksel = pl.ksel;
-    m.cand = reinterpret_cast<const Cand *>(w.cand);
-    m.meta = reinterpret_cast<const int4 *>(w.meta);
+    m.cand = reinterpret_cast<Cand *>(w.cand);
+    m.meta = reinterpret_cast<int4 *>(w.meta);
     m.qcount = qcount;
     m.bufs = Q * (int64_t)pl.splits;
     // the fixed-threshold launch; the rows it gives up follow in the adaptive one

@@ -142,4 +142,64 @@ __device__ __forceinline__ int warp_smallest_to_front(float *key, V *val, int n,
     return c;
 }
 
+// Reorders key/val[0, n) (n <= 512) so that the entries whose keys are at or
+// below some bound come first, and returns their number c: at least m (1 <= m
+// <= n), and at most `most` unless ties at the bound leave no such choice. Any
+// finite keys. Bisection as above, but for a count within [m, most].
+// Warp-cooperative; n, m and most uniform.
+template <typename V>
+__device__ __forceinline__ int warp_partition_keys(float *key, V *val, int n, int m, int most, int lane) {
+    constexpr int R = 16;
+    uint32_t u[R];
+    V v[R];
+    uint32_t lo = 0xffffffffu, hi = 0u;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int t = r * 32 + lane;
+        u[r] = 0xffffffffu;  // past n: above every key
+        if (t < n) {
+            u[r] = float_key(key[t]);
+            v[r] = val[t];
+            lo = min(lo, u[r]);
+            hi = max(hi, u[r]);
+        }
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    int c = n;
+    while (lo < hi && c > most) {
+        const uint32_t mid = lo + ((hi - lo) >> 1);
+        int c0 = 0, c1 = 0;
+#pragma unroll
+        for (int r = 0; r < R; r += 2) {
+            c0 += u[r] <= mid;
+            c1 += u[r + 1] <= mid;
+        }
+        const int cm = (int)__reduce_add_sync(0xffffffffu, (unsigned)(c0 + c1));
+        if (cm >= m) {
+            hi = mid;
+            c = cm;
+        } else {
+            lo = mid + 1;
+        }
+    }
+    __syncwarp();  // every entry is in registers before it is overwritten
+    const unsigned below = (1u << lane) - 1u;
+    int front = 0, back = c;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const bool on = r * 32 + lane < n, in = on && u[r] <= hi;
+        const unsigned bi = __ballot_sync(0xffffffffu, in), bo = __ballot_sync(0xffffffffu, on && !in);
+        if (on) {
+            const int pos = in ? front + __popc(bi & below) : back + __popc(bo & below);
+            key[pos] = key_of_bits(u[r]);
+            val[pos] = v[r];
+        }
+        front += __popc(bi);
+        back += __popc(bo);
+    }
+    __syncwarp();
+    return c;
+}
+
 }  // namespace atsne
