@@ -125,20 +125,21 @@ atsne_status atsne_knn(const float *X, int64_t N, int32_t D, const int32_t *quer
 
 /*
  * Gaussian bandwidths and conditional probabilities, Eq. 3 and Eq. 4 (Sec. 3)
- * over the kNN support of Eq. 8: for each row, beta = 1/(2 sigma^2) is found by
- * bisection so that exp(H) = perplexity (H in nats, equal to Eq. 4's base-2
+ * over the kNN support of Eq. 8: for each row, beta = 1/(2 sigma^2) is searched
+ * so that exp(H) = perplexity (H in nats, equal to Eq. 4's base-2
  * form), and P_cond[r][j] = exp(-beta d2[r][j]) / sum_l exp(-beta d2[r][l]).
  *  d2         [rows][k] fp32 squared distances (any order; >= 0). +inf marks an
  *             absent neighbour (a row shortened by atsne_delete_rows): it takes
  *             no part in the sums and gets P 0. NaN or a negative value raises
  *             the device status.
  *  perplexity 0 < perplexity < k.   tol: stop when |H - ln perplexity| < tol
- *  (<= 0 selects 1e-5).  max_iter: bisection steps (<= 0 selects 200).
+ *  (<= 0 selects 1e-5).  max_iter: bisection steps (<= 0 selects 200). With the
+ *  two defaults and k <= 256 the search takes Newton steps in ln beta instead.
  *  P_cond_out [rows][k] fp32 (rows sum to 1), beta_out [rows] fp32 (may be NULL).
  * Rows whose target is unreachable (k equal distances, or at least
  * `perplexity` neighbours tied at the smallest distance) end at max_iter.
  * A row of n present neighbours with n <= perplexity (its entropy is at most
- * ln n, reached only at beta = 0) takes the bisection's limit: beta = 0 and
+ * ln n, reached only at beta = 0) takes the search's limit: beta = 0 and
  * P = 1/n on the present entries; a row with none gets P 0 and beta 0.
  */
 atsne_status atsne_calibrate_P(const float *d2, int64_t rows, int32_t k, float perplexity,
@@ -205,7 +206,7 @@ atsne_status atsne_refine_subset_noalloc(const float *X, int64_t N, int32_t D,
  * atsne_refine_subset on every selection in any order, and each point of the
  * union is computed once: the union is formed on the device (bitmap, then an
  * ordered compaction) and refined by one exact kNN on the tensor cores, one
- * bisection and one row scatter.
+ * bandwidth search and one row scatter over as many rows.
  *  refined_count  device int64 receiving the size of the union (may be NULL).
  *  lists may be NULL when total is 0 (nothing is refined).
  * Stream-ordered, with no host synchronisation and no allocation: the call can
@@ -236,8 +237,8 @@ atsne_status atsne_knn_rows(const float *X, int64_t N, int32_t D, const int32_t 
 /*
  * Autotuner of the exact tensor-core kNN. Its tunable is the column split: the
  * corpus columns are cut into `splits` ranges, each (row tile, range) unit runs
- * its own streaming top-k, and the partial lists are merged. Fewer splits mean
- * fewer survivors to merge, more splits more units to fill the SMs with when
+ * into its own candidate buffers, and the buffers are merged. Fewer splits mean
+ * fewer and longer buffers, more splits more units to fill the SMs with when
  * the rows are few. This call times the candidates (one split, and the counts
  * giving about 152 .. 8192 units) on the given problem (the kNN of
  * atsne_knn with method EXACT on the tensor cores: `queries` [S] or all N rows
@@ -320,7 +321,7 @@ atsne_status atsne_merge_neighbors(int32_t *idx, float *d2, int64_t rows, int32_
  * 0..N-R-1: X ([N][D]), idx/d2/P_cond ([N][k]), beta and rho ([N]) are
  * compacted in place and every index renumbered. Every remaining row's Gaussian
  * is then calibrated again over its remaining neighbours (Eq. 3, Eq. 4 over
- * N_i; bisection as atsne_calibrate_P with its default tolerance), which the
+ * N_i; searched as atsne_calibrate_P with its default tolerance), which the
  * absent entries do not enter. A later insertion fills an absent entry with a
  * new point closer than the row's farthest remaining neighbour (d_i^Max over
  * N_i as it stands, atsne_row_dmax). An index out of range or listed twice raises the device

@@ -230,7 +230,7 @@ def atsne_tune_clear():
 
 
 def atsne_calibrate_P(d2, perplexity, tol=0.0, max_iter=0, stream=None, P_out=None, beta_out=None):
-    """Conditional rows P_{j|i} and beta by bisection -- Eq. 3-4 over N_i.
+    """Conditional rows P_{j|i} and beta of a perplexity -- Eq. 3-4 over N_i.
     P_out / beta_out: contiguous tensors to write into (else new ones)."""
     _dev(d2, torch.float32, "d2")
     rows, k = d2.shape

@@ -71,6 +71,7 @@ constexpr int TC_BN = 256;       // corpus points per tile (TMEM columns per acc
 constexpr int TC_BK = 64;        // BF16 per k-block (one 128-byte swizzle row)
 constexpr uint64_t WAIT_NS = 1000000000ull;
 constexpr int MERGE_WARPS = 4;
+constexpr int RERANK_KEYS = 512;    // keys of a row that knn_rerank_kernel holds
 constexpr int MERGE_ONE_ROWS = 4;   // rows per SM up to which a block merges one row
 constexpr int RCAP = 256;        // candidates re-ranked per row at most (certified modes)
 constexpr int MSTAGE = 1024;     // keys below tau staged per row for the merge's select
@@ -1115,6 +1116,9 @@ struct MergeParams {
     int D, k, ksel;
     int rc, mst;            // re-rank set and staged keys per row (shared memory)
     bool bounded;           // the keys' error is bounded (key_error_bound)
+    // certified modes, if given: the rows with too many keys for knn_rerank_kernel,
+    // which knn_merge_kernel then takes
+    int32_t *big_rows, *big_count;
     const float *nrm;
     const float4 *stats;
     const float *Xq;        // queries from another array (row r = Xq[r]), else nullptr
@@ -1258,7 +1262,7 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : SELECT ? 6 : 5) k
                w * TIE_MAX;
     const int sel = CERT ? p.k : p.ksel;  // rank of the key that bounds the re-rank set
     const bool cross = p.Xq != nullptr;
-    int64_t Q = p.qcount ? min(*p.qcount, p.Q) : p.Q;
+    int64_t Q = p.big_rows ? *p.big_count : p.qcount ? min(*p.qcount, p.Q) : p.Q;
     int S = p.splits;
     if (p.rcount) {
         const UnitPlan up = retry_plan(*p.rcount, p.N, p.bufs);
@@ -1283,8 +1287,9 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : SELECT ? 6 : 5) k
             __syncthreads();
         }
     }
-    for (int64_t row = (int64_t)blockIdx.x * ROWS + w; row < Q; row += (int64_t)gridDim.x * ROWS) {
+    for (int64_t it = (int64_t)blockIdx.x * ROWS + w; it < Q; it += (int64_t)gridDim.x * ROWS) {
     __syncwarp();
+    const int64_t row = p.big_rows ? p.big_rows[it] : it;
     const int64_t r0 = p.rlist ? p.rlist[row] : row;  // the query row
     const int qid = cross ? (int)r0 : (p.qlist ? p.qlist[r0] : (int)r0);
     const int self = cross ? -1 : qid;                // the fixed threshold buffers the query itself too
@@ -1616,6 +1621,12 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : SELECT ? 6 : 5) k
 // still be among the k nearest: the same lists with about half the gathers.
 // k = 90 of 360 keys: 1,000,000 x 128 41.0 ms in one kernel, 13.1 + 15.4 now;
 // 300,000 x 128 9.2 and 2.1 + 3.5 ms. What is left is bound by the L2's gather rate.
+// With a certificate (CERT) it takes the row's buffers as they are: a row rarely
+// has more than RERANK_KEYS keys, and those rows are listed for knn_merge_kernel.
+// 70,000 x 784 bytes, k = 90 (273 keys per row): 2,505 us in the one kernel (128
+// registers, 16 warps per SM), 1,768 + 13; 50,021 x 50 1,017 and 647 + 65; 200,000
+// x 128 2,876 and 1,510 + 47; 2,000 x 64 44 and 31 + 12.
+template <bool CERT>
 __global__ void __launch_bounds__(MERGE_WARPS * 32, 8) knn_rerank_kernel(MergeParams p) {
     extern __shared__ __align__(16) unsigned char mg_smem[];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1627,54 +1638,130 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, 8) knn_rerank_kernel(MergePa
     const int64_t Q = p.qcount ? min(*p.qcount, p.Q) : p.Q;
     const int64_t row = (int64_t)blockIdx.x * MERGE_WARPS + w;
     if (row >= Q) return;
-    const int n = p.meta[(size_t)row * p.splits].x;
-    if (n < 0) return;  // flagged
+    const int S = p.splits;
+    const int4 *mt = p.meta + (size_t)row * S;
+    const Cand *cb = p.cand + (size_t)row * S * p.cap;
     const int qid = cross ? (int)row : (p.qlist ? p.qlist[row] : (int)row);
     const int64_t orow = p.perm ? p.perm[row] : row;
     const float *xq = cross ? p.Xq + row * p.D : p.X + (p.perm ? orow : (int64_t)qid) * p.D;
-    const Cand *cb = p.cand + (size_t)row * p.splits * p.cap;
+    const bool exact_hi = CERT && p.hi && !p.perm && p.gmax[3] == 0u;
+    int n = 0;
+    float tau_min = INFINITY;
+    bool good = true, ovf = false;
+    if (!CERT) {
+        n = mt[0].x;
+        if (n < 0) return;  // flagged
 #pragma unroll 4
-    for (int t = lane; t < n; t += 32) {
-        const Cand e = cb[t];
-        rdw[t] = e.key;
-        rjw[t] = e.idx;
+        for (int t = lane; t < n; t += 32) {
+            const Cand e = cb[t];
+            rdw[t] = e.key;
+            rjw[t] = e.idx;
+        }
+    } else {
+        int total = 0;
+        for (int u = lane; u < S; u += 32) {
+            const int4 m = mt[u];
+            ovf |= m.z || m.w != p.tag;  // or a unit that a stopped launch never finished
+            total += min(max(m.x, 0), p.cap);
+            tau_min = fminf(tau_min, __int_as_float(m.y));
+        }
+        ovf = __any_sync(0xffffffffu, ovf);
+        total = (int)__reduce_add_sync(0xffffffffu, (unsigned)total);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) tau_min = fminf(tau_min, __shfl_xor_sync(0xffffffffu, tau_min, o));
+        good = !ovf && total >= p.k && qid >= 0 && (cross || qid < p.N);
+        if (good && total > RERANK_KEYS) {
+            if (lane == 0) p.big_rows[atomicAdd(p.big_count, 1)] = (int)row;
+            return;
+        }
+        const int self = cross ? -1 : qid;
+        // 32 buffers at a time, their entries as one sequence: a lane finds its
+        // entry's buffer by a binary search over the lanes' counts
+        for (int u0 = 0; good && u0 < S; u0 += 32) {
+            const int c = u0 + lane < S ? min(max(mt[u0 + lane].x, 0), p.cap) : 0;
+            int incl = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += t;
+            }
+            const int all = __shfl_sync(0xffffffffu, incl, 31);
+            for (int base = 0; base < all; base += 128) {
+                Cand e[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int t = base + 32 * q + lane;
+                    int b = 0;  // the first buffer whose inclusive count exceeds t
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1)
+                        if (__shfl_sync(0xffffffffu, incl, b + o - 1) <= t) b += o;
+                    const int first = __shfl_sync(0xffffffffu, incl - c, b);
+                    e[q] = Cand{INFINITY, -1};
+                    if (t < all) e[q] = cb[(size_t)(u0 + b) * p.cap + (t - first)];
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const bool on = base + 32 * q + lane < all && e[q].idx != self;
+                    const unsigned tm = __ballot_sync(0xffffffffu, on);
+                    const int pos = n + __popc(tm & lanemask_lt());
+                    if (on) {
+                        rdw[pos] = e[q].key;
+                        rjw[pos] = e[q].idx;
+                    }
+                    n += __popc(tm);
+                }
+            }
+        }
+        good = good && n >= p.k;
     }
     __syncwarp();
-    // the k and some best keys first: of the others only those that can still be
-    // among the k nearest need their distances
-    int from = 0, to = n, nr = n;
-    if (p.bounded && n > p.k + p.k / 4 + 8 && n <= 512)
-        to = warp_partition_keys(rdw, rjw, n, p.k, p.k + p.k / 8, lane);
+    if (good) {
+        // the k and some best keys first: of the others only those that can
+        // still be among the k nearest need their distances
+        int from = 0, to = n, nr = n;
+        if ((CERT || p.bounded) && n > p.k + p.k / 4 + 8 && n <= 512)
+            to = warp_partition_keys(rdw, rjw, n, p.k, p.k + p.k / 8, lane);
+        float Ec = 0.f;
 #pragma unroll 1
-    for (;;) {
-        map_positions(p, rjw, from, to, lane);
-        rerank_rows(p, xq, rjw, rdw, from, to, 0, 1, false, lane);
-        __syncwarp();
-        if (from > 0 || to == n) break;
-        float Ec;
-        const float lim = key_limit(p, rdw, to, cross ? p.qstats[row] : p.stats[qid], cross ? p.qnrm[row] : p.nrm[qid],
-                                    lane, Ec);
-        nr = to;
-        for (int base = to; base < n; base += 32) {
-            const int i = base + lane;
-            const float key = i < n ? rdw[i] : 0.f;
-            const int idx = i < n ? rjw[i] : -1;
-            const bool take = i < n && !(key > lim);
-            __syncwarp();  // compacted in place
-            const unsigned tm = __ballot_sync(0xffffffffu, take);
-            const int pos = nr + __popc(tm & lanemask_lt());
-            if (take) rjw[pos] = idx;
-            nr += __popc(tm);
+        for (;;) {
+            map_positions(p, rjw, from, to, lane);
+            rerank_rows(p, xq, rjw, rdw, from, to, 0, 1, exact_hi, lane);
+            __syncwarp();
+            if (from > 0 || (!CERT && to == n)) break;
+            const float lim = key_limit(p, rdw, to, cross ? p.qstats[row] : p.stats[qid],
+                                        cross ? p.qnrm[row] : p.nrm[qid], lane, Ec);
+            nr = to;
+            for (int base = to; base < n; base += 32) {
+                const int i = base + lane;
+                const float key = i < n ? rdw[i] : 0.f;
+                const int idx = i < n ? rjw[i] : -1;
+                const bool take = i < n && !(key > lim);
+                __syncwarp();  // compacted in place
+                const unsigned tm = __ballot_sync(0xffffffffu, take);
+                const int pos = nr + __popc(tm & lanemask_lt());
+                if (take) rjw[pos] = idx;
+                nr += __popc(tm);
+            }
+            __syncwarp();
+            from = to;
+            to = nr;
+            if (from == to) break;
         }
-        __syncwarp();
-        from = to;
-        to = nr;
-        if (from == to) break;
+        order_row(p, xq, rdw, rjw, nr, dmw, mpw, lane);
+        if (CERT) {
+            // certified: no point outside the buffers can be closer than the k-th
+            const float lb = (cross ? p.qnrm[row] : p.nrm[qid]) + tau_min - Ec;
+            good = isinf(tau_min) || rdw[p.k - 1] < lb * (1.f - 1e-6f);
+        }
     }
-    order_row(p, xq, rdw, rjw, nr, dmw, mpw, lane);
-    for (int t = lane; t < p.k; t += 32) {
-        p.idx_out[orow * p.k + t] = rjw[t];
-        p.d2_out[orow * p.k + t] = rdw[t];
+    if (good) {
+        for (int t = lane; t < p.k; t += 32) {
+            p.idx_out[orow * p.k + t] = rjw[t];
+            p.d2_out[orow * p.k + t] = rdw[t];
+        }
+    } else if (lane == 0) {
+        p.flag_rows[atomicAdd(p.flag_count, 1)] = (int)(p.flag_out ? orow : row);
+        if (p.tau_mark && !ovf) p.tau_mark[row] = INFINITY;
     }
 }
 
@@ -1951,6 +2038,7 @@ static void plan_filter(TcPlan &pl, int64_t N, int64_t Q, int splits) {
     pl.fsplits = (int)((N + pl.fcols - 1) / pl.fcols);
     // a row's neighbours may all lie in one split (a corpus sorted by class),
     // but spread over the parts of its tiles
+    pl.fkeys = (int)expect;
     int64_t cap = (int64_t)ceil(2.0 * expect / F_PARTS) + 48;
     if (cap > per * cw) cap = per * cw;
     pl.fcap = (int)((cap + 15) / 16 * 16);
@@ -2040,7 +2128,7 @@ size_t tc_workspace(Carver &c, int64_t N, int D, int64_t Q, bool list, const TcP
     w.hist_rows = pl.filter ? (pl.S > 0 ? hmin(Q, RETRY_SPLIT_ROWS) : 0) : pl.splits > 1 ? Q : 0;
     w.row_hist = w.hist_rows > 0 ? c.take<unsigned>((size_t)w.hist_rows * GH_BUCKETS) : nullptr;
     w.flag_rows = c.take<int32_t>((size_t)Q);
-    w.flag_count = c.take<int32_t>(2);
+    w.flag_count = c.take<int32_t>(3);
     w.bext = pl.passes == 1 ? c.take<uint16_t>((size_t)((N + TC_BN - 1) / TC_BN * TC_BN) * 16) : nullptr;
     w.aext = pl.passes == 1 || pl.S > 0 ? c.take<uint16_t>((size_t)TC_BM * 16) : nullptr;
     if (pl.filter) w.tau = c.take<float>((size_t)Q);
@@ -2095,19 +2183,33 @@ static atsne_status merge_launch(const TcPlan &pl, MergeParams m, cudaStream_t s
     // one row per block while the rows leave most of the SMs' warps idle, and for
     // those given up by the fixed threshold, which are few
     const bool one = m.rcount || m.Q <= MERGE_ONE_ROWS * num_sms();
+    auto rerank = [&](void (*k)(MergeParams)) {
+        const size_t rs = (size_t)MERGE_WARPS * ((size_t)m.rc * 8 + TIE_MAX * 12);
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs);
+        if (e != cudaSuccess) return cuda_error(e, "knn_tc_merge attribute");
+        return launch_kernel("knn_rerank", k, ceil_div(m.Q, MERGE_WARPS), MERGE_WARPS * 32, rs, stream, m);
+    };
     const bool split = !pl.certify && !one;
-    const size_t ms = merge_smem_bytes(pl.certify, m.rc, m.mst, one ? 1 : MERGE_WARPS);
-    void (*kern)(MergeParams) = pl.certify ? (one ? knn_merge_kernel<true, 1> : knn_merge_kernel<true, MERGE_WARPS>)
-                                           : (one ? knn_merge_kernel<false, 1> : knn_merge_kernel<false, MERGE_WARPS, true>);
-    const int grid = m.rcount ? (int)hmin(4 * num_sms(), m.Q) : ceil_div(m.Q, one ? 1 : MERGE_WARPS);
+    // certified modes: the lighter kernel where a row's expected keys leave room
+    // (two thirds: about a row in a hundred then has more than RERANK_KEYS, and
+    // goes to the one kernel afterwards), else, as for few rows, the one kernel
+    const bool light = pl.certify && !one && m.big_rows && 3 * pl.fkeys <= 2 * RERANK_KEYS && m.k <= RERANK_KEYS / 2;
+    if (light) {
+        m.rc = RERANK_KEYS;
+        ATSNE_TRY(rerank(knn_rerank_kernel<true>));
+        m.rc = RCAP;
+    } else {
+        m.big_rows = m.big_count = nullptr;
+    }
+    const bool few = one || light;
+    const size_t ms = merge_smem_bytes(pl.certify, m.rc, m.mst, few ? 1 : MERGE_WARPS);
+    void (*kern)(MergeParams) = pl.certify ? (few ? knn_merge_kernel<true, 1> : knn_merge_kernel<true, MERGE_WARPS>)
+                                           : (few ? knn_merge_kernel<false, 1> : knn_merge_kernel<false, MERGE_WARPS, true>);
+    const int grid = m.rcount || light ? (int)hmin(4 * num_sms(), m.Q) : ceil_div(m.Q, one ? 1 : MERGE_WARPS);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ms);
     if (e != cudaSuccess) return cuda_error(e, "knn_tc_merge attribute");
     ATSNE_TRY(launch_kernel(split ? "knn_select" : "knn_tc_merge", kern, grid, MERGE_WARPS * 32, ms, stream, m));
-    if (!split) return ATSNE_OK;
-    const size_t rs = (size_t)MERGE_WARPS * ((size_t)m.rc * 8 + TIE_MAX * 12);
-    e = cudaFuncSetAttribute(knn_rerank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs);
-    if (e != cudaSuccess) return cuda_error(e, "knn_tc_merge attribute");
-    return launch_kernel("knn_tc_merge", knn_rerank_kernel, grid, MERGE_WARPS * 32, rs, stream, m);
+    return split ? rerank(knn_rerank_kernel<false>) : ATSNE_OK;
 }
 
 atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist, int64_t Q, int k,
@@ -2116,7 +2218,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
                           const int64_t *qcount) {
     int *status = device_status_word();
     cudaError_t e = cudaMemsetAsync(w.gmax, 0, 4 * sizeof(unsigned), stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(w.flag_count, 0, 2 * sizeof(int32_t), stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w.flag_count, 0, 3 * sizeof(int32_t), stream);
     if (e == cudaSuccess && w.clock) e = cudaMemsetAsync(w.clock, 0, sizeof(unsigned long long), stream);
     if (e == cudaSuccess && w.row_hist)
         e = cudaMemsetAsync(w.row_hist, 0, (size_t)w.hist_rows * GH_BUCKETS * sizeof(unsigned), stream);
@@ -2233,6 +2335,8 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
         m.flag_rows = retry ? w.retry_rows : w.flag_rows;
         m.flag_count = retry ? w.flag_count + 1 : w.flag_count;
         m.tau_mark = retry ? w.tau : nullptr;
+        m.big_rows = retry ? w.flag_rows : nullptr;  // not in use before the retried rows' merge
+        m.big_count = w.flag_count + 2;
         if (radius) {
             ATSNE_TRY(launch_kernel("knn_tc_merge", radius_merge_kernel, ceil_div(Q, MERGE_WARPS),
                                     MERGE_WARPS * 32, 0, stream, m, radius));
@@ -2331,6 +2435,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
     m.tag = retry ? META_RETRY : META_FIRST;
     m.flag_out = true;
     m.tau_mark = nullptr;
+    m.big_rows = nullptr;
     m.flag_rows = w.flag_rows;
     m.flag_count = w.flag_count;
     ATSNE_TRY(merge_launch(pl, m, stream));
