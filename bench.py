@@ -271,7 +271,8 @@ TRAFFIC_SOURCES = {
     "forest_traverse_u8": ["forest_query.cu", "common.cuh", "internal.h"],
     "forest_dist": ["forest_query.cu", "common.cuh", "internal.h"],
     "forest_dist_u8": ["forest_query.cu", "common.cuh", "internal.h"],
-    "knn_tc": ["knn_tc.cu", "tc_ptx.cuh", "common.cuh", "internal.h", "warp_sort.cuh"],
+    "knn_filter": ["knn_filter.cu", "knn_keys.cuh", "tc_ptx.cuh", "common.cuh", "internal.h"],
+    "knn_tc": ["knn_tc.cu", "knn_keys.cuh", "tc_ptx.cuh", "common.cuh", "internal.h", "warp_sort.cuh"],
 }
 
 
@@ -549,13 +550,14 @@ def timed_steps(torch, fn, steps, stream, l2_flush=None):
     return [a.elapsed_time(b) for a, b in evs], out
 
 
-PROFILED = ["knn_order", "knn_prep", "knn_tc", "knn_tc_merge", "knn_fallback", "knn_bruteforce", "calibrate_beta",
-            "sym_fwd", "sym_rev", "sym_len", "sym_write", "sym_sort_long", "sym_write_long",
+PROFILED = ["knn_order", "knn_prep", "knn_sample", "knn_bound", "knn_tau", "knn_filter", "knn_gather", "knn_retry_tau",
+            "knn_tc", "knn_select", "knn_rerank", "knn_tc_merge", "knn_fallback", "knn_bruteforce", "calibrate_beta",
+            "sym_count", "sym_place", "sym_merge", "sym_mid", "sym_hub", "sym_copy",
             "scan_reduce", "scan_partials", "scan_down",
             "forest_traverse", "forest_traverse_u8", "forest_dist", "forest_dist_u8", "forest_u8_prep",
             "forest_choose", "forest_partial", "forest_sort_smem", "forest_sort_global", "forest_keys",
             "forest_scatter", "forest_leaf_pt", "refine_scatter", "knn_precision"]
-SYM_PARTS = ("sym_fwd", "sym_rev", "sym_len", "sym_write", "sym_sort_long", "sym_write_long",
+SYM_PARTS = ("sym_count", "sym_place", "sym_merge", "sym_mid", "sym_hub", "sym_copy",
              "scan_reduce", "scan_partials", "scan_down")
 
 
@@ -576,15 +578,18 @@ def exact_rooflines(per_kernel, steps, N, D, k, nnz, passes, prec, peaks, worklo
     hbm, hbm_src = peak_of(peaks, "hbm_gbs")
     bf16, bf16_src = peak_of(peaks, "bf16_tflops")
     lines = {}
-    if "knn_tc" in per_kernel:
-        pk = per_kernel["knn_tc"]
+    # the contraction: the fixed-threshold kernel, or the adaptive one where it
+    # does the whole work (FP8, small corpora)
+    knn = max((n for n in ("knn_filter", "knn_tc") if n in per_kernel), key=lambda n: per_kernel[n]["ms"], default=None)
+    if knn:
+        pk = per_kernel[knn]
         avg = pk["ms"] / pk["launches"]
         peak = bf16 * (2.0 if prec == "fp8" else 1.0)
         ach = algorithmic_flops_knn(N, N, D) / (avg / 1e3) / 1e12
-        lines["knn_tc"] = {
-            "kernel": "knn_tc", "bound": "tensor", "achieved": round(ach, 1), "peak": round(peak, 1),
+        lines["knn"] = {
+            "kernel": knn, "bound": "tensor", "achieved": round(ach, 1), "peak": round(peak, 1),
             "unit": "TFLOP/s", "frac": round(ach / peak, 4), "launch_ms": round(avg, 3),
-            "traffic": recorded_traffic("knn_tc", workload, prec),
+            "traffic": recorded_traffic(knn, workload, prec),
             "algorithmic_flops_per_launch": algorithmic_flops_knn(N, N, D), "tensor_passes": passes,
             "peak_source": bf16_src + (" x 2 (FP8 nominal ratio)" if prec == "fp8" else "")}
     Dp = 64 * ((D + 63) // 64)
@@ -606,10 +611,11 @@ def exact_rooflines(per_kernel, steps, N, D, k, nnz, passes, prec, peaks, worklo
                        "frac": round(ach / hbm, 4), "ms": round(ms, 3), "algorithmic_bytes": int(bytes_),
                        "peak_source": hbm_src}
     if "calibrate_beta" in lines:
-        lines["calibrate_beta"]["note"] = ("bound by the exponentials of the bisection (about 40-60 "
+        lines["calibrate_beta"]["note"] = ("bound by the exponentials of the search (about 5 Newton "
                                            "steps of k exp per row), not by its bytes")
-    if "knn_tc_merge" in per_kernel:
-        lines["knn_tc_merge"] = {"bound": "gather", "ms": round(per_kernel["knn_tc_merge"]["ms"] / steps, 3)}
+    merge = [n for n in ("knn_select", "knn_rerank", "knn_tc_merge") if n in per_kernel]
+    if merge:
+        lines["knn_merge"] = {"bound": "gather", "ms": round(sum(per_kernel[n]["ms"] for n in merge) / steps, 3)}
     return lines
 
 
@@ -678,7 +684,7 @@ def run_ours(args, world, rank, local, pg):
     passes = passes_of(args.precision)
     rooflines = exact_rooflines(per_kernel, args.steps, N, D, K_NN, nnz, passes, args.precision, peaks,
                                 args.workload)
-    roofline = rooflines.get("knn_tc")
+    roofline = rooflines.get("knn")
     idx_by_prec = {args.precision: idx_head.cpu().numpy()}
     del out, idx_head
     torch.cuda.empty_cache()
@@ -743,7 +749,7 @@ def run_ours(args, world, rank, local, pg):
         modes[prec] = {"what": PREC_NAME[prec], "steps": reps, "ms": round(med, 3),
                        "points_per_s": round(world * N / (med / 1e3), 1),
                        "stage_ms": {k_: round(v["ms"] / reps, 3) for k_, v in pk.items()},
-                       "knn_tc": rl.get("knn_tc")}
+                       "knn": rl.get("knn")}
         idx_by_prec[prec] = out[0].cpu().numpy()
         del out, st
         torch.cuda.empty_cache()
@@ -799,7 +805,7 @@ def run_ours(args, world, rank, local, pg):
             "recall_vs_fp32": head_recall, "recall_vs_oracle": recall_oracle, "nnz_P": nnz,
             "stage_ms": {k_: round(v["ms"] / args.steps, 3) for k_, v in per_kernel.items()},
             "step_ms": [round(t, 3) for t in step_ms],
-            "roofline": roofline, "bandwidth_kernels": {k_: v for k_, v in rooflines.items() if k_ != "knn_tc"},
+            "roofline": roofline, "bandwidth_kernels": {k_: v for k_, v in rooflines.items() if k_ != "knn"},
             "modes": modes, "approx_path": approx, "refine_batch": refine_batch, "serving": serving,
             "cpu_baseline": cpu, "e2e": e2e, "clocks": clk, "gpu_launches": int(launches),
         }
