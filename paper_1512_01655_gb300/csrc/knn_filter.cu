@@ -26,8 +26,8 @@
 // 1,000,000 x 128 Gamma clusters, one BF16 pass, ksel 360: 270 ms to 178 ms
 // (+ 7 ms for the thresholds), about 1.6 PFLOP/s, near the rate the power limit
 // leaves (the contraction alone 0.65 us per 256 x 256 x 144 pair tile, MMAs
-// 90% of it); 200,000 x 128, three passes, ksel 128: 22.7 to 14.4 ms; 50,021 x
-// 50 log-normal, ksel 188: 4.6 to 1.0 ms; 70,000 x 784 bytes: 6.4 to 5.0 ms;
+// 90% of it); 200,000 x 128, three passes, ksel 128: 22.7 to 14.0 ms; 50,021 x
+// 50 log-normal, ksel 188: 4.6 to 0.94 ms; 70,000 x 784 bytes: 6.4 to 4.5 ms;
 // 7,013 queries against 107,013 x 50: 9.1 to 0.3 ms.
 //
 // Layout. Two CTAs on neighbouring SMs form a pair (cta_group::2): M = 256

@@ -13,10 +13,11 @@
 //              taken from a sample of the corpus; the keys below it are
 //              buffered. The path of every corpus of at least
 //              FILTER_MIN_ROWS rows in the BF16 and FP32 modes.
-//   knn_merge  one warp per query: the k-th smallest buffered key is selected,
-//              every candidate within 2E of it (E bounds the key error, see
-//              key_error_bound) is re-ranked by FP32 direct differences, and a
-//              certificate is checked: if the k-th exact distance is below
+//   knn_merge, knn_rerank (and knn_merge as knn_select, in the modes without a
+//              certificate)  one warp per query: the k best buffered keys are
+//              re-ranked by FP32 direct differences, then every candidate whose
+//              key lies within E (the bound on its error, see key_error_bound)
+//              of the largest distance found, and a certificate is checked: if the k-th exact distance is below
 //              ||x_i||^2 + min(tau) - E, no point outside the buffers can
 //              belong to the k nearest, and the row is exact.
 //   knn_tc     the same contraction with a threshold that adapts as the columns
