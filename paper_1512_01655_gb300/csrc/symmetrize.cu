@@ -21,7 +21,7 @@
 //   6. copy:  rows to their final places, scaled by 1 / 2N.
 // A warp's sort moves one word per entry: column, forward/reverse bit and the
 // entry's slot (where its value waits in shared memory) in 32 bits while the
-// column fits (N <= 2^21), else 64; a compare-exchange is a shuffle and a
+// column fits (N < 2^21), else 64; a compare-exchange is a shuffle and a
 // min/max. Sorting forward and reverse rows separately as (key, value) pairs in
 // shared memory, with a binary search of each entry in the other list, twice,
 // took 3.08, 13.7 and 1.63 ms (300,000 rows of separate clusters, 1,000,000
@@ -39,7 +39,10 @@ namespace {
 constexpr int SYM_WARPS = 4;
 constexpr int SYM_BULK = 512;         // entries of a row sorted by sym_merge_kernel
 constexpr int SYM_MID = 1024;         // by sym_mid_kernel
-constexpr int64_t SYM_KEY32 = int64_t(1) << 21;  // columns that fit a 32-bit key with 10 slot bits
+// Below so many rows an entry's key fits 32 bits: 21 column bits, the reverse
+// bit, 10 slot bits. With one row more, the last column's reverse entry in the
+// last slot would be all ones, the mark for no entry.
+constexpr int64_t SYM_KEY32 = int64_t(1) << 21;
 constexpr int HUB_THREADS = 1024;
 constexpr int SYM_MAX_K = 512;
 constexpr int64_t HUB_COLS = int64_t(1) << 19;   // columns per bitmap (64 KB, and as much for its prefix sums)
@@ -416,7 +419,7 @@ atsne_status symmetrize_launch(const int32_t *idx, const float *P, int64_t N, in
                                int64_t *row_ptr, int32_t *col, float *val, int64_t *nnz_dev,
                                const SymWs &w, cudaStream_t stream) {
     if (k > SYM_MAX_K) return set_error(ATSNE_EUNSUPPORTED, "symmetrize: k=%d above %d", k, SYM_MAX_K);
-    if (N <= SYM_KEY32) return symmetrize_t<uint32_t>(idx, P, N, k, row_ptr, col, val, nnz_dev, w, stream);
+    if (N < SYM_KEY32) return symmetrize_t<uint32_t>(idx, P, N, k, row_ptr, col, val, nnz_dev, w, stream);
     return symmetrize_t<unsigned long long>(idx, P, N, k, row_ptr, col, val, nnz_dev, w, stream);
 }
 

@@ -84,3 +84,28 @@ def test_columns_beyond_32_bit_keys(at):
     s = torch.zeros(u.numel(), dtype=torch.float64, device="cuda").index_add_(0, inv, p) / (2 * N)
     assert torch.equal(col.long(), u % N) and torch.equal(rp[1:], (u // N).bincount(minlength=N).cumsum(0))
     assert ((val - s).abs().max() * N).item() <= 1e-5
+
+
+@pytest.mark.parametrize("N", [(1 << 21) - 1, 1 << 21, (1 << 21) + 5])
+def test_every_key_differs_from_the_mark_for_none(at, N):
+    # the largest column in the last slot of a row of 1024 entries, with 21
+    # column bits the largest key of all; and such rows with wider keys: four
+    # rows are listed by 1,020 others, row N - 1 (whose entry is placed last,
+    # or near it) among them
+    k = 4
+    i = torch.arange(N, device="cuda")
+    idx = torch.stack([(i + t) % N for t in range(1, k + 1)], 1)
+    at_row = torch.tensor([100000, 200000, 300000, 400000], device="cuda")
+    for t in range(4):
+        idx[500000 + 4 * t + 16 * torch.arange(1015, device="cuda"), 3] = at_row[t]
+    idx[N - 1] = at_row
+    P = torch.rand((N, k), device="cuda")
+    rp, col, val = at.atsne_symmetrize(idx.int().contiguous(), P)
+    at.atsne_check()
+    src = i.repeat_interleave(k)
+    assert torch.equal((idx.flatten() == at_row[:, None]).sum(1), torch.full((4,), 1024 - k, device="cuda"))
+    key = torch.cat([src * N + idx.flatten(), idx.flatten() * N + src])
+    u, inv = key.unique(return_inverse=True)
+    s = torch.zeros(u.numel(), dtype=torch.float64, device="cuda").index_add_(0, inv, P.double().flatten().repeat(2)) / (2 * N)
+    assert torch.equal(col.long(), u % N) and torch.equal(rp[1:], (u // N).bincount(minlength=N).cumsum(0))
+    assert ((val - s).abs().max() * N).item() <= 1e-5
