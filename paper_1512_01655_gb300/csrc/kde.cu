@@ -151,10 +151,12 @@ kde_kernel(const float2 *__restrict__ Y, int64_t N, const float *__restrict__ rh
                     const float fs = fy[j] * p.z, fr = fy[j] * p.w;
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
-                        const float ei = __fmaf_rn(dx[i], dx[i], dy2) <= r2 ? e[i] : 0.f;
-                        F[j][i] = fmaf(ei, fy[j], F[j][i]);
-                        S[j][i] = fmaf(ei, fs, S[j][i]);
-                        R[j][i] = fmaf(ei, fr, R[j][i]);
+                        // (left out, not added as 0: rho may be any value)
+                        if (__fmaf_rn(dx[i], dx[i], dy2) <= r2) {
+                            F[j][i] = fmaf(e[i], fy[j], F[j][i]);
+                            S[j][i] = fmaf(e[i], fs, S[j][i]);
+                            R[j][i] = fmaf(e[i], fr, R[j][i]);
+                        }
                     }
                 }
             }

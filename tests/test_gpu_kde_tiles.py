@@ -34,3 +34,28 @@ def test_kde_tile_and_chunk_edges(N, W, H, cutoff, sorted_by):
     live = of > 1e-9
     for u, v in ((gs, os_), (ga, oa), (gal, oal)):
         assert np.abs(u - v)[live].max(initial=0.0) <= 1e-5
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_a_precision_out_of_reach_does_not_count(bad):
+    # a point's rho enters the pixels within cutoff * h of it and no other, whatever its value
+    import paper_1512_01655_gb300 as at
+    rng = np.random.default_rng(7)
+    N, W, H, h, cutoff, px = 2000, 70, 50, 0.3, 2.0, 0.1
+    Y = (rng.random((N, 2)) * [7.0, 5.0]).astype(np.float32)
+    rho = rng.random(N).astype(np.float32)
+    Y[11] = (3.02, 2.04)
+    args = (0.0, 0.0, px, W, H, h)
+    a0 = at.atsne_kde_map(torch.from_numpy(Y).cuda(), *args, cutoff=cutoff, rho=torch.from_numpy(rho).cuda())[2].cpu().numpy()
+    rho[11] = bad
+    a1 = at.atsne_kde_map(torch.from_numpy(Y).cuda(), *args, cutoff=cutoff, rho=torch.from_numpy(rho).cuda())[2].cpu().numpy()
+    # the decision as the interface states it: centres and distances in FP32, each operation rounded once
+    f = np.float32
+    cx = (np.arange(W, dtype=np.float64) + 0.5) * float(f(px))
+    cy = (np.arange(H, dtype=np.float64) + 0.5) * float(f(px))
+    dx, dy = (cx.astype(f) - Y[11, 0]).astype(f), (cy.astype(f) - Y[11, 1]).astype(f)
+    d2 = (dx.astype(np.float64)[None, :] ** 2 + (dy * dy).astype(np.float64)[:, None]).astype(f)
+    r = f(cutoff) * f(h)
+    near = d2 <= r * r
+    assert near.any() and not np.isfinite(a1[near]).any()
+    assert np.array_equal(a1[~near], a0[~near])
