@@ -105,10 +105,9 @@ atsne_status calibrate_launch(const float *d2, int64_t rows, int k, float perple
 
 // ---- symmetrize -------------------------------------------------------------
 struct SymWs {
-    int2 *rev = nullptr;       // reverse lists: source rows and their conditionals, [N * k]
-    int32_t *rank = nullptr;   // each entry's place in its reverse list (in tcol's memory)
-    int32_t *tcol = nullptr;   // the union's rows before they move to row_ptr's places, [2 N k]
-    float *tval = nullptr;
+    int2 *rev = nullptr;       // reverse lists: source rows and their conditionals, [N * k]; then the union's rows
+    int2 *tail = nullptr;      // and what of them does not fit their reverse lists' places, [N][k]
+    int32_t *rank = nullptr;   // each entry's place in its reverse list (in tail's memory)
     int32_t *rcnt = nullptr, *len = nullptr, *mid_rows = nullptr, *hub_rows = nullptr, *n_list = nullptr;
     int64_t *roff = nullptr, *rtot = nullptr;  // reverse list offsets [N + 1], total
     int64_t *scan = nullptr;

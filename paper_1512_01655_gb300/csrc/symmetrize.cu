@@ -11,14 +11,17 @@
 //   2. scan:  offsets of the reverse lists.
 //   3. place: (i, p_{j|i}) written to that place, one 8-byte write per entry.
 //   4. merge: row r's k + |R_r| entries sorted by column, mutual pairs added,
-//             the row written to the workspace (its place there, r k + the
-//             reverse offset, does not depend on the lengths) and its length
-//             kept. Three classes of rows: up to 512 entries a warp sorts them
-//             in registers (sym_merge_kernel), up to 1024 the same with more
-//             registers (sym_mid_kernel), beyond that (hub rows) a CTA takes
-//             each entry's rank from a bitmap of the columns (sym_hub_kernel).
+//             the row kept in the workspace (its first |R_r| entries in its
+//             reverse list's place, which it has read, the up to k others in k
+//             places of its own) and its length kept. Rows of up to 512 entries
+//             are sorted by a warp in registers (sym_merge_kernel), up to 1024
+//             the same with more registers (sym_mid_kernel); of longer ones (hub
+//             rows) only the length is taken, |F_r| + |R_r| less the neighbours
+//             that list r.
 //   5. scan:  row_ptr.
-//   6. copy:  rows to their final places, scaled by 1 / 2N.
+//   6. copy:  rows to their final places, scaled by 1 / 2N; a hub row is written
+//             there by a CTA that takes each entry's rank from a bitmap of the
+//             columns (sym_hub_kernel).
 // A warp's sort moves one word per entry: column, forward/reverse bit and the
 // entry's slot (where its value waits in shared memory) in 32 bits while the
 // column fits (N < 2^21), else 64; a compare-exchange is a shuffle and a
@@ -140,9 +143,8 @@ struct SymRow {
     int64_t N;
     int k;
     const int64_t *roff;
-    const int2 *rev;
-    int32_t *tcol;  // the rows of the union in the workspace, values not yet scaled
-    float *tval;
+    int2 *rev;   // reverse lists (column, value); then the first entries of the union's rows, not yet scaled
+    int2 *tail;  // their other entries, [N][k]
     int32_t *len;
     int *status;
 };
@@ -210,12 +212,8 @@ __device__ __forceinline__ void sym_merge_row(const SymRow &s, int64_t r, int m,
         }
     }
     __syncwarp();
-    int32_t *tc = s.tcol + row + b0;
-    float *tv = s.tval + row + b0;
-    for (int t = lane; t < total; t += 32) {
-        tc[t] = oc[t];
-        tv[t] = ov[t];
-    }
+    int2 *first = s.rev + b0, *rest = s.tail + (row - m);
+    for (int t = lane; t < total; t += 32) (t < m ? first : rest)[t] = make_int2(oc[t], __float_as_int(ov[t]));
     if (lane == 0) s.len[r] = total;
 }
 
@@ -230,8 +228,12 @@ sym_merge_kernel(SymRow s, int32_t *__restrict__ mid_rows, int32_t *__restrict__
     const int64_t m64 = s.roff[r + 1] - s.roff[r];
     if (m64 + s.k > SYM_BULK) {
         if (lane == 0) {
-            if (m64 + s.k > SYM_MID) hub_rows[atomicAdd(n_list + 1, 1)] = (int)r;
-            else mid_rows[atomicAdd(n_list, 1)] = (int)r;
+            if (m64 + s.k > SYM_MID) {
+                hub_rows[atomicAdd(n_list + 1, 1)] = (int)r;
+                s.len[r] = (int)m64;  // the forward entries follow in sym_mid_kernel
+            } else {
+                mid_rows[atomicAdd(n_list, 1)] = (int)r;
+            }
         }
         return;
     }
@@ -244,7 +246,8 @@ sym_merge_kernel(SymRow s, int32_t *__restrict__ mid_rows, int32_t *__restrict__
 
 template <typename K>
 __global__ void __launch_bounds__(SYM_WARPS * 32)
-sym_mid_kernel(SymRow s, const int32_t *__restrict__ mid_rows, const int32_t *__restrict__ n_list) {
+sym_mid_kernel(SymRow s, const int32_t *__restrict__ mid_rows, const int32_t *__restrict__ hub_rows,
+               const int32_t *__restrict__ n_list) {
     __shared__ float v[SYM_WARPS][SYM_MID], ov[SYM_WARPS][SYM_MID];
     __shared__ int oc[SYM_WARPS][SYM_MID];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -253,14 +256,32 @@ sym_mid_kernel(SymRow s, const int32_t *__restrict__ mid_rows, const int32_t *__
         sym_merge_row<32, K>(s, r, (int)(s.roff[r + 1] - s.roff[r]), v[w], oc[w], ov[w], lane);
         __syncwarp();
     }
+    // the hub rows' lengths: eight lanes per forward entry, which adds one to its
+    // row's reverse entries unless its column lists the row (and is among them)
+    const int64_t items = (int64_t)n_list[1] * s.k;
+    const int gl = lane & 7;
+    const unsigned group = 0xffu << (lane & 24);
+    for (int64_t q = (int64_t)(blockIdx.x * SYM_WARPS + w) * 4 + (lane >> 3); q < items;
+         q += (int64_t)gridDim.x * SYM_WARPS * 4) {
+        const int64_t r = hub_rows[q / s.k];
+        const int c = s.idx[r * s.k + q % s.k];
+        if (c < 0 || c >= s.N || c == r) continue;
+        const int32_t *row = s.idx + (int64_t)c * s.k;
+        bool mutual = false;
+#pragma unroll 4
+        for (int t = gl; t < s.k; t += 8) mutual |= row[t] == r;
+        if (!__any_sync(group, mutual) && gl == 0) atomicAdd(&s.len[r], 1);
+    }
 }
 
-// Hub rows, one CTA each: a bitmap of the columns of the union gives every
-// entry its place (bits below it), HUB_COLS columns at a time. The reverse
-// entries are set first, so a forward entry that finds its bit set is mutual;
-// it adds its value to the one its partner has written.
+// Hub rows, one CTA each, written to their places in the CSR: a bitmap of the
+// columns of the union gives every entry its place (bits below it), HUB_COLS
+// columns at a time. The reverse entries are set first, so a forward entry that
+// finds its bit set is mutual; it adds its value to the one its partner has
+// written. The range's values are then scaled.
 __global__ void __launch_bounds__(HUB_THREADS)
-sym_hub_kernel(SymRow s, const int32_t *__restrict__ hub_rows, const int32_t *__restrict__ n_list, int words) {
+sym_hub_kernel(SymRow s, const int32_t *__restrict__ hub_rows, const int32_t *__restrict__ n_list, int words,
+               float inv2n, const int64_t *__restrict__ row_ptr, int32_t *col, float *val) {
     extern __shared__ uint32_t hub_smem[];
     uint32_t *bits = hub_smem, *below = hub_smem + words;  // below: set bits before each word, in this range
     __shared__ int wsum[HUB_THREADS / 32], wbase[HUB_THREADS / 32 + 1];
@@ -269,8 +290,8 @@ sym_hub_kernel(SymRow s, const int32_t *__restrict__ hub_rows, const int32_t *__
     const int per = (words + HUB_THREADS - 1) / HUB_THREADS * 32;
     for (int q = blockIdx.x; q < n_list[1]; q += gridDim.x) {
         const int64_t r = hub_rows[q], b0 = s.roff[r], m = s.roff[r + 1] - b0, row = r * s.k;
-        int32_t *tc = s.tcol + row + b0;
-        float *tv = s.tval + row + b0;
+        int32_t *tc = col + row_ptr[r];
+        float *tv = val + row_ptr[r];
         int64_t done = 0;  // entries of the ranges before
         for (int64_t c0 = 0; c0 < s.N; c0 += (int64_t)words * 32) {
             const int64_t c1 = min(s.N, c0 + (int64_t)words * 32);
@@ -344,24 +365,39 @@ sym_hub_kernel(SymRow s, const int32_t *__restrict__ hub_rows, const int32_t *__
                 tc[at] = (int)fc;
                 tv[at] = mutual ? p + tv[at] : p;
             }
-            done += wbase[HUB_THREADS / 32];
             __syncthreads();
+            const int64_t end = done + wbase[HUB_THREADS / 32];
+            for (int64_t t = done + tid; t < end; t += HUB_THREADS) tv[t] *= inv2n;
+            done = end;
         }
-        if (tid == 0) s.len[r] = (int)done;
     }
 }
 
 __global__ void __launch_bounds__(256)
-sym_copy_kernel(const int32_t *__restrict__ tcol, const float *__restrict__ tval, int64_t N, int k, float inv2n,
+sym_copy_kernel(const int2 *__restrict__ rev, const int2 *__restrict__ tail, int64_t N, int k, float inv2n,
                 const int64_t *__restrict__ roff, const int64_t *__restrict__ row_ptr, int32_t *__restrict__ col,
                 float *__restrict__ val) {
     const int lane = threadIdx.x & 31;
     const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (r >= N) return;
-    const int64_t from = r * k + roff[r], to = row_ptr[r], n = row_ptr[r + 1] - to;
-    for (int64_t t = lane; t < n; t += 32) {
-        col[to + t] = tcol[from + t];
-        val[to + t] = tval[from + t] * inv2n;
+    const int64_t b0 = roff[r], m = roff[r + 1] - b0, to = row_ptr[r], n = row_ptr[r + 1] - to;
+    if (m + k > SYM_MID) return;  // a hub row, written in its place
+    const int2 *first = rev + b0, *rest = tail + (r * k - m);
+    for (int t0 = lane; t0 < n; t0 += 128) {  // four loads in flight per lane
+        int2 e[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int t = t0 + 32 * u;
+            if (t < n) e[u] = (t < m ? first : rest)[t];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int t = t0 + 32 * u;
+            if (t < n) {
+                col[to + t] = e[u].x;
+                val[to + t] = __int_as_float(e[u].y) * inv2n;
+            }
+        }
     }
 }
 
@@ -379,20 +415,22 @@ atsne_status symmetrize_t(const int32_t *idx, const float *P, int64_t N, int k, 
     ATSNE_TRY(scan_rowlen(w.rcnt, N, 0, w.roff, w.rtot, w.scan, stream));
     ATSNE_TRY(launch_kernel("sym_place", sym_place_kernel, row_blocks, 256, 0, stream, idx, P, N, k,
                             (const int32_t *)w.rank, (const int64_t *)w.roff, w.rev));
-    const SymRow s{idx, P, N, k, w.roff, w.rev, w.tcol, w.tval, w.len, status};
+    const SymRow s{idx, P, N, k, w.roff, w.rev, w.tail, w.len, status};
     ATSNE_TRY(launch_kernel("sym_merge", sym_merge_kernel<K>, ceil_div(N, SYM_WARPS), SYM_WARPS * 32, 0, stream, s,
                             w.mid_rows, w.hub_rows, w.n_list));
     ATSNE_TRY(launch_kernel("sym_mid", sym_mid_kernel<K>, (int)hmin(4 * num_sms(), ceil_div(N, SYM_WARPS)),
-                            SYM_WARPS * 32, 0, stream, s, (const int32_t *)w.mid_rows, (const int32_t *)w.n_list));
+                            SYM_WARPS * 32, 0, stream, s, (const int32_t *)w.mid_rows, (const int32_t *)w.hub_rows,
+                            (const int32_t *)w.n_list));
+    ATSNE_TRY(scan_rowlen(w.len, N, 0, row_ptr, nnz_dev, w.scan, stream));
     const int words = (int)((hmin(N, HUB_COLS) + 31) / 32);
     const size_t smem = (size_t)words * 8;
     e = cudaFuncSetAttribute(sym_hub_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_error(e, "sym_hub attribute");
     ATSNE_TRY(launch_kernel("sym_hub", sym_hub_kernel, (int)hmin(4 * num_sms(), N), HUB_THREADS, smem, stream, s,
-                            (const int32_t *)w.hub_rows, (const int32_t *)w.n_list, words));
-    ATSNE_TRY(scan_rowlen(w.len, N, 0, row_ptr, nnz_dev, w.scan, stream));
-    return launch_kernel("sym_copy", sym_copy_kernel, row_blocks, 256, 0, stream, (const int32_t *)w.tcol,
-                         (const float *)w.tval, N, k, inv2n, (const int64_t *)w.roff, (const int64_t *)row_ptr, col, val);
+                            (const int32_t *)w.hub_rows, (const int32_t *)w.n_list, words, inv2n,
+                            (const int64_t *)row_ptr, col, val));
+    return launch_kernel("sym_copy", sym_copy_kernel, row_blocks, 256, 0, stream, (const int2 *)w.rev,
+                         (const int2 *)w.tail, N, k, inv2n, (const int64_t *)w.roff, (const int64_t *)row_ptr, col, val);
 }
 
 }  // namespace
@@ -400,9 +438,8 @@ atsne_status symmetrize_t(const int32_t *idx, const float *P, int64_t N, int k, 
 size_t symmetrize_workspace(Carver &c, int64_t N, int k, SymWs *ws) {
     SymWs w;
     w.rev = c.take<int2>((size_t)N * k);
-    w.tcol = c.take<int32_t>((size_t)2 * N * k);
-    w.rank = w.tcol;  // read by the placement, before the merge writes
-    w.tval = c.take<float>((size_t)2 * N * k);
+    w.tail = c.take<int2>((size_t)N * k);
+    w.rank = reinterpret_cast<int32_t *>(w.tail);  // read by the placement, before the merge writes
     w.rcnt = c.take<int32_t>((size_t)N);
     w.len = c.take<int32_t>((size_t)N);
     w.roff = c.take<int64_t>((size_t)N + 1);
