@@ -31,7 +31,7 @@ struct TcPlan {
     // adaptive launch over the rows it gives up
     bool filter = false;
     int S = 0, blk = 0, rank = 0, rank2 = 0;     // sampled rows, columns per block, the thresholds' ranks
-    int fsplits = 1, fcols = 0, fcap = 0, fkeys = 0;  // fkeys: keys a row is expected to buffer
+    int fsplits = 1, fcap = 0, fkeys = 0;  // fkeys: keys a row is expected to buffer
 };
 // Row and column order of a large self kNN (points grouped by nearest
 // centroid; each row tile streams its own groups' column tiles first).

@@ -106,7 +106,7 @@ struct FParams {
     const int64_t *qcount;   // if given, the rows in use (device; at most Q)
     int64_t Q, N;
     int KB, last_steps;      // k-blocks; K = 16 steps of the last one
-    int splits, cols_per_split;
+    int splits;              // split sp takes the column tiles sp, sp + splits, ...
     int cap;
     Cand *cand;              // [Q][splits * F_PARTS][cap]
     int4 *meta;
@@ -163,6 +163,7 @@ knn_filter_kernel(const __grid_constant__ FParams p) {
     const int pairs = (int)((Q + 2 * F_BM - 1) / (2 * F_BM));
     const int64_t n_units = (int64_t)pairs * p.splits;
     const int64_t u0 = blockIdx.x >> 1, ustep = gridDim.x >> 1;
+    const int64_t cstep = (int64_t)p.splits * F_BN;
     // an expired wait stops both CTAs' roles at their next wait
     auto give_up = [&]() {
         s.abort_flag = 1;
@@ -185,9 +186,7 @@ knn_filter_kernel(const __grid_constant__ FParams p) {
             for (int64_t u = u0; u < n_units && ok; u += ustep) {
                 const int pt = (int)(u % pairs), sp = (int)(u / pairs);
                 const int ar = (2 * pt + (int)rank) * F_BM;
-                const int64_t c0 = (int64_t)sp * p.cols_per_split;
-                const int64_t c1 = min(p.N, c0 + p.cols_per_split);
-                for (int64_t ct = c0; ct < c1 && ok; ct += F_BN) {
+                for (int64_t ct = (int64_t)sp * F_BN; ct < p.N && ok; ct += cstep) {
                     const int br = (int)ct + (int)rank * F_BH;
                     for (int kb = 0; kb < p.KB; ++kb) {
                         if (!mbar_wait(&s.empty[stage], phase ^ 1u, &s.abort_flag, p.wait_ns)) {
@@ -232,9 +231,7 @@ knn_filter_kernel(const __grid_constant__ FParams p) {
             if (C::FOLD) ok = __all_sync(0xffffffffu, mbar_wait(&s.ext_bar, 0, &s.abort_flag, p.wait_ns));
             for (int64_t u = u0; u < n_units && ok; u += ustep) {
                 const int sp = (int)(u / pairs);
-                const int64_t c0 = (int64_t)sp * p.cols_per_split;
-                const int64_t c1 = min(p.N, c0 + p.cols_per_split);
-                for (int64_t ct = c0; ct < c1 && ok; ct += F_BN) {
+                for (int64_t ct = (int64_t)sp * F_BN; ct < p.N && ok; ct += cstep) {
                     ok = __all_sync(0xffffffffu,
                                     mbar_wait(&s.acc_empty[acc], acc_phase ^ 1u, &s.abort_flag, p.wait_ns));
                     if (!ok) break;
@@ -296,8 +293,7 @@ knn_filter_kernel(const __grid_constant__ FParams p) {
         bool ok = true;
         for (int64_t u = u0; u < n_units && ok; u += ustep) {
             const int pt = (int)(u % pairs), sp = (int)(u / pairs);
-            const int64_t c0 = (int64_t)sp * p.cols_per_split;
-            const int64_t c1 = min(p.N, c0 + p.cols_per_split);
+            const int64_t c0 = (int64_t)sp * F_BN;
             const int64_t row = ((int64_t)2 * pt + rank) * F_BM + quarter * 32 + lane;
             const bool live = row < Q;
             // survivors are the values v above thr: v = x.y - ||y||^2/2 with
@@ -323,17 +319,17 @@ knn_filter_kernel(const __grid_constant__ FParams p) {
 #pragma unroll
                 for (int q = 0; q < C::NCH; ++q) {
                     const int64_t cc = c0 + part * C::CW + q * 32 + lane;
-                    nyn[q] = cc < c1 ? -p.nrm[cc] : -INFINITY;
+                    nyn[q] = cc < p.N ? -p.nrm[cc] : -INFINITY;
                 }
             }
-            for (int64_t ct = c0; ct < c1; ct += F_BN) {
+            for (int64_t ct = c0; ct < p.N; ct += cstep) {
                 float nyc[C::NCH];
                 if (!C::FOLD) {
 #pragma unroll
                     for (int q = 0; q < C::NCH; ++q) {
                         nyc[q] = nyn[q];
-                        const int64_t cc = ct + F_BN + part * C::CW + q * 32 + lane;
-                        nyn[q] = cc < c1 ? -p.nrm[cc] : -INFINITY;
+                        const int64_t cc = ct + cstep + part * C::CW + q * 32 + lane;
+                        nyn[q] = cc < p.N ? -p.nrm[cc] : -INFINITY;
                     }
                 }
                 ok = mbar_wait(&s.acc_full[acc], acc_phase, &s.abort_flag, p.wait_ns);
@@ -401,7 +397,7 @@ knn_filter_kernel(const __grid_constant__ FParams p) {
                             if (c + 1 == C::NCH && live) mrow[colb0 / C::CW] = pm;
                         }
                     } else if (__any_sync(0xffffffffu, gm > thr)) {
-                        // a buffer without room for the chunk is closed (the row is given up)
+                        // a buffer without room for the chunk's survivors is closed (the row is given up)
                         if (cnt > p.cap - 32) {
                             thr = INFINITY;
                             full = 1;
@@ -624,14 +620,11 @@ atsne_status f_launch(const FParams &p, int64_t units, cudaStream_t stream) {
 // split costs the fixed threshold nothing but a few more (shorter) buffers per
 // row, so it is chosen for the last wave: the fewest splits whose critical path
 // (waves of units, each its tiles and about two tiles of start-up) is within 2%
-// of the shortest found.
+// of the shortest found. The splits take the tiles in turn, so that neighbours
+// that follow one another in the corpus (sorted by class) spread over them.
 int filter_splits(int64_t Qp, int64_t tiles, int max_splits) {
     const int64_t C = num_sms() / 2 > 0 ? num_sms() / 2 : 1;
-    auto cost = [&](int64_t s) {
-        const int64_t per = (tiles + s - 1) / s;
-        const int64_t used = (tiles + per - 1) / per;
-        return (double)((Qp * used + C - 1) / C) * (double)(per + 2);
-    };
+    auto cost = [&](int64_t s) { return (double)((Qp * s + C - 1) / C) * (double)((tiles + s - 1) / s + 2); };
     double best = cost(1);
     for (int s = 2; s <= max_splits && s <= tiles; ++s) best = fmin(best, cost(s));
     for (int s = 1; s <= max_splits && s <= tiles; ++s)
@@ -662,8 +655,6 @@ atsne_status knn_filter_launch(const TcPlan &pl, const TcWs &w, const FilterArgs
         ATSNE_TRY(tc_map_ext(&p.tm_b_ext, w.sext, pl.S, F_BH));
         p.N = pl.S;
         p.splits = filter_splits(pairs, pl.S / F_BN, 16);
-        p.cols_per_split = (pl.S / F_BN + p.splits - 1) / p.splits * F_BN;
-        p.splits = (pl.S + p.cols_per_split - 1) / p.cols_per_split;
         p.minima = w.minima;
         p.m = pl.S / pl.blk;
         p.blk = pl.blk;
@@ -693,7 +684,6 @@ atsne_status knn_filter_launch(const TcPlan &pl, const TcWs &w, const FilterArgs
     p.nrm = w.nrm;
     p.tau = w.tau;
     p.splits = pl.fsplits;
-    p.cols_per_split = pl.fcols;
     p.cap = pl.fcap;
     p.cand = reinterpret_cast<Cand *>(w.cand);
     p.meta = reinterpret_cast<int4 *>(w.meta);

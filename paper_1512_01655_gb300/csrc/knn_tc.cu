@@ -1998,7 +1998,7 @@ int tc_splits(const TcPlan &pl) { return pl.filter ? pl.fsplits : pl.splits; }
 static void plan_filter(TcPlan &pl, int64_t N, int64_t Q, int splits) {
     const int64_t pairs = (Q + 2 * TC_BM - 1) / (2 * TC_BM);
     const int64_t col_tiles = (N + TC_BN - 1) / TC_BN;
-    const int cw = TC_BN / F_PARTS;
+    const int cw = TC_BN / F_PARTS;  // columns of a part
     if (N < FILTER_MIN_ROWS) return;
     // S rows, about 32 sqrt(N): the sample's pass and what the thresholds let
     // through then cost about the same
@@ -2034,14 +2034,30 @@ static void plan_filter(TcPlan &pl, int64_t N, int64_t Q, int splits) {
     if (splits <= 0) splits = filter_splits(pairs, col_tiles, 64);
     if (splits > 64) splits = 64;
     if (splits > col_tiles) splits = (int)col_tiles;
-    const int64_t per = (col_tiles + splits - 1) / splits;
-    pl.fcols = (int)(per * TC_BN);
-    pl.fsplits = (int)((N + pl.fcols - 1) / pl.fcols);
-    // a row's neighbours may all lie in one split (a corpus sorted by class),
-    // but spread over the parts of its tiles
+    pl.fsplits = splits;
     pl.fkeys = (int)expect;
-    int64_t cap = (int64_t)ceil(2.0 * expect / F_PARTS) + 48;
-    if (cap > per * cw) cap = per * cw;
+}
+
+// The fixed threshold's buffers: twice a part's share of the keys a row is
+// expected to keep. They spread over a row's splits and the parts of its tiles,
+// unless its neighbours all lie in one part (a corpus whose classes repeat every
+// 256 rows). Where the rows keep their order (knn_order.cu regroups those of
+// large sets) a buffer then holds its share of one part, and more by the spread
+// of a threshold taken from r sampled keys, as far as the adaptive launch's
+// buffers, whose memory these take, leave room. 60,000 x 32, four clusters in turn
+// in blocks of 64 rows: with every row given up after the filter had run 4.4 ms
+// (FP32) and 13.5 ms (BF16 approximate), now 1.5 and 2.1 ms; the same rows
+// shuffled 2.0 and 2.6 ms.
+static void plan_buffers(TcPlan &pl, int64_t N, bool ordered) {
+    const int64_t per = ((N + TC_BN - 1) / TC_BN + pl.fsplits - 1) / pl.fsplits * (TC_BN / F_PARTS);  // columns of a buffer
+    int64_t cap = (pl.fkeys + 1) / 2 + 48;
+    if (!ordered) {
+        const double r = (double)pl.fkeys * pl.S / (double)N;
+        const int64_t part = (int64_t)ceil(pl.fkeys * (1.0 + 2.0 / sqrt(r)) / pl.fsplits) + 48;
+        const int64_t room = (int64_t)pl.splits * pl.halves * pl.cap / (pl.fsplits * F_PARTS);
+        if (cap < part) cap = part < room ? part : cap < room ? room : cap;
+    }
+    if (cap > per) cap = per;
     pl.fcap = (int)((cap + 15) / 16 * 16);
 }
 
@@ -2086,6 +2102,7 @@ TcPlan tc_plan(int64_t N, int D, int64_t Q, int k, int precision, int rerank_k, 
     // the epilogue's bucket counts are 16 bits and never exceed the buffer's size
     if (cap > 65504) cap = 65504;
     pl.cap = (int)((cap + 31) / 32 * 32);
+    if (pl.filter) plan_buffers(pl, N, knn_ordered(N, D, Q != N, pl));
     return pl;
 }
 
@@ -2097,8 +2114,7 @@ TcPlan tc_plan_radius(int64_t N, int D, int64_t Q, int k, int precision, int rer
     const int s = filter_splits((Q + 2 * TC_BM - 1) / (2 * TC_BM), col_tiles, 64);
     pl.filter = true;
     pl.S = 0;
-    pl.fcols = (int)((col_tiles + s - 1) / s * TC_BN);
-    pl.fsplits = (int)((N + pl.fcols - 1) / pl.fcols);
+    pl.fsplits = s;
     pl.fcap = RADIUS_CAP;
     return pl;
 }

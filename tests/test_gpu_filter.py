@@ -84,3 +84,36 @@ def test_queries_from_another_array(at, Nq, Nc):
     assert torch.equal(i, ri) and torch.equal(d.isinf(), rd.isinf())
     fin = ~d.isinf()
     assert ((d[fin] - rd[fin]).abs() <= 16 * 2.0 ** -24 * rd[fin]).all()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "bf16_approx"])
+def test_neighbours_all_in_one_part_of_the_tiles(at, precision):
+    # four clusters in turn, 64 rows each, over 2,048 rows: a row's neighbours
+    # all pass through one buffer. The rows are kept, not given up: the call
+    # takes no longer than the same rows in random order (measured 0.7 and 0.8
+    # times; 2.2 and 5.3 times where every row was given up)
+    N, D, k = 60000, 32, 90
+    g = torch.Generator(device="cuda").manual_seed(3)
+    i = torch.arange(N, device="cuda")
+    c = (i // 2048) * 4 + (i // 64) % 4
+    X = (4 * torch.randn((int(c.max()) + 1, D), generator=g, device="cuda"))[c] + torch.randn((N, D), generator=g, device="cuda")
+    Y = X[torch.randperm(N, generator=g, device="cuda")].contiguous()
+
+    def ms(A):
+        best = float("inf")
+        for _ in range(4):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            at.atsne_knn(A, k, precision=precision)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        return best
+
+    assert ms(X) <= 1.6 * ms(Y)
+    if precision == "fp32":
+        q = torch.arange(0, N, 601, dtype=torch.int32, device="cuda")
+        ri, rd = at.atsne_knn(X, k + 1, queries=q, precision="fp32_cuda")
+        ti, td = at.atsne_knn(X, k)
+        at.atsne_check()
+        assert torch.equal(ti[q.long()], ri[:, :k]) and torch.equal(td[q.long()], rd[:, :k])
