@@ -207,7 +207,7 @@ size_t knn_ws(Carver &c, int64_t N, int32_t D, int32_t k, int64_t S, const atsne
               TcWs *tws = nullptr) {
     if (exact_on_tensor_cores(o, k)) {
         const int64_t Q = S > 0 ? S : N;
-        const TcPlan pl = tc_plan(N, D, Q, k, o.precision, o.rerank_k);
+        const TcPlan pl = tc_plan(N, D, Q, S > 0, k, o.precision, o.rerank_k);
         if (plan) *plan = pl;
         tc_workspace(c, N, D, Q, S > 0, pl, tws);
     }
@@ -251,7 +251,7 @@ size_t refine_ws(Carver &c, int64_t N, int32_t D, int64_t S, int32_t k, int32_t 
     if (tb) *tb = q;
     if (hint) *hint = h;
     if (S >= REFINE_TC_MIN_ROWS && k <= 200) {
-        const TcPlan pl = tc_plan(N, D, S, k, ATSNE_FP32, 0);
+        const TcPlan pl = tc_plan(N, D, S, true, k, ATSNE_FP32, 0);
         if (plan) *plan = pl;
         tc_workspace(c, N, D, S, true, pl, tws);
     }
@@ -263,7 +263,7 @@ size_t cross_ws(Carver &c, int64_t Nq, int64_t Nc, int32_t D, int32_t k, const a
                 bool radius, TcPlan *plan, TcWs *tws) {
     if (exact_on_tensor_cores(o, k) && Nq > 0 && !(radius && o.precision == ATSNE_FP8_RERANK)) {
         const TcPlan pl = radius ? tc_plan_radius(Nc, D, Nq, k, o.precision, o.rerank_k)
-                                 : tc_plan(Nc, D, Nq, k, o.precision, o.rerank_k);
+                                 : tc_plan(Nc, D, Nq, true, k, o.precision, o.rerank_k);
         if (plan) *plan = pl;
         tc_workspace(c, Nc, D, Nq, true, pl, tws);
     }
@@ -276,12 +276,12 @@ size_t tune_ws(int64_t N, int32_t D, int32_t k, int64_t S, const atsne_knn_opts 
     const int64_t Q = S > 0 ? S : N;
     int c_[TUNE_MAX_CAND];
     int *cs = cand ? cand : c_;
-    const int n = tc_split_candidates(N, D, Q, k, o.precision, o.rerank_k, cs, TUNE_MAX_CAND);
+    const int n = tc_split_candidates(N, D, Q, S > 0, k, o.precision, o.rerank_k, cs, TUNE_MAX_CAND);
     if (n_cand) *n_cand = n;
     size_t need = 0;
     for (int i = 0; i < n; ++i) {
         Carver c(nullptr);
-        tc_workspace(c, N, D, Q, S > 0, tc_plan(N, D, Q, k, o.precision, o.rerank_k, cs[i]), nullptr);
+        tc_workspace(c, N, D, Q, S > 0, tc_plan(N, D, Q, S > 0, k, o.precision, o.rerank_k, cs[i]), nullptr);
         if (c.bytes() > need) need = c.bytes();
     }
     return need;
@@ -290,15 +290,13 @@ size_t tune_ws(int64_t N, int32_t D, int32_t k, int64_t S, const atsne_knn_opts 
 // Batched refinement: the union's rows (padded to min(N, total)), its bitmap,
 // then the refinement of that many rows.
 size_t refine_batch_ws(Carver &c, int64_t N, int32_t D, int64_t total, int32_t k, int32_t **rows,
-                       uint32_t **bitmap, int64_t **count, int32_t **ti, float **td, float **tp, float **tb,
+                       uint32_t **bitmap, int32_t **ti, float **td, float **tp, float **tb,
                        TcPlan *plan, TcWs *tws, float **hint = nullptr) {
     const int64_t rows_max = total < N ? total : N;
     int32_t *r = c.take<int32_t>((size_t)(rows_max > 0 ? rows_max : 1));
     uint32_t *b = c.take<uint32_t>((size_t)((N + 31) / 32));
-    int64_t *n = c.take<int64_t>(1);
     if (rows) *rows = r;
     if (bitmap) *bitmap = b;
-    if (count) *count = n;
     return refine_ws(c, N, D, rows_max, k, ti, td, tp, tb, plan, tws, hint);
 }
 
@@ -428,7 +426,7 @@ size_t atsne_workspace_bytes(int32_t op, int64_t N, int32_t D, int32_t k, int64_
     case ATSNE_OP_KNN_CROSS_RADIUS:
         return cross_ws(c, S, N, D, k, o, true, nullptr, nullptr);
     case ATSNE_OP_REFINE_BATCH:
-        return refine_batch_ws(c, N, D, S, k, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
+        return refine_batch_ws(c, N, D, S, k, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
                                nullptr, nullptr);
     default:
         return 0;
@@ -494,7 +492,7 @@ atsne_status atsne_tune_knn(const float *X, int64_t N, int32_t D, const int32_t 
     int best = 0;
     float best_ms = FLT_MAX;
     for (int i = 0; i < n_cand && e == cudaSuccess && st == ATSNE_OK; ++i) {
-        const TcPlan pl = tc_plan(N, D, Q, k, o.precision, o.rerank_k, cand[i]);
+        const TcPlan pl = tc_plan(N, D, Q, queries != nullptr, k, o.precision, o.rerank_k, cand[i]);
         Carver c(workspace);
         TcWs w;
         tc_workspace(c, N, D, Q, queries != nullptr, pl, &w);
@@ -640,28 +638,29 @@ atsne_status atsne_refine_batch(const float *X, int64_t N, int32_t D, const int3
     Carver c(workspace);
     int32_t *rows, *ti;
     uint32_t *bitmap;
-    int64_t *count;
     float *td, *tp, *tb, *hint;
     TcPlan plan;
     TcWs tws;
-    refine_batch_ws(c, N, D, total, k, &rows, &bitmap, &count, &ti, &td, &tp, &tb, &plan, &tws, &hint);
+    refine_batch_ws(c, N, D, total, k, &rows, &bitmap, &ti, &td, &tp, &tb, &plan, &tws, &hint);
     if (!workspace || ws_bytes < c.bytes())
         return set_error(ATSNE_ENOMEM, "refine batch: workspace of %zu bytes, %zu needed", ws_bytes,
                          c.bytes());
     if ((st = check_base(workspace, "refine batch workspace"))) return st;
     if ((st = check_indices(lists, total, N, stream))) return st;
     const int64_t S = total < N ? total : N;
-    if ((st = union_launch(lists, total, N, bitmap, rows, S, count, stream))) return st;
-    if (refined_count) {
-        cudaError_t e = cudaMemcpyAsync(refined_count, count, sizeof(int64_t), cudaMemcpyDeviceToDevice, stream);
-        if (e != cudaSuccess) return cuda_error(e, "refine batch: count");
-    }
     // The rows past the union repeat its first one. The fixed-threshold search
     // and what follows it leave them out (64 selections of
     // 200 to 20,000 points of 500,000 x 256, about 250 K listed, 190 K distinct:
     // 106 to 78 ms).
     const int64_t *used = nullptr;
-    if (S >= REFINE_TC_MIN_ROWS && k <= 200) {  // the prep kernel checks X for non-finite values
+    const bool tensor = S >= REFINE_TC_MIN_ROWS && k <= 200;
+    int64_t *count = tensor && plan.filter ? tws.row_count : refined_count;
+    if ((st = union_launch(lists, total, N, bitmap, rows, S, count, stream))) return st;
+    if (refined_count && count != refined_count) {
+        cudaError_t e = cudaMemcpyAsync(refined_count, count, sizeof(int64_t), cudaMemcpyDeviceToDevice, stream);
+        if (e != cudaSuccess) return cuda_error(e, "refine batch: count");
+    }
+    if (tensor) {  // the prep kernel checks X for non-finite values
         used = plan.filter ? count : nullptr;
         if ((st = gather_hint_launch(rows, S, N, k, d2, hint, stream))) return st;
         if ((st = knn_exact_tc(X, N, D, rows, S, k, plan, tws, ti, td, stream, nullptr, nullptr, hint, used)))

@@ -27,6 +27,8 @@ struct TcPlan {
     int passes = 1, Dp = 0, row_tiles = 0, splits = 1, cols_per_split = 0, ksel = 0, cap = 0;
     int halves = 1;  // candidate buffers per (row, split): one per column half of a tile
     bool certify = true;  // rows certified exact (else the ksel best keys re-ranked, approximate)
+    int64_t rrows = 0;      // rows the adaptive launch takes
+    size_t cand_bytes = 0;  // the region of the launches' buffers
     // fixed thresholds (knn_filter.cu); the fields above then describe the
     // adaptive launch over the rows it gives up
     bool filter = false;
@@ -56,6 +58,8 @@ struct TcWs {
     float *scale = nullptr, *qscale = nullptr;  // FP8 row scales
     float *qnrm = nullptr, *qstats = nullptr;   // queries from another array: norms, error stats
     int32_t *flag_rows = nullptr, *flag_count = nullptr;
+    int64_t *row_count = nullptr;               // for a caller's count of the rows in use
+    int64_t ext_rows = 0;                       // rows of bext
     uint16_t *bext = nullptr, *aext = nullptr;  // one-pass BF16: the norm slices
     bool ordered = false;                       // rows and columns in the order of OrderWs
     unsigned long long *clock = nullptr;        // one split: tiles issued by all CTAs
@@ -71,15 +75,17 @@ uint64_t pipeline_wait_ns();
 void set_pipeline_wait_ns(uint64_t ns);
 // splits > 0 forces the column split count; 0: the one atsne_tune_knn recorded
 // for this shape, else the rule; < 0: the rule.
-TcPlan tc_plan(int64_t N, int D, int64_t Q, int k, int precision, int rerank_k, int splits = 0);
+// list: the query rows are listed, or from another array.
+TcPlan tc_plan(int64_t N, int D, int64_t Q, bool list, int k, int precision, int rerank_k, int splits = 0);
 TcPlan tc_plan_radius(int64_t N, int D, int64_t Q, int k, int precision, int rerank_k);
 int tc_splits(const TcPlan &pl);  // the plan's column splits (the tunable)
+double filter_path(int64_t row_pairs, int64_t col_tiles, int splits);
 int filter_splits(int64_t row_pairs, int64_t col_tiles, int max_splits);
 int tuned_splits(int64_t N, int D, int64_t Q, int k, int precision, int rerank_k);
 void set_tuned_splits(int64_t N, int D, int64_t Q, int k, int precision, int rerank_k, int splits);
 void clear_tuned_splits();
 // Distinct column split counts worth timing for a shape (at most max_out).
-int tc_split_candidates(int64_t N, int D, int64_t Q, int k, int precision, int rerank_k, int *out, int max_out);
+int tc_split_candidates(int64_t N, int D, int64_t Q, bool list, int k, int precision, int rerank_k, int *out, int max_out);
 size_t tc_workspace(Carver &c, int64_t N, int D, int64_t Q, bool list, const TcPlan &pl, TcWs *ws);
 bool knn_ordered(int64_t N, int D, bool list, const TcPlan &pl);
 size_t order_workspace(Carver &c, int64_t N, int D, const TcPlan &pl, OrderWs *ws);

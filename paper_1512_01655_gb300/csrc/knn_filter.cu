@@ -616,19 +616,24 @@ atsne_status f_launch(const FParams &p, int64_t units, cudaStream_t stream) {
 
 }  // namespace
 
-// The splits of Qp row pairs against `tiles` column tiles over the SM pairs: a
-// split costs the fixed threshold nothing but a few more (shorter) buffers per
-// row, so it is chosen for the last wave: the fewest splits whose critical path
-// (waves of units, each its tiles and about two tiles of start-up) is within 2%
-// of the shortest found. The splits take the tiles in turn, so that neighbours
-// that follow one another in the corpus (sorted by class) spread over them.
-int filter_splits(int64_t Qp, int64_t tiles, int max_splits) {
+// The critical path, in column tiles, of Qp row pairs against `tiles` column
+// tiles in s splits over the SM pairs: waves of units, each its tiles and about
+// two tiles of start-up.
+double filter_path(int64_t Qp, int64_t tiles, int s) {
     const int64_t C = num_sms() / 2 > 0 ? num_sms() / 2 : 1;
-    auto cost = [&](int64_t s) { return (double)((Qp * s + C - 1) / C) * (double)((tiles + s - 1) / s + 2); };
-    double best = cost(1);
-    for (int s = 2; s <= max_splits && s <= tiles; ++s) best = fmin(best, cost(s));
+    return (double)((Qp * s + C - 1) / C) * (double)((tiles + s - 1) / s + 2);
+}
+
+// A split costs the fixed threshold nothing but a few more (shorter) buffers per
+// row, so it is chosen for the last wave: the fewest splits whose critical path
+// is within 2% of the shortest found. The splits take the tiles in turn, so that
+// neighbours that follow one another in the corpus (sorted by class) spread over
+// them.
+int filter_splits(int64_t Qp, int64_t tiles, int max_splits) {
+    double best = filter_path(Qp, tiles, 1);
+    for (int s = 2; s <= max_splits && s <= tiles; ++s) best = fmin(best, filter_path(Qp, tiles, s));
     for (int s = 1; s <= max_splits && s <= tiles; ++s)
-        if (cost(s) <= 1.02 * best) return s;
+        if (filter_path(Qp, tiles, s) <= 1.02 * best) return s;
     return 1;
 }
 

@@ -168,7 +168,7 @@ struct TcParams {
     // query row rlist[r], *rcount rows in all, their splits from retry_plan
     const int32_t *rlist, *rcount;
     const float *tau0;     // [Q] key thresholds those rows start from
-    int64_t bufs;          // room for that many (row, split) buffers
+    int64_t rmax, bufs;    // of which at most rmax are taken, in room for that many (row, split) buffers
     int64_t Q, N;
     int KB;                // Dp / 64
     int splits, cols_per_split, row_tiles;
@@ -320,17 +320,18 @@ knn_prep_kernel(const float *__restrict__ X, const int32_t *__restrict__ rows, i
                 int D, int Dp, int passes, __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo,
                 float *__restrict__ nrm, float4 *__restrict__ stats, unsigned *__restrict__ gmax,
                 __nv_bfloat16 *__restrict__ bext, __nv_bfloat16 *__restrict__ aext, int *status,
-                const int64_t *__restrict__ count) {
+                const int64_t *__restrict__ count, int64_t ext_rows) {
     const int lane = threadIdx.x & 31;
     if (count) nrows = min(*count, nrows);
     if (aext && blockIdx.x == 0) fold_query_slice(aext);
-    const int64_t last = bext ? (nrows + TC_BN - 1) / TC_BN * TC_BN : nrows;
+    const int64_t last = bext ? ext_rows : nrows;
     const int64_t step = ((int64_t)gridDim.x * blockDim.x) >> 5;
     float ma = 0.f, me = 0.f, ml = 0.f;
     bool finite = true, exact = true;
     for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < last; r += step) {
         if (r >= nrows) {
-            // the norm slices of the rows that fill the last column tile: +inf, a key no row keeps
+            // the norm slices of the rows that fill the last column tile (the fixed
+            // threshold's): +inf, a key no row keeps
             if (lane < 16) bext[r * 16 + lane] = __float2bfloat16_rn(lane == 0 ? INFINITY : 0.f);
             continue;
         }
@@ -510,7 +511,7 @@ __global__ void __launch_bounds__(TcCfg<PASSES>::THREADS, 1) knn_tc_kernel(const
     fence_after_sync();
     const uint32_t tbase = s.tmem_base;
     UnitPlan up{p.Q, p.row_tiles, p.splits, p.cols_per_split};
-    if (p.rcount) up = retry_plan(*p.rcount, p.N, p.bufs);
+    if (p.rcount) up = retry_plan(min((int64_t)*p.rcount, p.rmax), p.N, p.bufs);
     const int n_units = up.row_tiles * up.splits;
 
     if (warp == 0) {
@@ -1106,7 +1107,7 @@ struct MergeParams {
     const int32_t *perm;
     // the rows given up by the fixed-threshold kernel (as in TcParams), or nullptr
     const int32_t *rlist, *rcount;
-    int64_t bufs;
+    int64_t rmax, bufs;
     const int64_t *qcount;  // if given, the rows in use (device; at most Q)
     int tag;                // of the launch that wrote the buffers
     bool flag_out;          // flag output rows (for the brute-force kernel), else query rows
@@ -1266,7 +1267,7 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : SELECT ? 6 : 5) k
     int64_t Q = p.big_rows ? *p.big_count : p.qcount ? min(*p.qcount, p.Q) : p.Q;
     int S = p.splits;
     if (p.rcount) {
-        const UnitPlan up = retry_plan(*p.rcount, p.N, p.bufs);
+        const UnitPlan up = retry_plan(min((int64_t)*p.rcount, p.rmax), p.N, p.bufs);
         Q = up.Q;
         S = up.splits * p.splits;  // splits of a row by buffers of a split
     }
@@ -1975,15 +1976,15 @@ void clear_tuned_splits() {
     g_tuned.clear();
 }
 
-int tc_split_candidates(int64_t N, int D, int64_t Q, int k, int precision, int rerank_k, int *out, int max_out) {
+int tc_split_candidates(int64_t N, int D, int64_t Q, bool list, int k, int precision, int rerank_k, int *out, int max_out) {
     const int64_t row_tiles = (Q + TC_BM - 1) / TC_BM;
     const int64_t units[] = {0, 152, 304, 608, 1216, 2048, 4096, 8192};
     int n = 0;
-    out[n++] = tc_splits(tc_plan(N, D, Q, k, precision, rerank_k, -1));  // the rule's
+    out[n++] = tc_splits(tc_plan(N, D, Q, list, k, precision, rerank_k, -1));  // the rule's
     for (int64_t u : units) {
         if (n == max_out) break;
         const int want = u == 0 ? 1 : (int)((u + row_tiles - 1) / row_tiles);
-        const int s = tc_splits(tc_plan(N, D, Q, k, precision, rerank_k, want));
+        const int s = tc_splits(tc_plan(N, D, Q, list, k, precision, rerank_k, want));
         bool dup = false;
         for (int i = 0; i < n; ++i) dup |= out[i] == s;
         if (!dup) out[n++] = s;
@@ -1993,91 +1994,12 @@ int tc_split_candidates(int64_t N, int D, int64_t Q, int k, int precision, int r
 
 int tc_splits(const TcPlan &pl) { return pl.filter ? pl.fsplits : pl.splits; }
 
-// The fixed-threshold plan (knn_filter.cu): the sample its thresholds come from
-// and the buffers for what lies below them.
-static void plan_filter(TcPlan &pl, int64_t N, int64_t Q, int splits) {
-    const int64_t pairs = (Q + 2 * TC_BM - 1) / (2 * TC_BM);
-    const int64_t col_tiles = (N + TC_BN - 1) / TC_BN;
-    const int cw = TC_BN / F_PARTS;  // columns of a part
-    if (N < FILTER_MIN_ROWS) return;
-    // S rows, about 32 sqrt(N): the sample's pass and what the thresholds let
-    // through then cost about the same
-    int S = 512;
-    while (S < 65536 && (double)S * S < 0.5 * 1024.0 * (double)N) S <<= 1;
-    while (S > N / 2) S >>= 1;
-    // of n keys below a threshold about x = n S / N are sampled; taking the
-    // r-th smallest sampled key as the threshold leaves fewer than ksel corpus
-    // keys below it when r or more of x = ksel S / N expected fall there:
-    // r - 3 sqrt(r) = x, about one row in a thousand
-    const double x = (double)pl.ksel * S / (double)N;
-    const double rt = 1.5 + sqrt(2.25 + x);
-    const double r = rt * rt;
-    const double expect = r * (double)N / S;
-    if (expect > 0.4 * (double)N) return;
-    // only the best key of each block of sampled columns is kept: a share q of
-    // the blocks holds one of the r. The largest block that leaves q below 0.6
-    const double f = r / S;
-    int blk = cw;
-    auto share = [&](int b) { return 1.0 - pow(1.0 - f, b); };
-    if (share(cw) > 0.6) blk = 32;
-    if (blk == 32 && share(32) > 0.6) blk = 8;
-    while (S / blk > 1024) blk = blk == 8 ? 32 : cw;
-    if (share(blk) > 0.9) return;
-    pl.filter = true;
-    pl.S = S;
-    pl.blk = blk;
-    pl.rank = (int)fmax(1.0, floor(share(blk) * (S / blk) + 0.5));
-    // a row given up for too few keys starts again from a rank that leaves it
-    // short with a probability below 10^-9: r - 7 sqrt(r) = x
-    const double rt2 = 3.5 + sqrt(12.25 + x), f2 = fmin(0.9, rt2 * rt2 / S);
-    pl.rank2 = (int)fmin((double)(S / blk), floor((1.0 - pow(1.0 - f2, blk)) * (S / blk) + 1.0));
-    if (splits <= 0) splits = filter_splits(pairs, col_tiles, 64);
-    if (splits > 64) splits = 64;
-    if (splits > col_tiles) splits = (int)col_tiles;
-    pl.fsplits = splits;
-    pl.fkeys = (int)expect;
-}
-
-// The fixed threshold's buffers: twice a part's share of the keys a row is
-// expected to keep. They spread over a row's splits and the parts of its tiles,
-// unless its neighbours all lie in one part (a corpus whose classes repeat every
-// 256 rows). Where the rows keep their order (knn_order.cu regroups those of
-// large sets) a buffer then holds its share of one part, and more by the spread
-// of a threshold taken from r sampled keys, as far as the adaptive launch's
-// buffers, whose memory these take, leave room. 60,000 x 32, four clusters in turn
-// in blocks of 64 rows: with every row given up after the filter had run 4.4 ms
-// (FP32) and 13.5 ms (BF16 approximate), now 1.5 and 2.1 ms; the same rows
-// shuffled 2.0 and 2.6 ms.
-static void plan_buffers(TcPlan &pl, int64_t N, bool ordered) {
-    const int64_t per = ((N + TC_BN - 1) / TC_BN + pl.fsplits - 1) / pl.fsplits * (TC_BN / F_PARTS);  // columns of a buffer
-    int64_t cap = (pl.fkeys + 1) / 2 + 48;
-    if (!ordered) {
-        const double r = (double)pl.fkeys * pl.S / (double)N;
-        const int64_t part = (int64_t)ceil(pl.fkeys * (1.0 + 2.0 / sqrt(r)) / pl.fsplits) + 48;
-        const int64_t room = (int64_t)pl.splits * pl.halves * pl.cap / (pl.fsplits * F_PARTS);
-        if (cap < part) cap = part < room ? part : cap < room ? room : cap;
-    }
-    if (cap > per) cap = per;
-    pl.fcap = (int)((cap + 15) / 16 * 16);
-}
-
-TcPlan tc_plan(int64_t N, int D, int64_t Q, int k, int precision, int rerank_k, int splits) {
-    TcPlan pl;
-    pl.passes = precision == ATSNE_FP32 ? 3 : precision == ATSNE_FP8_RERANK ? 8 : 1;
-    pl.certify = precision != ATSNE_FP8_RERANK && precision != ATSNE_BF16_RERANK_APPROX;
-    const int ke = pl.passes == 8 ? 128 : TC_BK;  // elements per 128-byte row
-    pl.Dp = ((D + ke - 1) / ke) * ke;
-    int ks = rerank_k > 0 ? rerank_k : (pl.passes == 3 ? k + 38 : !pl.certify ? 4 * k : 2 * k);
-    if (!pl.certify && ks > RCAP_FP8 / 2) ks = RCAP_FP8 / 2;
-    if (ks < k) ks = k;
-    pl.ksel = ks;
-    if (splits == 0) splits = tuned_splits(N, D, Q, k, precision, rerank_k);
-    if (pl.passes != 8) plan_filter(pl, N, Q, splits);
-    if (pl.filter) splits = 0;  // the adaptive kernel then only takes the rows given up
-    // The adaptive kernel: (row tile, column split) units, one split per row
-    // tile when the row tiles alone give every SM at least two units (a split
-    // restarts the streaming top-k, whose k' ln(n / k') survivors dominate the
-    // epilogue), else about 2048 units, each at least 4 column tiles long
+// The adaptive launch over all Q rows: (row tile, column split) units, one split
+// per row tile when the row tiles alone give every SM at least two units (a
+// split restarts the streaming top-k, whose k' ln(n / k') survivors dominate the
+// epilogue), else about 2048 units, each at least 4 column tiles long.
+static void plan_adaptive(TcPlan &pl, int64_t N, int64_t Q, int splits) {
+    const int ks = pl.ksel;
     pl.row_tiles = (int)((Q + TC_BM - 1) / TC_BM);
     const int64_t col_tiles = (N + TC_BN - 1) / TC_BN;
     int64_t S = splits > 0 ? splits : pl.row_tiles >= 304 ? 1 : (2048 + pl.row_tiles - 1) / pl.row_tiles;
@@ -2102,20 +2024,186 @@ TcPlan tc_plan(int64_t N, int D, int64_t Q, int k, int precision, int rerank_k, 
     // the epilogue's bucket counts are 16 bits and never exceed the buffer's size
     if (cap > 65504) cap = 65504;
     pl.cap = (int)((cap + 31) / 32 * 32);
-    if (pl.filter) plan_buffers(pl, N, knn_ordered(N, D, Q != N, pl));
+    pl.rrows = Q;
+    pl.cand_bytes = (size_t)Q * pl.splits * pl.halves * pl.cap * sizeof(Cand);
+}
+
+static size_t plan_bytes(int64_t N, int D, int64_t Q, bool list, const TcPlan &pl) {
+    Carver c(nullptr);
+    return tc_workspace(c, N, D, Q, list, pl, nullptr);
+}
+
+// The thresholds from a sample of S rows; false: they would let too much through.
+static bool plan_sample(TcPlan &pl, int64_t N, int S) {
+    // of n keys below a threshold about x = n S / N are sampled; taking the
+    // r-th smallest sampled key as the threshold leaves fewer than ksel corpus
+    // keys below it when r or more of x = ksel S / N expected fall there:
+    // r - 3 sqrt(r) = x, about one row in a thousand
+    const double x = (double)pl.ksel * S / (double)N;
+    const double rt = 1.5 + sqrt(2.25 + x);
+    const double r = rt * rt;
+    const double expect = r * (double)N / S;
+    if (expect > 0.4 * (double)N) return false;
+    // only the best key of each block of sampled columns is kept: a share q of
+    // the blocks holds one of the r. The largest block that leaves q below 0.6
+    const int cw = TC_BN / F_PARTS;  // columns of a part
+    const double f = r / S;
+    int blk = cw;
+    auto share = [&](int b) { return 1.0 - pow(1.0 - f, b); };
+    if (share(cw) > 0.6) blk = 32;
+    if (blk == 32 && share(32) > 0.6) blk = 8;
+    while (S / blk > 1024) blk = blk == 8 ? 32 : cw;
+    if (share(blk) > 0.9) return false;
+    pl.S = S;
+    pl.blk = blk;
+    pl.rank = (int)fmax(1.0, floor(share(blk) * (S / blk) + 0.5));
+    // a row given up for too few keys starts again from a rank that leaves it
+    // short with a probability below 10^-9: r - 7 sqrt(r) = x
+    const double rt2 = 3.5 + sqrt(12.25 + x), f2 = fmin(0.9, rt2 * rt2 / S);
+    pl.rank2 = (int)fmin((double)(S / blk), floor((1.0 - pow(1.0 - f2, blk)) * (S / blk) + 1.0));
+    pl.fkeys = (int)expect;
+    return true;
+}
+
+// The fixed-threshold launch with pl.fsplits splits and the adaptive one after it,
+// in the `most` bytes of workspace that the adaptive launch over all rows would
+// take by itself (false: they do not fit), or, without a limit, in what they need.
+//
+// The candidate region holds, in turn, the sampled rows and the block values,
+// the fixed threshold's buffers (and the block values, where the rows given up
+// start from them) and the adaptive launch's buffers. The latter get up to a
+// quarter less per row than by themselves, which pays for the copies of the rows
+// given up (a list's take the place of the list's own copies) and the
+// thresholds; where that is not enough (long rows), they hold fewer rows, at
+// least half, and what is given up beyond those goes to the brute-force kernel.
+//
+// A buffer holds twice a part's share of the keys a row is expected to keep.
+// They spread over a row's splits and the parts of its tiles, unless its
+// neighbours all lie in one part (a corpus whose classes repeat every 256
+// rows). Where the rows keep their order (knn_order.cu regroups those of large
+// sets) a buffer then holds its share of one part, and more by the spread of a
+// threshold taken from r sampled keys, as far as the region leaves room. 60,000
+// x 32, four clusters in turn in blocks of 64 rows: with every row given up
+// after the filter had run 4.4 ms (FP32) and 13.5 ms (BF16 approximate), now
+// 1.5 and 2.1 ms; the same rows shuffled 2.0 and 2.6 ms.
+static bool plan_region(TcPlan &pl, int64_t N, int D, int64_t Q, bool list, size_t most) {
+    const int64_t per = ((N + TC_BN - 1) / TC_BN + pl.fsplits - 1) / pl.fsplits * (TC_BN / F_PARTS);  // columns of a buffer
+    const double r = (double)pl.fkeys * pl.S / (double)N;
+    // keys per buffer, at least: its share, the threshold's spread (one row in a
+    // thousand is above it), the share's, and the chunk that closes a buffer.
+    // Neighbours that follow one another fill no more than four of the splits
+    const double share = (double)pl.fkeys / (F_PARTS * hmin(pl.fsplits, 4));
+    const int64_t least = hmin(per, (int64_t)ceil(share * (1.0 + 3.5 / sqrt(r)) + 3.0 * sqrt(share)) + 32);
+    int64_t want = (hmin(per, (int64_t)(pl.fkeys + 1) / 2 + 48) + 15) / 16 * 16, part = 0;
+    if (!knn_ordered(N, D, list, pl))
+        part = hmin(per, (int64_t)ceil(pl.fkeys * (1.0 + 2.0 / sqrt(r)) / pl.fsplits) + 48);
+    // bytes of the region's other tenants
+    const size_t minima = ((size_t)Q * (pl.S / pl.blk) * sizeof(float) + 255) / 256 * 256;
+    const size_t sample = (size_t)pl.S * (pl.Dp + 16) * sizeof(uint16_t) + minima;
+    const size_t kept = pl.certify ? 0 : minima;
+    const size_t per_key = (size_t)Q * pl.fsplits * F_PARTS * sizeof(Cand);
+    const size_t row_key = (size_t)pl.splits * pl.halves * sizeof(Cand);  // of the adaptive launch, per row and key
+    const size_t cap0 = (size_t)pl.cap;
+    auto larger = [](size_t a, size_t b) { return a > b ? a : b; };
+    pl.filter = true;
+    if (!most) {
+        pl.cand_bytes = larger(larger(sample, kept + want * per_key), Q * row_key * cap0);
+    } else {
+        const size_t need = larger(sample, kept + least * per_key);
+        auto room = [&](int64_t rows) {
+            pl.rrows = rows;
+            pl.cand_bytes = 0;
+            const size_t b = plan_bytes(N, D, Q, list, pl);
+            return most > b ? (most - b) / 256 * 256 : (size_t)0;
+        };
+        auto fits = [&](int64_t rows) {
+            const size_t got = room(rows);
+            return got >= need && got >= rows * row_key * cap0;
+        };
+        size_t got = room(Q);
+        const size_t cap = got / (Q * row_key) / 2 * 2;
+        if (cap < cap0) {
+            if (cap >= larger(cap0 - cap0 / 4, pl.ksel + TC_BN / pl.halves + 32)) {
+                pl.cap = (int)cap;
+            } else {
+                if (!fits((Q + 1) / 2)) return false;
+                int64_t lo = (Q + 1) / 2, hi = Q;  // the most rows that fit
+                while (lo < hi) {
+                    const int64_t mid = hi - (hi - lo) / 2;
+                    if (fits(mid)) lo = mid;
+                    else hi = mid - 1;
+                }
+                got = room(lo);
+            }
+        }
+        if (got < need) return false;
+        pl.cand_bytes = got;
+        if (want < least) want = least;
+    }
+    const int64_t keys = (int64_t)((pl.cand_bytes - kept) / per_key);  // per buffer that fit
+    pl.fcap = (int)hmin((want > part ? want : part) + 15, keys);
+    if (pl.fcap / 16 * 16 >= want) pl.fcap = pl.fcap / 16 * 16;
+    return true;
+}
+
+// The fixed-threshold plan (knn_filter.cu), if there is one: the sample its
+// thresholds come from and the launches' buffers.
+static bool plan_filter(TcPlan &pl, int64_t N, int D, int64_t Q, bool list, int splits) {
+    if (N < FILTER_MIN_ROWS) return false;
+    const int64_t pairs = (Q + 2 * TC_BM - 1) / (2 * TC_BM);
+    const int64_t col_tiles = (N + TC_BN - 1) / TC_BN;
+    const size_t most = plan_bytes(N, D, Q, list, pl);
+    // S rows, about 32 sqrt(N): the sample's pass and what the thresholds let
+    // through then cost about the same
+    int S = 512;
+    while (S < 65536 && (double)S * S < 0.5 * 1024.0 * (double)N) S <<= 1;
+    while (S > N / 2) S >>= 1;
+    if (!plan_sample(pl, N, S)) return false;
+    pl.fsplits = splits > 0 ? (int)hmin(hmin((int64_t)splits, (int64_t)64), col_tiles) : filter_splits(pairs, col_tiles, 64);
+    // within the adaptive launch's workspace if that costs no speed: as many
+    // splits, or fewer with no longer a critical path. What does not fit are a
+    // few queries (their sample: 1 query of 70,000 x 784 takes 13 MB more, 0.41
+    // instead of 0.80 ms) and small k in one pass (the few keys of a row spread
+    // by the threshold: 376,008 x 205, k = 6, 44 instead of 166 ms)
+    const double best = filter_path(pairs, col_tiles, pl.fsplits);
+    for (int n = pl.fsplits; n > 0; n = splits > 0 ? 0 : n - 1) {
+        if (filter_path(pairs, col_tiles, n) > best) continue;
+        TcPlan g = pl;
+        g.fsplits = n;
+        if (!plan_region(g, N, D, Q, list, most)) continue;
+        pl = g;
+        return true;
+    }
+    return plan_region(pl, N, D, Q, list, 0);
+}
+
+TcPlan tc_plan(int64_t N, int D, int64_t Q, bool list, int k, int precision, int rerank_k, int splits) {
+    TcPlan pl;
+    pl.passes = precision == ATSNE_FP32 ? 3 : precision == ATSNE_FP8_RERANK ? 8 : 1;
+    pl.certify = precision != ATSNE_FP8_RERANK && precision != ATSNE_BF16_RERANK_APPROX;
+    const int ke = pl.passes == 8 ? 128 : TC_BK;  // elements per 128-byte row
+    pl.Dp = ((D + ke - 1) / ke) * ke;
+    int ks = rerank_k > 0 ? rerank_k : (pl.passes == 3 ? k + 38 : !pl.certify ? 4 * k : 2 * k);
+    if (!pl.certify && ks > RCAP_FP8 / 2) ks = RCAP_FP8 / 2;
+    if (ks < k) ks = k;
+    pl.ksel = ks;
+    if (splits == 0) splits = tuned_splits(N, D, Q, k, precision, rerank_k);
+    plan_adaptive(pl, N, Q, pl.passes == 8 ? splits : 0);
+    if (pl.passes != 8 && !plan_filter(pl, N, D, Q, list, splits)) plan_adaptive(pl, N, Q, splits);
     return pl;
 }
 
 // Queries from another array with radii: the radii are the thresholds, nothing
 // is sampled, and what does not fit the buffers goes to the brute-force kernel.
 TcPlan tc_plan_radius(int64_t N, int D, int64_t Q, int k, int precision, int rerank_k) {
-    TcPlan pl = tc_plan(N, D, Q, k, precision, rerank_k);
+    TcPlan pl = tc_plan(N, D, Q, true, k, precision, rerank_k);
     const int64_t col_tiles = (N + TC_BN - 1) / TC_BN;
     const int s = filter_splits((Q + 2 * TC_BM - 1) / (2 * TC_BM), col_tiles, 64);
     pl.filter = true;
     pl.S = 0;
     pl.fsplits = s;
     pl.fcap = RADIUS_CAP;
+    pl.cand_bytes = (size_t)Q * s * F_PARTS * RADIUS_CAP * sizeof(Cand);
     return pl;
 }
 
@@ -2134,28 +2222,31 @@ size_t tc_workspace(Carver &c, int64_t N, int D, int64_t Q, bool list, const TcP
     w.stats = c.take<float>((size_t)N * 4);
     w.gmax = c.take<unsigned>(4);
     // the adaptive kernel's launch (all rows, or those given up) and the
-    // fixed-threshold one before it use the same buffers in turn
+    // fixed-threshold one before it use the same buffers in turn (plan_region)
     const bool adaptive = !pl.filter || pl.S > 0;
-    const size_t abufs = adaptive ? (size_t)Q * pl.splits * pl.halves : 0;
+    const size_t abufs = adaptive ? (size_t)pl.rrows * pl.splits * pl.halves : 0;
     const size_t fbufs = pl.filter ? (size_t)Q * pl.fsplits * F_PARTS : 0;
-    const size_t cands = abufs * pl.cap > fbufs * pl.fcap ? abufs * pl.cap : fbufs * pl.fcap;
-    w.cand = c.take<char>(cands * sizeof(Cand));
+    w.cand = c.take<char>(pl.cand_bytes);
     w.metas = abufs > fbufs ? abufs : fbufs;
     w.meta = c.take<char>(w.metas * sizeof(int4));
-    w.hist_rows = pl.filter ? (pl.S > 0 ? hmin(Q, RETRY_SPLIT_ROWS) : 0) : pl.splits > 1 ? Q : 0;
+    w.hist_rows = pl.filter ? (pl.S > 0 ? hmin(pl.rrows, RETRY_SPLIT_ROWS) : 0) : pl.splits > 1 ? Q : 0;
     w.row_hist = w.hist_rows > 0 ? c.take<unsigned>((size_t)w.hist_rows * GH_BUCKETS) : nullptr;
     w.flag_rows = c.take<int32_t>((size_t)Q);
-    w.flag_count = c.take<int32_t>(3);
-    w.bext = pl.passes == 1 ? c.take<uint16_t>((size_t)((N + TC_BN - 1) / TC_BN * TC_BN) * 16) : nullptr;
+    w.flag_count = c.take<int32_t>(6);
+    w.row_count = reinterpret_cast<int64_t *>(w.flag_count + 4);
+    w.ext_rows = pl.filter ? (N + TC_BN - 1) / TC_BN * TC_BN : N;
+    w.bext = pl.passes == 1 ? c.take<uint16_t>((size_t)w.ext_rows * 16) : nullptr;
     w.aext = pl.passes == 1 || pl.S > 0 ? c.take<uint16_t>((size_t)TC_BM * 16) : nullptr;
     if (pl.filter) w.tau = c.take<float>((size_t)Q);
     if (pl.S > 0) {
-        w.shi = c.take<uint16_t>((size_t)pl.S * per);
-        w.sext = c.take<uint16_t>((size_t)pl.S * 16);
-        w.minima = c.take<float>((size_t)Q * (pl.S / pl.blk));
+        // the sampled rows at the region's start, the block values at its end
+        w.shi = reinterpret_cast<uint16_t *>(w.cand);
+        w.sext = w.shi + (size_t)pl.S * per;
+        w.minima = reinterpret_cast<float *>(
+            w.cand + (pl.cand_bytes - ((size_t)Q * (pl.S / pl.blk) * sizeof(float) + 255) / 256 * 256));
         w.retry_rows = c.take<int32_t>((size_t)Q);
-        w.rhi = c.take<uint16_t>((size_t)Q * per);
-        w.rlo = pl.passes == 3 ? c.take<uint16_t>((size_t)Q * per) : nullptr;
+        w.rhi = list ? w.qhi : c.take<uint16_t>((size_t)pl.rrows * per);
+        w.rlo = list ? w.qlo : pl.passes == 3 ? c.take<uint16_t>((size_t)pl.rrows * per) : nullptr;
     }
     w.ordered = knn_ordered(N, D, list, pl);
     // the global column clock where many units stream a corpus larger than L2
@@ -2168,17 +2259,28 @@ size_t tc_workspace(Carver &c, int64_t N, int D, int64_t Q, bool list, const TcP
     return c.bytes();
 }
 
-// The BF16 copies of the rows given up by the fixed threshold, one warp per row.
+// The BF16 copies of the rows given up by the fixed threshold, as knn_prep makes
+// them, one warp per row; rows beyond the `room` of the adaptive launch go to the
+// brute-force kernel's list.
 __global__ void __launch_bounds__(256)
-knn_gather_kernel(const int32_t *__restrict__ rows, const int32_t *__restrict__ count, int Dp,
-                  const uint16_t *__restrict__ hi, const uint16_t *__restrict__ lo, uint16_t *__restrict__ rhi,
-                  uint16_t *__restrict__ rlo) {
+knn_gather_kernel(const float *__restrict__ X, const int32_t *__restrict__ qlist, const int32_t *__restrict__ perm,
+                  int64_t N, int D, int Dp, const int32_t *__restrict__ rows, const int32_t *__restrict__ count,
+                  int64_t room, __nv_bfloat16 *__restrict__ rhi, __nv_bfloat16 *__restrict__ rlo,
+                  int32_t *__restrict__ flag_rows, int32_t *__restrict__ flag_count) {
     const int lane = threadIdx.x & 31, n = *count;
     for (int r = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); r < n; r += (int)(gridDim.x * blockDim.x) >> 5) {
-        const int64_t a = (int64_t)rows[r] * Dp, b = (int64_t)r * Dp;
-        for (int t = lane; t < (Dp >> 3); t += 32) {
-            reinterpret_cast<uint4 *>(rhi + b)[t] = reinterpret_cast<const uint4 *>(hi + a)[t];
-            if (lo) reinterpret_cast<uint4 *>(rlo + b)[t] = reinterpret_cast<const uint4 *>(lo + a)[t];
+        const int q = rows[r];
+        int64_t src = qlist ? qlist[q] : perm ? perm[q] : q;
+        if (r >= room) {
+            if (lane == 0) flag_rows[atomicAdd(flag_count, 1)] = perm ? (int)src : q;
+            continue;
+        }
+        if (src < 0 || src >= N) src = 0;  // as in knn_prep: flagged by the caller's index check
+        for (int d = lane; d < Dp; d += 32) {
+            const float v = d < D ? X[src * D + d] : 0.f;
+            const __nv_bfloat16 h = __float2bfloat16_rn(v);
+            rhi[(int64_t)r * Dp + d] = h;
+            if (rlo) rlo[(int64_t)r * Dp + d] = __float2bfloat16_rn(v - __bfloat162float(h));
         }
     }
 }
@@ -2266,7 +2368,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
         auto *lo = reinterpret_cast<__nv_bfloat16 *>(w.lo);
         // ordered rows and columns: the copies, norms and statistics in the order
         if (ordered) ATSNE_TRY(knn_order_launch(X, N, D, pl, TC_BM, TC_BN, w.ord, stream));
-        const int64_t prows = w.bext ? (N + TC_BN - 1) / TC_BN * TC_BN : N;  // the norm slices fill whole tiles
+        const int64_t prows = w.bext ? w.ext_rows : N;
         const int64_t most = 8 * num_sms();
         ATSNE_TRY(launch_kernel("knn_prep", knn_prep_kernel, (int)hmin(most, ceil_div(prows * 32, 256)), 256, 0, stream, X,
                                 ordered ? (const int32_t *)w.ord.perm : (const int32_t *)nullptr, N, N, D,
@@ -2274,7 +2376,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
                                 reinterpret_cast<float4 *>(w.stats), w.gmax,
                                 reinterpret_cast<__nv_bfloat16 *>(w.bext),
                                 reinterpret_cast<__nv_bfloat16 *>(pl.passes == 1 ? w.aext : nullptr), status,
-                                (const int64_t *)nullptr));
+                                (const int64_t *)nullptr, w.ext_rows));
         if (Xq) {
             ATSNE_TRY(launch_kernel("knn_prep", knn_prep_kernel, (int)hmin(most, ceil_div(Q * 32, 256)), 256, 0, stream, Xq,
                                     (const int32_t *)nullptr, Q, Q, D, pl.Dp, pl.passes,
@@ -2282,7 +2384,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
                                     reinterpret_cast<__nv_bfloat16 *>(w.qlo), w.qnrm,
                                     reinterpret_cast<float4 *>(w.qstats), (unsigned *)nullptr,
                                     (__nv_bfloat16 *)nullptr, (__nv_bfloat16 *)nullptr, status,
-                                    (const int64_t *)nullptr));
+                                    (const int64_t *)nullptr, (int64_t)0));
             a_hi = w.qhi;
             a_lo = w.qlo;
         } else if (qlist) {
@@ -2291,7 +2393,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
                                     reinterpret_cast<__nv_bfloat16 *>(w.qhi),
                                     reinterpret_cast<__nv_bfloat16 *>(w.qlo), (float *)nullptr,
                                     (float4 *)nullptr, (unsigned *)nullptr, (__nv_bfloat16 *)nullptr,
-                                    (__nv_bfloat16 *)nullptr, status, qcount));
+                                    (__nv_bfloat16 *)nullptr, status, qcount, (int64_t)0));
             a_hi = w.qhi;
             a_lo = w.qlo;
         }
@@ -2325,7 +2427,8 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
     m.cand = reinterpret_cast<Cand *>(w.cand);
     m.meta = reinterpret_cast<int4 *>(w.meta);
     m.qcount = qcount;
-    m.bufs = Q * (int64_t)pl.splits;
+    m.rmax = pl.rrows;
+    m.bufs = pl.rrows * pl.splits;
     // the fixed-threshold launch; the rows it gives up follow in the adaptive one
     const bool retry = pl.filter && !radius;
     if (pl.filter) {
@@ -2364,14 +2467,15 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
         }
         ATSNE_TRY(merge_launch(pl, m, stream));
         ATSNE_TRY(launch_kernel("knn_gather", knn_gather_kernel, (int)hmin(4 * num_sms(), ceil_div(Q * 32, 256)), 256,
-                                0, stream, (const int32_t *)w.retry_rows, (const int32_t *)(w.flag_count + 1), pl.Dp,
-                                reinterpret_cast<const uint16_t *>(a_hi), reinterpret_cast<const uint16_t *>(a_lo),
-                                w.rhi, w.rlo));
+                                0, stream, Xq ? Xq : X, Xq ? (const int32_t *)nullptr : qlist, m.perm, Xq ? Q : N, D,
+                                pl.Dp, (const int32_t *)w.retry_rows, (const int32_t *)(w.flag_count + 1), pl.rrows,
+                                reinterpret_cast<__nv_bfloat16 *>(w.rhi), reinterpret_cast<__nv_bfloat16 *>(w.rlo),
+                                w.flag_rows, w.flag_count));
         if (!pl.certify) ATSNE_TRY(knn_retry_tau_launch(pl, w, stream));
         a_hi = w.rhi;
         a_lo = w.rlo;
     }
-    const int64_t a_rows = (qlist || Xq || retry) ? Q : N;
+    const int64_t a_rows = qlist || Xq ? Q : retry ? pl.rrows : N;
     TcParams p;
     memset(&p, 0, sizeof(p));
     if (fp8) {
@@ -2403,6 +2507,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
     p.rlist = retry ? w.retry_rows : nullptr;
     p.rcount = retry ? w.flag_count + 1 : nullptr;
     p.tau0 = retry ? w.tau : nullptr;
+    p.rmax = m.rmax;
     p.bufs = m.bufs;
     p.clock = w.clock;
     p.qst = reinterpret_cast<const float4 *>(w.qstats);

@@ -117,3 +117,13 @@ def test_neighbours_all_in_one_part_of_the_tiles(at, precision):
         ti, td = at.atsne_knn(X, k)
         at.atsne_check()
         assert torch.equal(ti[q.long()], ri[:, :k]) and torch.equal(td[q.long()], rd[:, :k])
+
+
+@pytest.mark.parametrize("N,D,k", [(4000, 4096, 30), (1500, 3360, 10)])
+def test_more_rows_given_up_than_the_adaptive_launch_holds(at, N, D, k):
+    # long rows with few distances between them: every row's threshold falls on
+    # a tie, and the copies of the rows given up do not fit for all of them
+    X = torch.zeros((N, D), device="cuda")
+    X[:, ::D // 7] = (rows(N, X[:, ::D // 7].shape[1], D) > 0).float()
+    same(at, X, k)
+    same(at, X, k, queries=torch.arange(0, N, 3, dtype=torch.int32, device="cuda"))
