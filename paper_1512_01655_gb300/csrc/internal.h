@@ -33,7 +33,8 @@ struct TcPlan {
     // adaptive launch over the rows it gives up
     bool filter = false;
     int S = 0, blk = 0, rank = 0, rank2 = 0;     // sampled rows, columns per block, the thresholds' ranks
-    int fsplits = 1, fcap = 0, fkeys = 0;  // fkeys: keys a row is expected to buffer
+    int fsplits = 1, fparts = 4, fcap = 0;  // buffers per row: fsplits x fparts, of fcap keys
+    int fkeys = 0;                          // keys a row is expected to buffer
 };
 // Row and column order of a large self kNN (points grouped by nearest
 // centroid; each row tile streams its own groups' column tiles first).
@@ -93,7 +94,7 @@ atsne_status knn_order_launch(const float *X, int64_t N, int D, const TcPlan &pl
                               const OrderWs &w, cudaStream_t stream);
 // Xq != nullptr: the Q queries are the rows of Xq (another array), none excluded.
 // radius != nullptr (with Xq): only neighbours with d^2 < radius[row] are kept,
-// the row padded with (-1, +inf); the plan's cap is then RADIUS_CAP.
+// the row padded with (-1, +inf); the plan is then tc_plan_radius'.
 constexpr int RADIUS_CAP = 256;
 atsne_status radius_filter_launch(int32_t *idx, float *d2, int64_t rows, int k, const float *radius,
                                   cudaStream_t stream);

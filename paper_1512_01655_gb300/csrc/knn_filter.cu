@@ -93,6 +93,8 @@ struct __align__(1024) FSmem {
     uint64_t ext_bar;
     // per stage, the last load this CTA issued: its number from 1, its bytes
     uint32_t load_no[FC<PASSES>::MAX_STAGES], load_bytes[FC<PASSES>::MAX_STAGES];
+    // F_RADIUS: per row of three units in turn, its keys and the parts done with it
+    int row_cnt[3][F_BM], row_done[3][F_BM];
     uint32_t tmem_base;
     int abort_flag;
     int zero;
@@ -108,7 +110,7 @@ struct FParams {
     int KB, last_steps;      // k-blocks; K = 16 steps of the last one
     int splits;              // split sp takes the column tiles sp, sp + splits, ...
     int cap;
-    Cand *cand;              // [Q][splits * F_PARTS][cap]
+    Cand *cand;              // [Q][splits * buffers per split][cap]
     int4 *meta;
     float *minima;           // SAMPLE: [Q][m] block maxima of the accumulators
     int m, blk;              // blk: columns per block (8, 32 or 64)
@@ -116,10 +118,17 @@ struct FParams {
     uint64_t wait_ns;
 };
 
-template <int PASSES, bool SAMPLE>
+// F_SAMPLE: the sampled rows' block maxima. F_RADIUS: few keys lie below the
+// thresholds, and the four parts of a row append to one buffer, counted in shared
+// memory: a row's room is its own wherever its points lie (a buffer per part
+// for any distribution took four times the memory).
+enum : int { F_MAIN = 0, F_SAMPLE = 1, F_RADIUS = 2 };
+template <int PASSES, int MODE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(FC<PASSES>::THREADS, 1)
 knn_filter_kernel(const __grid_constant__ FParams p) {
     using C = FC<PASSES>;
+    constexpr bool SAMPLE = MODE == F_SAMPLE, RADIUS = MODE == F_RADIUS;
+    constexpr int PARTS = RADIUS ? 1 : F_PARTS;  // buffers per row and split
     extern __shared__ __align__(16) unsigned char f_raw[];
     const uint32_t pad = (1024u - (smem_u32(f_raw) & 1023u)) & 1023u;
     FSmem<PASSES> &s = *reinterpret_cast<FSmem<PASSES> *>(f_raw + pad);
@@ -145,6 +154,8 @@ knn_filter_kernel(const __grid_constant__ FParams p) {
         s.zero = 0;
         fence_mbar_init();
     }
+    if (RADIUS)
+        for (int i = threadIdx.x; i < 3 * F_BM; i += blockDim.x) (&s.row_cnt[0][0])[i] = (&s.row_done[0][0])[i] = 0;
     if (threadIdx.x == 32) {
         tma_prefetch_desc(&p.tm_a_hi);
         tma_prefetch_desc(&p.tm_b_hi);
@@ -287,7 +298,8 @@ knn_filter_kernel(const __grid_constant__ FParams p) {
         const int part = e >> 2;
         const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
         const uint32_t acc_empty0 = map_to_rank(smem_u32(&s.acc_empty[0]), 0);
-        const int subs = p.splits * F_PARTS;
+        const int subs = p.splits * PARTS;
+        int slot = 0;  // RADIUS: of the unit's counters
         int acc = 0;
         uint32_t acc_phase = 0;
         bool ok = true;
@@ -303,6 +315,7 @@ knn_filter_kernel(const __grid_constant__ FParams p) {
             float *mrow = nullptr;
             float tau = -INFINITY;
             int cnt = 0, full = 0;
+            int *row_cnt = RADIUS ? &s.row_cnt[slot][quarter * 32 + lane] : nullptr;
             if (live) {
                 if (SAMPLE) {
                     mrow = p.minima + row * p.m;
@@ -311,7 +324,7 @@ knn_filter_kernel(const __grid_constant__ FParams p) {
                     tau = p.tau[row];
                     const float tf = fminf(tau, FLT_MAX);
                     thr = C::FOLD ? -0.5f * tf : -tf;
-                    buf = p.cand + ((size_t)row * subs + (size_t)sp * F_PARTS + part) * p.cap;
+                    buf = p.cand + ((size_t)row * subs + (size_t)sp * PARTS + (RADIUS ? 0 : part)) * p.cap;
                 }
             }
             float nyn[C::NCH];
@@ -397,8 +410,8 @@ knn_filter_kernel(const __grid_constant__ FParams p) {
                             if (c + 1 == C::NCH && live) mrow[colb0 / C::CW] = pm;
                         }
                     } else if (__any_sync(0xffffffffu, gm > thr)) {
-                        // a buffer without room for the chunk's survivors is closed (the row is given up)
-                        if (cnt > p.cap - 32) {
+                        // a buffer without room for the chunk is closed (the row is given up)
+                        if (!RADIUS && cnt > p.cap - 32) {
                             thr = INFINITY;
                             full = 1;
                         }
@@ -409,7 +422,11 @@ knn_filter_kernel(const __grid_constant__ FParams p) {
 #pragma unroll
                             for (int j = 0; j < 8; ++j) {
                                 const float x = v[8 * q + j];
-                                if (x > thr) buf[cnt++] = Cand{C::FOLD ? -2.f * x : -x, col + 8 * q + j};
+                                if (x > thr) {
+                                    const int at = RADIUS ? atomicAdd(row_cnt, 1) : cnt++;
+                                    if (!RADIUS || at < p.cap) buf[at] = Cand{C::FOLD ? -2.f * x : -x, col + 8 * q + j};
+                                    else thr = INFINITY;  // full
+                                }
                             }
                         }
                     }
@@ -420,9 +437,22 @@ knn_filter_kernel(const __grid_constant__ FParams p) {
                 }
             }
             if (!ok) break;
-            if (!SAMPLE && live)
+            if (RADIUS) {
+                // the last part to finish the row's unit writes its count and
+                // clears it. A unit's counters are taken again three units
+                // later: its tiles start when every warp has arrived for the
+                // tile two before, which lies past the unit
+                __threadfence_block();
+                if (live && atomicAdd(&s.row_done[slot][quarter * 32 + lane], 1) == F_PARTS - 1) {
+                    const int n = atomicExch(row_cnt, 0);
+                    s.row_done[slot][quarter * 32 + lane] = 0;
+                    p.meta[(size_t)row * subs + sp] = make_int4(min(n, p.cap), __float_as_int(tau), n > p.cap, META_FIRST);
+                }
+                slot = slot == 2 ? 0 : slot + 1;
+            } else if (!SAMPLE && live) {
                 p.meta[(size_t)row * subs + (size_t)sp * F_PARTS + part] =
                     make_int4(cnt, __float_as_int(tau), full, META_FIRST);
+            }
         }
     }
     fence_before_sync();
@@ -603,14 +633,14 @@ size_t f_smem_bytes() {
 static_assert(sizeof(FSmem<1>) + 1024 <= 232448, "filter shared memory above 227 KB");
 static_assert(sizeof(FSmem<3>) + 1024 <= 232448, "filter shared memory above 227 KB");
 
-template <int PASSES, bool SAMPLE>
+template <int PASSES, int MODE>
 atsne_status f_launch(const FParams &p, int64_t units, cudaStream_t stream) {
     const size_t smem = f_smem_bytes<PASSES>();
-    cudaError_t e = cudaFuncSetAttribute(knn_filter_kernel<PASSES, SAMPLE>,
+    cudaError_t e = cudaFuncSetAttribute(knn_filter_kernel<PASSES, MODE>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_error(e, "knn_filter attribute");
     const int grid = 2 * (int)hmin(units, num_sms() / 2);
-    return launch_kernel(SAMPLE ? "knn_bound" : "knn_filter", knn_filter_kernel<PASSES, SAMPLE>, grid,
+    return launch_kernel(MODE == F_SAMPLE ? "knn_bound" : "knn_filter", knn_filter_kernel<PASSES, MODE>, grid,
                          FC<PASSES>::THREADS, smem, stream, p);
 }
 
@@ -663,7 +693,7 @@ atsne_status knn_filter_launch(const TcPlan &pl, const TcWs &w, const FilterArgs
         p.minima = w.minima;
         p.m = pl.S / pl.blk;
         p.blk = pl.blk;
-        ATSNE_TRY((f_launch<1, true>(p, pairs * p.splits, stream)));
+        ATSNE_TRY((f_launch<1, F_SAMPLE>(p, pairs * p.splits, stream)));
         t.minima = w.minima;
         t.m = p.m;
         t.rank = pl.rank;
@@ -697,12 +727,12 @@ atsne_status knn_filter_launch(const TcPlan &pl, const TcWs &w, const FilterArgs
         ATSNE_TRY(tc_map_bf16(&p.tm_b_lo, w.lo, a.N, pl.Dp, F_BH));
         p.tm_a_ext = p.tm_b_ext = p.tm_a_hi;
         p.lo_max = a.lo_max;
-        return f_launch<3, false>(p, pairs * p.splits, stream);
+        return a.radius ? f_launch<3, F_RADIUS>(p, pairs * p.splits, stream) : f_launch<3, F_MAIN>(p, pairs * p.splits, stream);
     }
     // the norm pieces' rows are padded to a whole tile with +inf (norm_pieces)
     ATSNE_TRY(tc_map_ext(&p.tm_a_ext, w.aext, F_BM, F_BM));
     ATSNE_TRY(tc_map_ext(&p.tm_b_ext, w.bext, (a.N + F_BN - 1) / F_BN * F_BN, F_BH));
-    return f_launch<1, false>(p, pairs * p.splits, stream);
+    return a.radius ? f_launch<1, F_RADIUS>(p, pairs * p.splits, stream) : f_launch<1, F_MAIN>(p, pairs * p.splits, stream);
 }
 
 atsne_status knn_retry_tau_launch(const TcPlan &pl, const TcWs &w, cudaStream_t stream) {

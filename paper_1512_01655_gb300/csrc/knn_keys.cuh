@@ -20,7 +20,7 @@ struct Cand {
 // Which launch wrote a buffer's metadata (count, threshold bits, overflow, tag).
 enum : int { META_FIRST = 1, META_RETRY = 2 };
 
-constexpr int F_PARTS = 4;  // candidate buffers per (row, split) of the fixed-threshold kernel
+constexpr int F_PARTS = 4;  // parts of a tile's columns in the fixed-threshold kernel, a buffer each (with radii one)
 
 // Bound on |estimated - true| key (= squared distance - ||x_i||^2) for query
 // row statistics st = (||x||, residual norm of its BF16 copy, norm of its low

@@ -2177,7 +2177,7 @@ static bool plan_filter(TcPlan &pl, int64_t N, int D, int64_t Q, bool list, int 
     return plan_region(pl, N, D, Q, list, 0);
 }
 
-TcPlan tc_plan(int64_t N, int D, int64_t Q, bool list, int k, int precision, int rerank_k, int splits) {
+static TcPlan plan_mode(int D, int k, int precision, int rerank_k) {
     TcPlan pl;
     pl.passes = precision == ATSNE_FP32 ? 3 : precision == ATSNE_FP8_RERANK ? 8 : 1;
     pl.certify = precision != ATSNE_FP8_RERANK && precision != ATSNE_BF16_RERANK_APPROX;
@@ -2187,6 +2187,11 @@ TcPlan tc_plan(int64_t N, int D, int64_t Q, bool list, int k, int precision, int
     if (!pl.certify && ks > RCAP_FP8 / 2) ks = RCAP_FP8 / 2;
     if (ks < k) ks = k;
     pl.ksel = ks;
+    return pl;
+}
+
+TcPlan tc_plan(int64_t N, int D, int64_t Q, bool list, int k, int precision, int rerank_k, int splits) {
+    TcPlan pl = plan_mode(D, k, precision, rerank_k);
     if (splits == 0) splits = tuned_splits(N, D, Q, k, precision, rerank_k);
     plan_adaptive(pl, N, Q, pl.passes == 8 ? splits : 0);
     if (pl.passes != 8 && !plan_filter(pl, N, D, Q, list, splits)) plan_adaptive(pl, N, Q, splits);
@@ -2195,15 +2200,30 @@ TcPlan tc_plan(int64_t N, int D, int64_t Q, bool list, int k, int precision, int
 
 // Queries from another array with radii: the radii are the thresholds, nothing
 // is sampled, and what does not fit the buffers goes to the brute-force kernel.
+// The buffers, one per row and split, take the workspace of RADIUS_CAP keys for
+// each of the adaptive launch's units; in more splits only while a buffer keeps
+// room for nearly half of RADIUS_CAP (the most keys that are merged). With that
+// many for each of a split's four parts 100,000 queries against 7,013 points (k =
+// 90) took 0.86 GB instead of 0.24.
 TcPlan tc_plan_radius(int64_t N, int D, int64_t Q, int k, int precision, int rerank_k) {
-    TcPlan pl = tc_plan(N, D, Q, true, k, precision, rerank_k);
-    const int64_t col_tiles = (N + TC_BN - 1) / TC_BN;
-    const int s = filter_splits((Q + 2 * TC_BM - 1) / (2 * TC_BM), col_tiles, 64);
+    TcPlan pl = plan_mode(D, k, precision, rerank_k);
+    plan_adaptive(pl, N, Q, tuned_splits(N, D, Q, k, precision, rerank_k));
+    pl.cand_bytes = (size_t)Q * pl.splits * pl.halves * RADIUS_CAP * sizeof(Cand);
+    const size_t most = plan_bytes(N, D, Q, true, pl);
+    const int64_t pairs = (Q + 2 * TC_BM - 1) / (2 * TC_BM), col_tiles = (N + TC_BN - 1) / TC_BN;
     pl.filter = true;
-    pl.S = 0;
-    pl.fsplits = s;
-    pl.fcap = RADIUS_CAP;
-    pl.cand_bytes = (size_t)Q * s * F_PARTS * RADIUS_CAP * sizeof(Cand);
+    pl.fparts = 1;
+    for (int s = filter_splits(pairs, col_tiles, 64); s > 0; s = s > 1 ? filter_splits(pairs, col_tiles, s - 1) : 0) {
+        const size_t per_key = (size_t)Q * s * sizeof(Cand);
+        pl.fsplits = s;
+        pl.cand_bytes = 0;
+        const size_t b = plan_bytes(N, D, Q, true, pl);
+        pl.fcap = (int)hmin((int64_t)RADIUS_CAP, (int64_t)((most > b ? most - b : 0) / 256 * 256 / per_key));
+        // (with a handful of queries the carved pads outweigh the keys)
+        if (s == 1 && pl.fcap < RADIUS_CAP / 4) pl.fcap = RADIUS_CAP / 4;
+        pl.cand_bytes = per_key * pl.fcap;
+        if (pl.fcap >= RADIUS_CAP / 2 - 8) break;
+    }
     return pl;
 }
 
@@ -2225,7 +2245,7 @@ size_t tc_workspace(Carver &c, int64_t N, int D, int64_t Q, bool list, const TcP
     // fixed-threshold one before it use the same buffers in turn (plan_region)
     const bool adaptive = !pl.filter || pl.S > 0;
     const size_t abufs = adaptive ? (size_t)pl.rrows * pl.splits * pl.halves : 0;
-    const size_t fbufs = pl.filter ? (size_t)Q * pl.fsplits * F_PARTS : 0;
+    const size_t fbufs = pl.filter ? (size_t)Q * pl.fsplits * pl.fparts : 0;
     w.cand = c.take<char>(pl.cand_bytes);
     w.metas = abufs > fbufs ? abufs : fbufs;
     w.meta = c.take<char>(w.metas * sizeof(int4));
@@ -2448,7 +2468,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
         f.sq_coef = sq_coef;
         f.qcount = qcount;
         ATSNE_TRY(knn_filter_launch(pl, w, f, stream));
-        m.splits = pl.fsplits * F_PARTS;
+        m.splits = pl.fsplits * pl.fparts;
         m.cap = pl.fcap;
         m.tag = META_FIRST;
         m.flag_out = !retry;

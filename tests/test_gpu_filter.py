@@ -127,3 +127,29 @@ def test_more_rows_given_up_than_the_adaptive_launch_holds(at, N, D, k):
     X[:, ::D // 7] = (rows(N, X[:, ::D // 7].shape[1], D) > 0).float()
     same(at, X, k)
     same(at, X, k, queries=torch.arange(0, N, 3, dtype=torch.int32, device="cuda"))
+
+
+@pytest.mark.parametrize("precision", ["fp32", "bf16"])
+def test_radii_of_none_to_more_points_than_the_buffers_hold(at, precision):
+    # many queries (one buffer of about 250 keys per row), 0 to 329 points inside
+    # the radius, in runs of the corpus
+    Nq, Nc, D, k = 40000, 1500, 6, 120
+    Xq, Xc = rows(Nq, D, 1), rows(Nc, D, 2)
+    Xc = Xc[Xc[:, 0].argsort()].contiguous()
+    d = (Xq.double().square().sum(1)[:, None] - 2 * Xq.double() @ Xc.double().T + Xc.double().square().sum(1)).sort(1).values
+    m = torch.arange(Nq, device="cuda") % 330
+    r = (0.5 * (d.gather(1, m[:, None]) + d.gather(1, m[:, None] + 1))).squeeze(1).float().contiguous()
+    r[5::997] = float("inf")
+    i, dd = at.atsne_knn_cross(Xq, Xc, k, radius_d2=r, precision=precision)
+    ri, rd = at.atsne_knn_cross(Xq, Xc, k, radius_d2=r, precision="fp32_cuda")
+    at.atsne_check()
+    fin = ~rd.isinf()
+    bound = 12 * 2.0 ** -24 * rd.clamp(max=1e30)  # (4 ceil(D / 32) + 8) 2^-24: see above
+    assert torch.equal(dd.isinf(), rd.isinf()) and ((dd[fin] - rd[fin]).abs() <= bound[fin]).all()
+    # the points themselves, but where two distances (or the k-th and the next
+    # one) are within the bound of each other, whose order only FP64 settles
+    near = torch.zeros_like(fin)
+    near[:, 1:] |= rd[:, 1:] - rd[:, :-1] <= 2 * bound[:, 1:]
+    near[:, :-1] |= rd[:, 1:] - rd[:, :-1] <= 2 * bound[:, :-1]
+    near[:, -1] |= (d[:, k] - d[:, k - 1]).float() <= 2 * bound[:, -1]
+    assert torch.equal(i[fin & ~near], ri[fin & ~near]) and near[fin].float().mean() < 0.01

@@ -30,7 +30,12 @@ KNN = [  # the call, N (of the corpus), D, S (listed or other rows; 0: all), k, 
     ("refine_batch", 900, 16, 400, 30, None, 3385344),
     ("refine_batch", 50000, 64, 100, 30, None, 44032),
     ("knn_cross", 100000, 50, 2500, 90, "fp32", 2541501440),
-    ("knn_cross", 1500, 50, 2500, 20, "fp32", 33675520)]
+    ("knn_cross", 1500, 50, 2500, 20, "fp32", 33675520),
+    ("knn_cross_radius", 7013, 50, 100000, 90, "fp32", 236336896),
+    ("knn_cross_radius", 7013, 50, 100000, 90, "bf16", 429267712),
+    ("knn_cross_radius", 100000, 50, 100000, 90, "fp32", 262001152),
+    ("knn_cross_radius", 20000, 50, 20000, 90, "fp32", 592880896),
+    ("knn_cross_radius", 500, 16, 3000, 30, "fp32", 7171072)]
 
 
 @pytest.fixture(scope="module")
