@@ -21,6 +21,7 @@ struct Cand {
 enum : int { META_FIRST = 1, META_RETRY = 2 };
 
 constexpr int F_PARTS = 4;  // parts of a tile's columns in the fixed-threshold kernel, a buffer each (with radii one)
+constexpr int FILTER_MAX_SPLITS = 64;  // its column splits at most
 
 // Bound on |estimated - true| key (= squared distance - ||x_i||^2) for query
 // row statistics st = (||x||, residual norm of its BF16 copy, norm of its low

@@ -82,7 +82,9 @@ constexpr int HSHIFT = 18;       // float bits >> HSHIFT: exponent and 5 mantiss
 constexpr int GH_BUCKETS = 48;   // a row's global histogram (column splits): 6 octaves, 8 per octave
 constexpr int GH_SHIFT = 20;
 constexpr int64_t FILTER_MIN_ROWS = 1024;       // a smaller corpus is not sampled
-constexpr int64_t RETRY_MAX_SPLITS = 128;       // a row's buffers then fit the merge's register path
+constexpr int64_t RETRY_MAX_SPLITS = 128;       // with two halves a row's buffers then fit the merge's register path
+constexpr int MERGE_MAX_BUFS = 256;             // buffers per row there (their starts take the select's counters)
+static_assert(2 * RETRY_MAX_SPLITS <= MERGE_MAX_BUFS && FILTER_MAX_SPLITS * F_PARTS <= MERGE_MAX_BUFS, "a row's buffers");
 constexpr int64_t RETRY_SPLIT_ROWS = 32768;  // rows given up by the fixed threshold that may be split
 
 // PASSES: 1 = one BF16 pass, 3 = BF16 hi/lo in three passes, 8 = one FP8
@@ -169,6 +171,7 @@ struct TcParams {
     const int32_t *rlist, *rcount;
     const float *tau0;     // [Q] key thresholds those rows start from
     int64_t rmax, bufs;    // of which at most rmax are taken, in room for that many (row, split) buffers
+    int sms;               // of the device
     int64_t Q, N;
     int KB;                // Dp / 64
     int splits, cols_per_split, row_tiles;
@@ -187,7 +190,7 @@ struct UnitPlan {
     int64_t Q;
     int row_tiles, splits, cols_per_split;
 };
-__device__ __forceinline__ UnitPlan retry_plan(int64_t count, int64_t N, int64_t bufs) {
+__device__ __forceinline__ UnitPlan retry_plan(int64_t count, int64_t N, int64_t bufs, int sms) {
     UnitPlan u;
     u.Q = count;
     u.row_tiles = (int)((count + TC_BM - 1) / TC_BM);
@@ -195,7 +198,7 @@ __device__ __forceinline__ UnitPlan retry_plan(int64_t count, int64_t N, int64_t
     int64_t s = 1;
     if (count > 0 && count <= RETRY_SPLIT_ROWS)
         s = max((int64_t)1, min(min((tiles + 3) / 4, bufs / count),
-                                min((int64_t)((304 + u.row_tiles - 1) / u.row_tiles), RETRY_MAX_SPLITS)));
+                                min((int64_t)((2 * sms + u.row_tiles - 1) / u.row_tiles), RETRY_MAX_SPLITS)));
     u.cols_per_split = (int)((tiles + s - 1) / s * TC_BN);
     u.splits = (int)((N + u.cols_per_split - 1) / u.cols_per_split);
     return u;
@@ -511,7 +514,7 @@ __global__ void __launch_bounds__(TcCfg<PASSES>::THREADS, 1) knn_tc_kernel(const
     fence_after_sync();
     const uint32_t tbase = s.tmem_base;
     UnitPlan up{p.Q, p.row_tiles, p.splits, p.cols_per_split};
-    if (p.rcount) up = retry_plan(min((int64_t)*p.rcount, p.rmax), p.N, p.bufs);
+    if (p.rcount) up = retry_plan(min((int64_t)*p.rcount, p.rmax), p.N, p.bufs, p.sms);
     const int n_units = up.row_tiles * up.splits;
 
     if (warp == 0) {
@@ -1108,6 +1111,7 @@ struct MergeParams {
     // the rows given up by the fixed-threshold kernel (as in TcParams), or nullptr
     const int32_t *rlist, *rcount;
     int64_t rmax, bufs;
+    int sms;
     const int64_t *qcount;  // if given, the rows in use (device; at most Q)
     int tag;                // of the launch that wrote the buffers
     bool flag_out;          // flag output rows (for the brute-force kernel), else query rows
@@ -1267,7 +1271,7 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : SELECT ? 6 : 5) k
     int64_t Q = p.big_rows ? *p.big_count : p.qcount ? min(*p.qcount, p.Q) : p.Q;
     int S = p.splits;
     if (p.rcount) {
-        const UnitPlan up = retry_plan(min((int64_t)*p.rcount, p.rmax), p.N, p.bufs);
+        const UnitPlan up = retry_plan(min((int64_t)*p.rcount, p.rmax), p.N, p.bufs, p.sms);
         Q = up.Q;
         S = up.splits * p.splits;  // splits of a row by buffers of a split
     }
@@ -1320,7 +1324,7 @@ __global__ void __launch_bounds__(MERGE_WARPS * 32, CERT ? 4 : SELECT ? 6 : 5) k
     }
     bool good = !ovf && total >= sel && qid >= 0 && (cross || qid < p.N);
     int nr = 0;
-    const bool regs = total <= merge_reg_keys(CERT) && S <= 256;
+    const bool regs = total <= merge_reg_keys(CERT) && S <= MERGE_MAX_BUFS;
     // the staged indices: beside the staged keys, or, with the keys in
     // registers, in their place (without a certificate behind the re-rank set)
     int *sj = regs ? reinterpret_cast<int *>(sk0) + (CERT ? 0 : RC) : sjg;
@@ -2159,7 +2163,8 @@ static bool plan_filter(TcPlan &pl, int64_t N, int D, int64_t Q, bool list, int 
     while (S < 65536 && (double)S * S < 0.5 * 1024.0 * (double)N) S <<= 1;
     while (S > N / 2) S >>= 1;
     if (!plan_sample(pl, N, S)) return false;
-    pl.fsplits = splits > 0 ? (int)hmin(hmin((int64_t)splits, (int64_t)64), col_tiles) : filter_splits(pairs, col_tiles, 64);
+    pl.fsplits = splits > 0 ? (int)hmin(hmin((int64_t)splits, (int64_t)FILTER_MAX_SPLITS), col_tiles)
+                            : filter_splits(pairs, col_tiles, FILTER_MAX_SPLITS);
     // within the adaptive launch's workspace if that costs no speed: as many
     // splits, or fewer with no longer a critical path. What does not fit are a
     // few queries (their sample: 1 query of 70,000 x 784 takes 13 MB more, 0.41
@@ -2213,7 +2218,7 @@ TcPlan tc_plan_radius(int64_t N, int D, int64_t Q, int k, int precision, int rer
     const int64_t pairs = (Q + 2 * TC_BM - 1) / (2 * TC_BM), col_tiles = (N + TC_BN - 1) / TC_BN;
     pl.filter = true;
     pl.fparts = 1;
-    for (int s = filter_splits(pairs, col_tiles, 64); s > 0; s = s > 1 ? filter_splits(pairs, col_tiles, s - 1) : 0) {
+    for (int s = filter_splits(pairs, col_tiles, FILTER_MAX_SPLITS); s > 0; s = s > 1 ? filter_splits(pairs, col_tiles, s - 1) : 0) {
         const size_t per_key = (size_t)Q * s * sizeof(Cand);
         pl.fsplits = s;
         pl.cand_bytes = 0;
@@ -2449,6 +2454,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
     m.qcount = qcount;
     m.rmax = pl.rrows;
     m.bufs = pl.rrows * pl.splits;
+    m.sms = num_sms();
     // the fixed-threshold launch; the rows it gives up follow in the adaptive one
     const bool retry = pl.filter && !radius;
     if (pl.filter) {
@@ -2529,6 +2535,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
     p.tau0 = retry ? w.tau : nullptr;
     p.rmax = m.rmax;
     p.bufs = m.bufs;
+    p.sms = m.sms;
     p.clock = w.clock;
     p.qst = reinterpret_cast<const float4 *>(w.qstats);
     p.st = reinterpret_cast<const float4 *>(w.stats);
