@@ -36,8 +36,7 @@ struct TcPlan {
     int fsplits = 1, fparts = 4, fcap = 0;  // buffers per row: fsplits x fparts, of fcap keys
     int fkeys = 0;                          // keys a row is expected to buffer
 };
-// Row and column order of a large self kNN (points grouped by nearest
-// centroid; each row tile streams its own groups' column tiles first).
+// Row and column order of a large self kNN (points grouped by nearest centroid).
 constexpr int64_t ORD_MIN_ROWS = 65536;
 constexpr int ORD_MAX_DIM = 256;
 struct OrderWs {
@@ -46,7 +45,7 @@ struct OrderWs {
     int32_t *label = nullptr, *lab_sorted = nullptr;
     int32_t *perm = nullptr;  // position in the order -> row
     int32_t *bcnt = nullptr, *coff = nullptr;
-    int32_t *pro = nullptr;   // per row tile: first column tile of its groups, their count
+    int32_t *pro = nullptr;   // adaptive thresholds: per row tile, first column tile of its groups, their count
 };
 struct TcWs {
     uint16_t *hi = nullptr, *lo = nullptr, *qhi = nullptr, *qlo = nullptr;
@@ -65,8 +64,9 @@ struct TcWs {
     bool ordered = false;                       // rows and columns in the order of OrderWs
     unsigned long long *clock = nullptr;        // one split: tiles issued by all CTAs
     OrderWs ord;
-    // fixed thresholds: the rows' thresholds, the sampled rows' copies and norm
-    // pieces, the block values, and the rows given up with their copies
+    // fixed thresholds: the rows' thresholds; in the candidate region the sampled
+    // rows' copies and norm pieces and the block values; the rows given up with
+    // their copies (a list's in qhi, qlo)
     float *tau = nullptr, *minima = nullptr;
     uint16_t *shi = nullptr, *sext = nullptr, *rhi = nullptr, *rlo = nullptr;
     int32_t *retry_rows = nullptr;

@@ -487,8 +487,10 @@ knn_filter_kernel(const __grid_constant__ FParams p) {
 
 // Sampled corpus row i: one position of range (i * F_MIX) mod S of S equal
 // ranges of [0, N) (S a power of two: a permutation, so that neighbouring
-// sampled columns come from distant positions), jittered by a hash so that no
-// periodic layout of the corpus is met in step.
+// sampled columns come from distant positions), jittered by a hash (the
+// finaliser of MurmurHash3's 32-bit form, A. Appleby, public domain) so that no
+// periodic layout of the corpus is met in step. F_MIX is Knuth's golden ratio
+// multiplier.
 constexpr unsigned F_MIX = 2654435761u;
 __device__ __forceinline__ int64_t sample_position(unsigned i, unsigned S, int64_t N) {
     const unsigned r = (i * F_MIX) & (S - 1);

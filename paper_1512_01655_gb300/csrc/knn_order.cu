@@ -1,13 +1,22 @@
 // Order of rows and columns for the tensor-core exact kNN of a large point set
-// against itself (Eq. 8). The streaming filter of the tensor kernel keeps every
-// column below the current bound of a row; the bound falls only as near columns
-// arrive, so the survivors it must buffer are about ksel (1 + ln(n / ksel)) when
-// the columns come in random order. Grouping the points by their nearest of
-// ORD_C centroids puts a row's neighbours mostly in its own group: each row tile
-// first streams the column tiles of its own groups, which sets its bound near
-// the final one, then all the others. The result does not depend on the order
-// (the filter keeps a valid bound in any order and the merge returns the exact
-// lists); only the work of the filter does.
+// against itself (Eq. 8): the points grouped by their nearest of ORD_C centroids,
+// so that a row's neighbours lie mostly in its own group. The result does not
+// depend on the order (the merge returns the exact lists); only the work does.
+//
+// With fixed thresholds (knn_filter.cu) a row tile's survivors then come bunched
+// and its re-ranked rows lie close together: log-normal data and the approximate
+// mode gain, the others pay for the grouping and for mapping positions back (and
+// rows that BF16 holds exactly are gathered in FP32). kNN with and without the
+// order, k = 90, ms: 400,000 x 50 log-normal 41.3 and 44.7, 200,000 x 128 Gamma
+// BF16 approximate 12.9 and 13.3, 1,000,000 x 128 217.5 and 217.7, in FP32 427 and
+// 420, 200,000 x 128 FP32 17.4 and 16.7, 70,000 x 64 2.59 and 2.37, 400,000 x 128
+// bytes 44.3 and 42.9.
+//
+// With thresholds that adapt (the FP8 mode) a bound falls only as near columns
+// arrive, and the survivors to buffer are about ksel (1 + ln(n / ksel)) when the
+// columns come in random order: each row tile there first streams the column
+// tiles of its own groups, which sets its bound near the final one, then all the
+// others (ord_prologue_kernel).
 //
 // Centroids: ORD_ITERS Lloyd iterations (nearest centroid, then the mean of its
 // points) over ORD_SAMPLE evenly spaced rows, started from evenly spaced rows.
@@ -170,7 +179,7 @@ __global__ void ord_scatter_kernel(const int32_t *__restrict__ label, int64_t N,
         __syncwarp();
         if (live) {
             perm[base + rank] = (int32_t)r;
-            lab_sorted[base + rank] = l;
+            if (lab_sorted) lab_sorted[base + rank] = l;
             if (rank == 0) next[l] = base + __popc(peers);
         }
         __syncwarp();
@@ -196,8 +205,8 @@ __global__ void ord_prologue_kernel(const int32_t *__restrict__ lab_sorted, cons
 
 }  // namespace
 
-// Worth it where the filter, not the contraction, bounds the kernel: short rows
-// (a tile's MMAs take D / 64 k-blocks against a fixed filter per tile).
+// Short rows: the filter's and the merge's work, which the order changes, then
+// weighs most against the contraction's.
 bool knn_ordered(int64_t N, int D, bool list, const TcPlan &pl) {
     return !list && pl.splits == 1 && N >= ORD_MIN_ROWS && D <= ORD_MAX_DIM;
 }
@@ -210,11 +219,11 @@ size_t order_workspace(Carver &c, int64_t N, int D, const TcPlan &pl, OrderWs *w
     w.sum = c.take<float>((size_t)ORD_C * D);
     w.cnt = c.take<int>(ORD_C);
     w.label = c.take<int32_t>((size_t)N);
-    w.lab_sorted = c.take<int32_t>((size_t)N);
+    w.lab_sorted = pl.filter ? nullptr : c.take<int32_t>((size_t)N);
     w.perm = c.take<int32_t>((size_t)N);
     w.bcnt = c.take<int32_t>((size_t)nblk * ORD_C);
     w.coff = c.take<int32_t>(ORD_C + 1);
-    w.pro = c.take<int32_t>((size_t)2 * pl.row_tiles);
+    w.pro = pl.filter ? nullptr : c.take<int32_t>((size_t)2 * pl.row_tiles);
     if (ws) *ws = w;
     return c.bytes();
 }
@@ -246,6 +255,7 @@ atsne_status knn_order_launch(const float *X, int64_t N, int D, const TcPlan &pl
     ATSNE_TRY(launch_kernel("knn_order", ord_scan_kernel, 1, ORD_C, 0, stream, w.bcnt, nblk, N, w.coff));
     ATSNE_TRY(launch_kernel("knn_order", ord_scatter_kernel, nblk, 32, 0, stream, (const int32_t *)w.label, N,
                             (const int32_t *)w.bcnt, w.perm, w.lab_sorted));
+    if (!w.pro) return ATSNE_OK;
     const int col_tiles = (int)((N + bn - 1) / bn);
     return launch_kernel("knn_order", ord_prologue_kernel, ceil_div((int64_t)pl.row_tiles, 128), 128, 0, stream,
                          (const int32_t *)w.lab_sorted, (const int32_t *)w.coff, N, bm, bn, pl.row_tiles,

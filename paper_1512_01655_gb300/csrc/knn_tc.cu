@@ -1235,8 +1235,9 @@ __device__ __forceinline__ void map_positions(const MergeParams &p, int *rjw, in
 // re-ranked in FP32 and the k best of them kept, without a certificate.
 // p.mst keys are staged per row, p.rc candidates re-ranked at most. Without a
 // certificate the staged keys are read once, by the collection of the re-rank
-// set, so the re-rank set takes their place (p.rc <= p.mst) and five blocks
-// fit on an SM instead of four.
+// set, so the re-rank set takes their place (p.rc <= p.mst). Blocks per SM: four
+// certified, six of the select; a row per block without a certificate, for the
+// few rows that take it, keeps its registers (five).
 constexpr int merge_reg_keys(bool cert) { return 32 * (cert ? 24 : 36); }
 size_t merge_smem_bytes(bool cert, int rc, int mst, int rows) {
     return (size_t)rows * (256 * 4 + (size_t)mst * 8 + (cert ? (size_t)rc * 8 : 0) + TIE_MAX * 12);
@@ -2529,7 +2530,7 @@ atsne_status knn_exact_tc(const float *X, int64_t N, int D, const int32_t *qlist
     p.qscale = (qlist || Xq) ? w.qscale : nullptr;
     p.qnrm = Xq ? w.qnrm : nullptr;
     p.hint = hint;
-    p.pro = ordered && !retry ? w.ord.pro : nullptr;
+    p.pro = ordered ? w.ord.pro : nullptr;  // (the rows given up come in no order)
     p.rlist = retry ? w.retry_rows : nullptr;
     p.rcount = retry ? w.flag_count + 1 : nullptr;
     p.tau0 = retry ? w.tau : nullptr;
