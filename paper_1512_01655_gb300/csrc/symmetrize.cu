@@ -295,7 +295,7 @@ sym_hub_kernel(SymRow s, const int32_t *__restrict__ hub_rows, const int32_t *__
         int64_t done = 0;  // entries of the ranges before
         for (int64_t c0 = 0; c0 < s.N; c0 += (int64_t)words * 32) {
             const int64_t c1 = min(s.N, c0 + (int64_t)words * 32);
-            for (int t = tid; t < words; t += HUB_THREADS) bits[t] = 0u;
+            for (int t = tid; t < words; t += HUB_THREADS) bits[t] = below[t] = 0u;
             __syncthreads();
             for (int64_t t = tid; t < m; t += HUB_THREADS) {
                 const int64_t c = s.rev[b0 + t].x;
@@ -313,9 +313,12 @@ sym_hub_kernel(SymRow s, const int32_t *__restrict__ hub_rows, const int32_t *__
                 }
             }
             __syncthreads();
-            if (fc >= 0 && !mutual) {
+            if (fc >= 0) {
+                // (the forward entries' own bits, in `below` until its sums are
+                // made, show a column listed twice, mutual or not)
                 const uint32_t bit = 1u << ((fc - c0) & 31);
-                if (atomicOr(&bits[(fc - c0) >> 5], bit) & bit) raise_status(s.status, DEV_MALFORMED);  // listed twice
+                if (atomicOr(&below[(fc - c0) >> 5], bit) & bit) raise_status(s.status, DEV_MALFORMED);
+                if (!mutual) atomicOr(&bits[(fc - c0) >> 5], bit);
             }
             __syncthreads();
             // a warp's stretch of words: each word's set bits before it in the

@@ -109,3 +109,16 @@ def test_every_key_differs_from_the_mark_for_none(at, N):
     s = torch.zeros(u.numel(), dtype=torch.float64, device="cuda").index_add_(0, inv, P.double().flatten().repeat(2)) / (2 * N)
     assert torch.equal(col.long(), u % N) and torch.equal(rp[1:], (u // N).bincount(minlength=N).cumsum(0))
     assert ((val - s).abs().max() * N).item() <= 1e-5
+
+
+@pytest.mark.parametrize("N,k", [(1100, 12), (1200, 200)])
+def test_a_mutual_column_listed_twice_in_a_hub_row(at, N, k):
+    rng = np.random.default_rng(5)
+    idx = lists(N, k, [N - 1], rng)  # every row lists row 0, which lists each of its neighbours mutually
+    P = torch.full((N, k), 1.0 / k, device="cuda")
+    at.atsne_symmetrize(torch.from_numpy(idx).cuda(), P)
+    at.atsne_check()
+    idx[0, k - 1] = idx[0, 0]
+    at.atsne_symmetrize(torch.from_numpy(idx).cuda(), P)
+    with pytest.raises(at.AtsneError):
+        at.atsne_check()
