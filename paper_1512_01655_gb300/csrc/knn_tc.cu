@@ -2328,9 +2328,15 @@ static atsne_status merge_launch(const TcPlan &pl, MergeParams m, cudaStream_t s
     // one row per block while the rows leave most of the SMs' warps idle, and for
     // those given up by the fixed threshold, which are few
     const bool one = m.rcount || m.Q <= MERGE_ONE_ROWS * num_sms();
+    // (the limits set are those of any ksel: the attribute is the kernel's, and
+    // another thread's call may set it before this one's launch)
+    const int rc_most = pl.certify ? RCAP : RCAP_FP8;
+    const int mst_most = pl.certify ? MSTAGE : (RCAP_FP8 + merge_reg_keys(false)) / 2;
+    auto rerank_bytes = [](int rc) { return (size_t)MERGE_WARPS * ((size_t)rc * 8 + TIE_MAX * 12); };
     auto rerank = [&](void (*k)(MergeParams)) {
-        const size_t rs = (size_t)MERGE_WARPS * ((size_t)m.rc * 8 + TIE_MAX * 12);
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs);
+        const size_t rs = rerank_bytes(m.rc);
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)rerank_bytes(pl.certify ? RERANK_KEYS : RCAP_FP8));
         if (e != cudaSuccess) return cuda_error(e, "knn_tc_merge attribute");
         return launch_kernel("knn_rerank", k, ceil_div(m.Q, MERGE_WARPS), MERGE_WARPS * 32, rs, stream, m);
     };
@@ -2351,7 +2357,8 @@ static atsne_status merge_launch(const TcPlan &pl, MergeParams m, cudaStream_t s
     void (*kern)(MergeParams) = pl.certify ? (few ? knn_merge_kernel<true, 1> : knn_merge_kernel<true, MERGE_WARPS>)
                                            : (few ? knn_merge_kernel<false, 1> : knn_merge_kernel<false, MERGE_WARPS, true>);
     const int grid = m.rcount || light ? (int)hmin(4 * num_sms(), m.Q) : ceil_div(m.Q, one ? 1 : MERGE_WARPS);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ms);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)merge_smem_bytes(pl.certify, rc_most, mst_most, few ? 1 : MERGE_WARPS));
     if (e != cudaSuccess) return cuda_error(e, "knn_tc_merge attribute");
     ATSNE_TRY(launch_kernel(split ? "knn_select" : "knn_tc_merge", kern, grid, MERGE_WARPS * 32, ms, stream, m));
     return split ? rerank(knn_rerank_kernel<false>) : ATSNE_OK;

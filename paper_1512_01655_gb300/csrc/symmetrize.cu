@@ -427,7 +427,9 @@ atsne_status symmetrize_t(const int32_t *idx, const float *P, int64_t N, int k, 
     ATSNE_TRY(scan_rowlen(w.len, N, 0, row_ptr, nnz_dev, w.scan, stream));
     const int words = (int)((hmin(N, HUB_COLS) + 31) / 32);
     const size_t smem = (size_t)words * 8;
-    e = cudaFuncSetAttribute(sym_hub_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (the limit for any N: the attribute is the kernel's, and another thread's
+    // smaller call may set it before this one's launch)
+    e = cudaFuncSetAttribute(sym_hub_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(HUB_COLS / 4));
     if (e != cudaSuccess) return cuda_error(e, "sym_hub attribute");
     ATSNE_TRY(launch_kernel("sym_hub", sym_hub_kernel, (int)hmin(4 * num_sms(), N), HUB_THREADS, smem, stream, s,
                             (const int32_t *)w.hub_rows, (const int32_t *)w.n_list, words, inv2n,
