@@ -2095,7 +2095,8 @@ static bool plan_region(TcPlan &pl, int64_t N, int D, int64_t Q, bool list, size
     const int64_t per = ((N + TC_BN - 1) / TC_BN + pl.fsplits - 1) / pl.fsplits * (TC_BN / F_PARTS);  // columns of a buffer
     const double r = (double)pl.fkeys * pl.S / (double)N;
     // keys per buffer, at least: its share, the threshold's spread (one row in a
-    // thousand is above it), the share's, and the chunk that closes a buffer.
+    // thousand is above it), the share's, and room to spare (a buffer is closed
+    // once fewer than 8 places are left).
     // Neighbours that follow one another fill no more than four of the splits
     const double share = (double)pl.fkeys / (F_PARTS * hmin(pl.fsplits, 4));
     const int64_t least = hmin(per, (int64_t)ceil(share * (1.0 + 3.5 / sqrt(r)) + 3.0 * sqrt(share)) + 32);
