@@ -23,12 +23,13 @@
 // misses it goes to the adaptive kernel of knn_tc.cu.
 //
 // Measured against the adaptive kernel on all rows (one GB300, kernels alone):
-// 1,000,000 x 128 Gamma clusters, one BF16 pass, ksel 360: 270 ms to 178 ms
-// (+ 7 ms for the thresholds), about 1.6 PFLOP/s, near the rate the power limit
-// leaves (the contraction alone 0.65 us per 256 x 256 x 144 pair tile, MMAs
-// 90% of it); 200,000 x 128, three passes, ksel 128: 22.7 to 14.0 ms; 50,021 x
-// 50 log-normal, ksel 188: 4.6 to 0.94 ms; 70,000 x 784 bytes: 6.4 to 4.5 ms;
-// 7,013 queries against 107,013 x 50: 9.1 to 0.3 ms.
+// 1,000,000 x 128 Gamma clusters, one BF16 pass, ksel 360: 270 ms to 176 ms
+// (+ 7 ms for the thresholds), 1.45 PFLOP/s of 2 N^2 D (1.64 with the K step of
+// the norms), at the clock that the power limit leaves; 200,000 x 128, three
+// passes, ksel 128: 22.7 to 14.0 ms; 50,021 x 50 log-normal, ksel 188: 4.6 to 0.96
+// ms; 70,000 x 784 bytes: 6.4 to 4.5 ms; 7,013 queries against 107,013 x 50: 9.1
+// to 0.3 ms. With fewer columns a larger share of them survives, and appending
+// sets the pace: 100,000 x 128, one pass, tensor pipe active 49%, issue 67%.
 //
 // Layout. Two CTAs on neighbouring SMs form a pair (cta_group::2): M = 256
 // query rows, 128 per CTA, against N = 256 corpus rows, of which each CTA
@@ -37,9 +38,10 @@
 // of this contraction asks shared memory for more bytes per cycle than it has.
 // Per CTA: warp 0 issues the TMA loads, warp 1 (of the even CTA) the MMAs, and
 // FC::NEPI warps the epilogue, FC::NEPI / 4 per TMEM lane quadrant, each taking
-// 64 of a tile's 256 columns. The usual 32-column chunk holds no survivor of
-// any of the warp's rows and costs one tcgen05.ld, a tree of three-input maxima
-// (18 instructions) and one vote.
+// 64 of a tile's 256 columns. A 32-column chunk without a survivor of any of the
+// warp's rows (most of them in a large corpus, few at 50,000 rows) costs one
+// tcgen05.ld, a tree of three-input maxima (18 instructions) and one vote; one
+// with survivors a vote per group of eight columns and the groups' appends.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
