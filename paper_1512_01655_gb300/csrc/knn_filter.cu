@@ -422,14 +422,20 @@ knn_filter_kernel(const __grid_constant__ FParams p) {
                             // 32, k = 30, four clusters in blocks of 64 rows: 2.55
                             // ms, 1.63 now)
                             if (!RADIUS && cnt > p.cap - 8) thr = INFINITY;
+                            if (RADIUS) {
+                                // a lane's keys of the group take their places at once
+                                int n = 0;
+#pragma unroll
+                                for (int j = 0; j < 8; ++j) n += v[8 * q + j] > thr;
+                                if (n > 0) {
+                                    cnt = atomicAdd(row_cnt, n);
+                                    if (cnt > p.cap - n) thr = INFINITY;  // full
+                                }
+                            }
 #pragma unroll
                             for (int j = 0; j < 8; ++j) {
                                 const float x = v[8 * q + j];
-                                if (x > thr) {
-                                    const int at = RADIUS ? atomicAdd(row_cnt, 1) : cnt++;
-                                    if (!RADIUS || at < p.cap) buf[at] = Cand{C::FOLD ? -2.f * x : -x, col + 8 * q + j};
-                                    else thr = INFINITY;  // full
-                                }
+                                if (x > thr) buf[cnt++] = Cand{C::FOLD ? -2.f * x : -x, col + 8 * q + j};
                             }
                         }
                     }
